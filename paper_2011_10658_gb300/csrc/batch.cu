@@ -163,8 +163,10 @@ int BatchRunner::build(int node, const std::vector<int>& members, std::unique_pt
     // plans again now that all exist)
     for (int i = 0; i < 3; ++i) {
       KPlan& b = g->st[i];
+      bool gather = true;
       for (int m : members) {
         const KPlan& p = es_[m]->heff_plans(node, -1, false)->st[i];
+        gather = gather && p.gather;
         const int c0 = (int)b.chunks.size();
         for (KOutput o : p.outs) {
           o.chunk_begin += c0;
@@ -174,6 +176,7 @@ int BatchRunner::build(int node, const std::vector<int>& members, std::unique_pt
         append(&b.chunks, p.chunks);
       }
       b.finalize(4096);
+      b.gather = gather;
     }
   }
   for (int m : members) g->gens.push_back(es_[m]->gen_);
@@ -255,7 +258,7 @@ int BatchRunner::product(int node, const std::vector<int>& active) {
   }
   bool tuned = true;
   for (const KPlan& p : g->st)
-    if (!p.outs.empty() && p.shape[g->fp32] < 0 && e0->forced_shape_ < 0) tuned = false;
+    if (!p.outs.empty() && !p.gather && p.shape[g->fp32] < 0 && e0->forced_shape_ < 0) tuned = false;
   if (g->tg && !g->launched) tuned = false;   // first launch eager (one-time kernel set-up on the host)
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   const bool capturable = use_graphs_ && tuned && s != nullptr &&
@@ -265,7 +268,7 @@ int BatchRunner::product(int node, const std::vector<int>& active) {
   for (KPlan& p : g->st)
     if (!p.outs.empty()) {
       const int shape = e0->forced_shape_ >= 0 ? e0->forced_shape_ : p.shape[g->fp32];
-      e0->ensure_scratch(std::max<long long>(p.variant(shape, s).scratch_need, 1));
+      e0->ensure_scratch(std::max<long long>(p.scratch_need(shape, s), 1));
     }
   const long long before = launch_count();
   if (!e0->check(cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed), "graph capture")) return -3;

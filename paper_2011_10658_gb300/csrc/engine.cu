@@ -145,6 +145,7 @@ void KPlan::finalize(long long kp) {
     for (int c = o.chunk_begin; c < o.chunk_end; ++c)
       if (!chunks[c].add) flops += 2.0 * o.M * o.N * chunks[c].K;
   for (KVariant& v : var) v.ready = false;
+  bh.ready = false;
 }
 
 // Tiles of BM x BM (BM = 16, 32 or 64) per output.  Outputs with few tiles
@@ -263,6 +264,71 @@ void KVariant::upload(cudaStream_t s) {
   grow_upload(d_red, cap_red, red, s);
 }
 
+// Row tiles per output sector; every environment block once per chunk.
+BhPlan& KPlan::bh_plan(cudaStream_t s) {
+  BhPlan& b = bh;
+  if (b.ready) return b;
+  b.tiles.clear(); b.outs.clear(); b.chunks.clear(); b.jobs.clear();
+  b.w_elems = 0;
+  b.max_n = b.max_k = 1;
+  auto recip = [](int d) { return (unsigned)(((1ull << 32) + d - 1) / d); };   // ceil(2^32 / d), unused for d = 1
+  for (const KOutput& o : outs) {
+    BhOut bo{};
+    bo.C = o.C;
+    bo.M = o.M;
+    bo.N = o.N;
+    bo.div = recip(o.N);
+    bo.chunk_begin = (int)b.chunks.size();
+    b.max_n = std::max(b.max_n, o.N);
+    for (int ci = o.chunk_begin; ci < o.chunk_end; ++ci) {
+      const KChunk& c = chunks[ci];
+      BhChunk bc{};
+      bc.A = c.A;
+      bc.map = c.amap;
+      bc.val = c.aval;
+      bc.alpha = c.alpha;
+      bc.ld = (int)c.a_m;
+      if (!c.add) {
+        bc.K = c.K;
+        bc.div = recip(c.K);
+        bc.w = b.w_elems;
+        b.max_k = std::max(b.max_k, c.K);
+        BhJob j{};
+        j.B = c.B;
+        j.b_k = c.b_k;
+        j.b_n = c.b_n;
+        j.off = b.w_elems;
+        j.alpha = c.alpha;
+        j.K = c.K;
+        j.N = o.N;
+        b.jobs.push_back(j);
+        b.w_elems += (long long)c.K * o.N;
+      }
+      b.chunks.push_back(bc);
+    }
+    bo.chunk_end = (int)b.chunks.size();
+    b.outs.push_back(bo);
+  }
+  const int rows = bh_rows(b.max_n, b.max_k);
+  for (size_t oi = 0; oi < b.outs.size(); ++oi)
+    for (int r0 = 0; r0 < b.outs[oi].M; r0 += rows) b.tiles.push_back(BhTile{(int)oi, r0});
+  grow_upload(b.d_tiles, b.cap[0], b.tiles, s);
+  grow_upload(b.d_outs, b.cap[1], b.outs, s);
+  grow_upload(b.d_chunks, b.cap[2], b.chunks, s);
+  grow_upload(b.d_jobs, b.cap[3], b.jobs, s);
+  b.ready = true;
+  return b;
+}
+
+void BhPlan::release() {
+  void* ptrs[4] = {d_tiles, d_outs, d_chunks, d_jobs};
+  for (void* p : ptrs)
+    if (p) cudaFree(p);
+  d_tiles = nullptr; d_outs = nullptr; d_chunks = nullptr; d_jobs = nullptr;
+  for (size_t& c : cap) c = 0;
+  ready = false;
+}
+
 void KVariant::release() {
   if (d_chunks) cudaFree(d_chunks);
   if (d_outs) cudaFree(d_outs);
@@ -278,6 +344,7 @@ void KVariant::release() {
 
 void KPlan::release() {
   for (KVariant& v : var) v.release();
+  bh.release();
   for (auto& m : tev)
     for (auto& sh : m)
       for (auto& rep : sh)
@@ -443,7 +510,7 @@ bool Engine::in_own_range(const void* p, long long lo_bytes, long long hi_bytes)
 // Host-side check that every chunk and output of a plan stays inside a
 // known device allocation (enabled by QED_VALIDATE=1).  Row-mapped operands
 // are checked over their whole source sector by the row-map builder.
-bool Engine::validate_plan(const KPlan& pl, const KVariant& v, const char* what) {
+bool Engine::validate_plan(const KPlan& pl, const KVariant* v, const char* what) {
   for (const KOutput& o : pl.outs) {
     const long long hi = (long long)(o.M - 1) * o.c_m + (long long)(o.N - 1) * o.c_n;
     if (o.M <= 0 || o.N <= 0 || !in_range(o.C, 0, hi * 8 + 8)) {
@@ -478,13 +545,14 @@ bool Engine::validate_plan(const KPlan& pl, const KVariant& v, const char* what)
       }
     }
   }
-  for (const KTile& t : v.tiles) {
-    if (t.out < 0 || t.out >= (int)v.outs.size() || t.chunk_begin < 0 || t.chunk_end > (int)v.chunks.size()) {
+  if (!v) return true;
+  for (const KTile& t : v->tiles) {
+    if (t.out < 0 || t.out >= (int)v->outs.size() || t.chunk_begin < 0 || t.chunk_end > (int)v->chunks.size()) {
       err_ = std::string(what) + ": bad tile";
       return false;
     }
-    if (t.part >= 0 && !in_range(scratch_, v.outs[t.out].part_off * 8,
-                                 (v.outs[t.out].part_off + (long long)(t.part + 1) * v.outs[t.out].M * v.outs[t.out].N) * 8)) {
+    if (t.part >= 0 && !in_range(scratch_, v->outs[t.out].part_off * 8,
+                                 (v->outs[t.out].part_off + (long long)(t.part + 1) * v->outs[t.out].M * v->outs[t.out].N) * 8)) {
       err_ = std::string(what) + ": scratch out of range";
       return false;
     }
@@ -531,6 +599,14 @@ int KPlan::candidates(int* out) const {
 int Engine::launch_kplan(KPlan& pl, int fp32, bool tune) {
   if (pl.outs.empty()) return 0;
   const int mode = fp32;   // 0 FP64, 1 FP32, 2 float-float
+  if (pl.gather && mode != 1) {
+    BhPlan& b = pl.bh_plan(stream_);
+    ensure_scratch(std::max<long long>(b.w_elems, 1));
+    if (validate_ && !validate_plan(pl, nullptr, "plan")) return -1;
+    launch_bh(b.d_tiles, (int)b.tiles.size(), b.d_outs, b.d_chunks, b.d_jobs, (int)b.jobs.size(), b.max_n, b.max_k,
+              scratch_, stream_, mode == 2);
+    return check(cudaGetLastError(), "bottom-node product launch") ? 0 : -3;
+  }
   int shape = forced_shape_ >= 0 ? forced_shape_ : pl.shape[mode];
   if (shape < 0 && !tune) {   // one-off plans: the least padded shape
     int cand[KS_COUNT];
@@ -575,7 +651,7 @@ int Engine::launch_kplan(KPlan& pl, int fp32, bool tune) {
   }
   KVariant& v = pl.variant(shape, stream_);
   ensure_scratch(std::max<long long>(v.scratch_need, 1));
-  if (validate_ && !validate_plan(pl, v, "plan")) return -1;
+  if (validate_ && !validate_plan(pl, &v, "plan")) return -1;
   if (timed) {
     for (int i = 0; i < 2; ++i)
       if (!timed[i]) cudaEventCreate(&timed[i]);
@@ -1983,6 +2059,9 @@ Engine::HeffPlans* Engine::heff_plans(int node, int cls, bool adjoint) {
     for (int i = 0; i < 2; ++i) st[i].finalize(kKPart);
   }
   s3.finalize(kKPart);
+  int widest = 1;
+  for (int d : L.leg[2].dim) widest = std::max(widest, d);
+  s3.gather = bottom && bh_fits(widest, widest);
   for (int i = 0; i < 3; ++i) hp->flops += st[i].flops;
   if (!check(cudaGetLastError(), "plan")) return nullptr;
   HeffPlans* raw = hp.get();

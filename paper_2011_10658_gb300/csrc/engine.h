@@ -76,6 +76,25 @@ struct KVariant {
   ~KVariant() { release(); }
 };
 
+// A bottom-node product's work list in the form of the packed row-gather
+// kernel (kernels_bh.cu), cut from a KPlan's outputs and chunks.
+struct BhPlan {
+  std::vector<BhTile> tiles;
+  std::vector<BhOut> outs;
+  std::vector<BhChunk> chunks;
+  std::vector<BhJob> jobs;
+  BhTile* d_tiles = nullptr;
+  BhOut* d_outs = nullptr;
+  BhChunk* d_chunks = nullptr;
+  BhJob* d_jobs = nullptr;
+  size_t cap[4] = {0, 0, 0, 0};
+  long long w_elems = 0;   // staged environment entries (8 bytes each)
+  int max_n = 1, max_k = 1;
+  bool ready = false;
+  void release();
+  ~BhPlan() { release(); }
+};
+
 // Grouped-GEMM work list: outputs, each with its chunks (built through
 // add_output / add_chunk, flattened by finalize), cut into tiles per tile
 // shape on demand, with the chosen shape per arithmetic (FP64, FP32).
@@ -87,6 +106,14 @@ struct KPlan {
   int current = -1;
   long long k_part = 4096;
   double flops = 0.0;   // 2 M N K over the GEMM chunks (set by finalize)
+  // row-gather product of a bottom node: whole output sectors (row-major,
+  // not accumulated), A rows of unit stride; runs on kernels_bh.cu
+  bool gather = false;
+  BhPlan bh;
+  BhPlan& bh_plan(cudaStream_t s);
+  long long scratch_need(int shape, cudaStream_t s) {
+    return gather ? bh_plan(s).w_elems : variant(shape, s).scratch_need;
+  }
   KVariant var[KS_COUNT];
   int shape[3] = {-1, -1, -1};    // tuned tile shape per arithmetic (FP64, FP32, float-float), -1 while tuning
   int trials[3] = {0, 0, 0};
@@ -94,6 +121,7 @@ struct KPlan {
   void clear() {
     chunks.clear(); outs.clear(); out_chunks.clear(); out_index.clear(); current = -1; flops = 0.0;
     for (KVariant& v : var) v.ready = false;
+    gather = bh.ready = false;
   }
   int add_output(double* C, long long c_m, long long c_n, int M, int N, int accumulate);
   void add_chunk(const KChunk& c);
@@ -449,7 +477,7 @@ class Engine {
   // device allocations (base, bytes) for the optional plan validator
   std::map<uintptr_t, size_t> ranges_;
   bool validate_ = false;
-  bool validate_plan(const KPlan& pl, const KVariant& v, const char* what);
+  bool validate_plan(const KPlan& pl, const KVariant* v, const char* what);
   void track(void* p, size_t bytes) { if (p) ranges_[(uintptr_t)p] = bytes; }
   void untrack(void* p) { ranges_.erase((uintptr_t)p); }
   bool in_range(const void* p, long long lo_off, long long hi_off) const;   // own or a peer's

@@ -72,6 +72,48 @@ void launch_kc_gemm(const KTile* tiles, int n_tiles, const KOutput* outs, const 
 void launch_kc_reduce(const KOutput* outs, int n_outs, const int* red_list, int n_red, double* scratch,
                       cudaStream_t s);
 
+// ---- bottom-node products as packed row gathers (kernels_bh.cu) ----
+// Output sector of y (M x N, row-major): the sum over its chunks of
+//   K > 0:  alpha s(r) val(r) A[map(r) * ld + k] B[k, n]  (alpha B staged at w)
+//   K = 0:  alpha s(r) val(r) A[map(r) * ld + n]
+// with map sign-encoded as in KChunk (NULL: identity) and val optional.
+// div: ceil(2^32 / K) or, in an output, ceil(2^32 / N).
+struct BhChunk {
+  const double* A;
+  const int* map;
+  const double* val;
+  long long w;
+  double alpha;
+  int ld, K;
+  unsigned div;
+};
+struct BhOut {
+  double* C;
+  int M, N;
+  int chunk_begin, chunk_end;
+  unsigned div;
+};
+struct BhTile {
+  int out;
+  int row0;
+};
+// Staging job: w[off + k * N + n] = alpha B[k * b_k + n * b_n].
+struct BhJob {
+  const double* B;
+  long long b_k, b_n;
+  long long off;
+  double alpha;
+  int K, N;
+};
+// Rows of a tile for outputs up to max_n and terms up to max_k wide, the shared
+// memory of the warp that owns it, and whether that fits the SM.
+int bh_rows(int max_n, int max_k);
+size_t bh_warp_bytes(int max_n, int max_k, int rows);
+bool bh_fits(int max_n, int max_k);
+// w: staging of 8 bytes per entry.  ff_arith: float-float arithmetic.
+void launch_bh(const BhTile* tiles, int n_tiles, const BhOut* outs, const BhChunk* chunks, const BhJob* jobs,
+               int n_jobs, int max_n, int max_k, double* w, cudaStream_t s, int ff_arith);
+
 // ---- vector kernels (FP64) ----
 // partial sums per block then a single-block finish: deterministic.
 void launch_dot(const double* x, const double* y, long long n, double* partial, double* out, cudaStream_t s);
