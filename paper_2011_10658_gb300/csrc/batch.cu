@@ -326,9 +326,8 @@ int BatchRunner::lanczos(int node, const std::vector<double>& tol, int max_krylo
     if (rc) return rc;
     for (int b : active) {
       Engine* e = es_[b];
-      e->lz_iteration(st[b].j, st[b].n);
+      if ((rc = e->lz_iteration(st[b].j, st[b].n))) return rc;
       e->lz_queue_check(st[b].j);
-      e->lz_next_vector(st[b].j, st[b].n);
       st[b].iters += 1;
     }
     for (int b : active)
@@ -371,6 +370,8 @@ int BatchRunner::lanczos(int node, const std::vector<double>& tol, int max_krylo
     Engine* e = es_[b];
     e->use_mixed_ = false;
     e->last_conv_ = -1;
+    const int rc = e->lz_waits();
+    if (rc) return rc;
     (*energy)[b] = e->ring_host_[4 * kMaxKrylov];
     (*resid)[b] = e->ring_host_[4 * kMaxKrylov + 1];
     (*iters)[b] = st[b].iters;

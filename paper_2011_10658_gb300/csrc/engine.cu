@@ -747,8 +747,10 @@ Engine::Engine(const Params& p, int chi, uint64_t seed, int precision, cudaStrea
   grad_b_ = (double*)dalloc(nmax_ * sizeof(double));
   grad_c_ = (double*)dalloc(nmax_ * sizeof(double));
   d_scal_ = (double*)dalloc(8192 * sizeof(double));
-  d_partial_ = (double*)dalloc(1216 * (kMaxKrylov + 2) * sizeof(double));
-  d_err_ = (int*)dalloc(4 * sizeof(int));   // [0] tensor-core wait flag, [1] thick-restart count, [2] non-finite flag
+  d_partial_ = (double*)dalloc(kLzPartial * sizeof(double));
+  // [0] tensor-core wait flag, [1] thick-restart count, [2] non-finite flag,
+  // [3] Lanczos-step wait flag, [4..5] its grid barrier
+  d_err_ = (int*)dalloc(8 * sizeof(int));
   if (!check(cudaStreamCreateWithFlags(&aux_, cudaStreamNonBlocking), "side stream")) throw std::runtime_error(err_);
   for (int i = 0; i <= kMaxKrylov; ++i) {
     cudaEventCreateWithFlags(&ev_iter_[i], cudaEventDisableTiming);
@@ -757,7 +759,7 @@ Engine::Engine(const Params& p, int chi, uint64_t seed, int precision, cudaStrea
   ring_dev_ = (double*)dalloc(4 * (kMaxKrylov + 1) * sizeof(double));
   if (!check(cudaMallocHost(&ring_host_, 4 * (kMaxKrylov + 1) * sizeof(double)), "pinned ring"))
     throw std::runtime_error(err_);
-  cudaMemsetAsync(d_err_, 0, sizeof(int), stream_);
+  cudaMemsetAsync(d_err_, 0, 8 * sizeof(int), stream_);
   long long dmax = 1;
   for (const Sectors& b : bonds_) dmax = std::max<long long>(dmax, b.total());
   qr_G_ = (double*)dalloc(dmax * dmax * sizeof(double));
@@ -2710,8 +2712,7 @@ int Engine::lanczos(int node, double tol, int max_krylov, bool mixed, int max_re
 // drivers).  Scalars live in d_scal_: alpha[128], beta[128], s[128], out,
 // Gram-Schmidt coefficients, norms; a thick restart's k x keep combination.
 namespace {
-constexpr int kAlpha = 0, kBeta = 128, kSvec = 256, kOut = 384, kCoef = 512, kNrm2 = 640, kNrmPre = 641,
-              kNrmMid = 642, kCmat = 1024, kC1 = 2048, kC2 = 2304, kMid = 2500, kNrmSecond = 2501;
+constexpr int kAlpha = 0, kBeta = 128, kSvec = 256, kOut = 384, kNrm2 = 640, kCmat = 1024, kC1 = 2048;
 }
 
 int Engine::lz_prepare(int kmax) {
@@ -2746,18 +2747,26 @@ void Engine::lz_start(int node) {
 // second pass only if the first removed more than half of ||w'||^2 (Daniel-
 // Gragg-Kaufman-Stewart, decided on the device), beta_j = ||w|| and
 // v_{j+1} = w / beta_j (column kmax holds the residual vector of a full
-// cycle).  Eleven launches.
-void Engine::lz_iteration(int j, long long n) {
-  launch_lz_reorth(V_, nmax_, j + 1, y_out_, n, d_partial_, d_scal_ + kC1, d_scal_ + kC2, d_scal_ + kMid,
-                   d_scal_ + kNrmSecond, kReorthRatio, d_scal_ + kAlpha + j, j > 0 ? d_scal_ + kBeta + j - 1 : nullptr,
-                   d_scal_ + kBeta + j, d_scal_ + kNrm2, V_ + (long long)(j + 1) * nmax_, stream_,
-                   precision_ != PREC_FP64 ? 1 : 0);
-}
-
-// v_{j+1} is written by lz_iteration.
-void Engine::lz_next_vector(int j, long long n) {
-  (void)j;
-  (void)n;
+// cycle).  One launch (kernels_lz.cu).
+int Engine::lz_iteration(int j, long long n) {
+  LzStep p{};
+  p.V = V_;
+  p.ldq = nmax_;
+  p.k = j + 1;
+  p.y = y_out_;
+  p.n = n;
+  p.partial = d_partial_;
+  p.coef = d_scal_ + kC1;
+  p.ratio = kReorthRatio;
+  p.alpha_j = d_scal_ + kAlpha + j;
+  p.beta_prev = j > 0 ? d_scal_ + kBeta + j - 1 : nullptr;
+  p.beta_j = d_scal_ + kBeta + j;
+  p.v_next = V_ + (long long)(j + 1) * nmax_;
+  p.bar = (unsigned*)(d_err_ + 4);
+  p.err = d_err_ + 3;
+  const int rc = launch_lz_step(p, precision_ != PREC_FP64 ? 1 : 0, stream_);
+  if (rc) err_ = "Lanczos step launch failed";
+  return rc;
 }
 
 // Thick restart after a full cycle of k vectors (see lanczos_restart_kernel);
@@ -2800,6 +2809,18 @@ void Engine::lz_finish(int node, int k) {
   launch_dot(tmp_, tmp_, n, d_partial_, d_scal_ + kNrm2, stream_);
   launch_scale_inv_sqrt(tmp_, T_[node], n, d_scal_ + kNrm2, stream_);
   cudaMemcpyAsync(ring_host_ + 4 * kMaxKrylov, d_scal_ + kOut, 2 * sizeof(double), cudaMemcpyDeviceToHost, stream_);
+  cudaMemcpyAsync(ring_host_ + 4 * kMaxKrylov + 2, d_err_ + 3, sizeof(int), cudaMemcpyDeviceToHost, stream_);
+}
+
+// After the synchronisation behind lz_finish: -6 if a grid barrier of a
+// Lanczos step ran out (the flag is cleared for the next update).
+int Engine::lz_waits() {
+  int flag = 0;
+  std::memcpy(&flag, ring_host_ + 4 * kMaxKrylov + 2, sizeof(int));
+  if (!flag) return 0;
+  cudaMemsetAsync(d_err_ + 3, 0, sizeof(int), stream_);
+  err_ = "Lanczos step: a grid barrier hit its iteration limit";
+  return -6;
 }
 
 // Convergence data of iteration j (lowest Ritz pair of T_{j+1}, beta_j) into
@@ -2851,9 +2872,8 @@ int Engine::lanczos_run(int node, double tol, int max_krylov, bool mixed, int ma
     for (int j = j0; j < kmax; ++j) {
       if ((rc = apply_heff(V_ + j * nmax_, y_out_, -1))) return rc;
       ++total_iters;
-      lz_iteration(j, n);
+      if ((rc = lz_iteration(j, n))) return rc;
       lz_queue_check(j);
-      lz_next_vector(j, n);
       k = j + 1;
       if (!speculate) {
         if (!check(cudaEventSynchronize(ev_conv_[j]), "lanczos")) return -3;
@@ -2888,6 +2908,7 @@ int Engine::lanczos_run(int node, double tol, int max_krylov, bool mixed, int ma
   // a speculative iteration's convergence data may still be in flight
   if (last_conv_ >= 0 && !check(cudaEventSynchronize(ev_conv_[last_conv_]), "lanczos end")) return -3;
   last_conv_ = -1;
+  if ((rc = lz_waits())) return rc;
   *energy = ring_host_[4 * kMaxKrylov];
   *resid = ring_host_[4 * kMaxKrylov + 1];
   *iters = total_iters;

@@ -521,8 +521,8 @@ class Engine {
   // Lanczos building blocks
   int lz_prepare(int kmax);
   void lz_start(int node);
-  void lz_iteration(int j, long long n);
-  void lz_next_vector(int j, long long n);
+  int lz_iteration(int j, long long n);
+  int lz_waits();
   int lz_thick_restart(int k, int kmax, long long n, int* j0);
   void lz_finish(int node, int k);
   void lz_queue_check(int j);

@@ -104,11 +104,15 @@ __device__ __forceinline__ float to_t<float>(double v) { return d2f_bits(v); }
 template <>
 __device__ __forceinline__ ff to_t<ff>(double v) { return d2ff(v); }
 
-__device__ __forceinline__ ff d2ff(double d) {
+// Values outside the range of the short form below: zeros, magnitudes below
+// 2^-103 (whose lo part nears the FP32 subnormals) or past the FP32 range,
+// infinities and NaN.
+static __device__ __noinline__ ff d2ff_edge(double d) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(d);
   const float hi = d2f_bits(__longlong_as_double((long long)(b & ~((1ull << 29) - 1ull))));
   const int e = (int)((b >> 52) & 0x7ff);
   const unsigned low = (unsigned)(b & ((1ull << 29) - 1ull));
+  if (e == 0x7ff && low) return ff(__uint_as_float(0x7fc00000u), 0.f);
   float lo = 0.f;
   if (e != 0 && e != 0x7ff && low) {
     // low x 2^(e - 1075): convert the integer, then move its exponent
@@ -118,6 +122,18 @@ __device__ __forceinline__ ff d2ff(double d) {
     if (b >> 63) lo = -lo;
   }
   return ff(hi, lo);
+}
+
+// hi: the sign, the exponent rebiased by 896 and the top 23 fraction bits; lo:
+// the other 29 bits as an integer, rounded to 24, times 2^-29 of hi's last
+// place (a power of two taken from hi's own exponent field).
+__device__ __forceinline__ ff d2ff(double d) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  const unsigned top = h & 0x7fffffffu;
+  if (top - (920u << 20) >= (230u << 20)) return top == 0u && l == 0u ? ff(0.f) : d2ff_edge(d);   // 920 <= e < 1150
+  const unsigned hb = ((__funnelshift_l(l, h, 3) - (384u << 23)) & 0x7fffffffu) | (h & 0x80000000u);
+  const float ulp = __uint_as_float((hb & 0xff800000u) - (23u << 23));
+  return ff(__uint_as_float(hb), ((float)(l & 0x1fffffffu) * 0x1p-29f) * ulp);
 }
 
 template <typename T>

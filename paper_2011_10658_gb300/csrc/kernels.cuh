@@ -117,32 +117,36 @@ void launch_bh(const BhTile* tiles, int n_tiles, const BhOut* outs, const BhChun
 // ---- vector kernels (FP64) ----
 // partial sums per block then a single-block finish: deterministic.
 void launch_dot(const double* x, const double* y, long long n, double* partial, double* out, cudaStream_t s);
-// out[j] = <Q_j, w> for j < k (Q columns of length n, stride ldq).
-// Optional gate (device scalars): the call does nothing when
-// *gate_num >= ratio * *gate_den (a skipped reorthogonalisation pass).
-void launch_multidot(const double* Q, long long ldq, int k, const double* w, long long n, double* partial,
-                     double* out, cudaStream_t s, const double* gate_num = nullptr, const double* gate_den = nullptr,
-                     double ratio = 0.0);
-// w -= sum_j Q_j c[j]  (same optional gate)
-void launch_multiaxpy(const double* Q, long long ldq, int k, const double* c, double* w, long long n,
-                      cudaStream_t s, const double* gate_num = nullptr, const double* gate_den = nullptr,
-                      double ratio = 0.0);
 // x = sum_j c[j] Q_j
 void launch_combine(const double* Q, long long ldq, int k, const double* c, double* x, long long n, cudaStream_t s);
-// One Lanczos step after y = H v_{k-1} (V holds v_0 .. v_{k-1}, columns of
-// stride ldq): alpha_j = v_j . y, the three-term residual
+// One Lanczos step after y = H v_{k-1} (kernels_lz.cu; V holds v_0 .. v_{k-1},
+// columns of stride ldq, k <= 128): alpha_j = v_j . y, the three-term residual
 // w' = y - alpha_j v_j - beta_{j-1} v_{j-1} (beta_prev, unused for k = 1),
-// classical Gram-Schmidt of w' against all k vectors (c1 = V^T w', w'.w' in
-// c1[k]), a second pass into c2 when the Daniel-Gragg-Kaufman-Stewart test
-// asks for it (decided on the device), then beta_j = |w|, *nrm_out = |w|^2
-// and v_next = w / |w|.  Eleven launches; partial holds 1216 x (k + 1)
-// doubles; c1 k + 1 and c2 k doubles; k <= 128.  ff_arith != 0: the dots and
-// updates in float-float arithmetic on the FP32 pipes (about 2^-44 relative
-// rounding per operation; the data stay FP64).
-void launch_lz_reorth(const double* V, long long ldq, int k, double* y, long long n, double* partial, double* c1,
-                      double* c2, double* mid, double* nrm_second, double ratio, double* alpha_j,
-                      const double* beta_prev, double* beta_j, double* nrm_out, double* v_next, cudaStream_t s,
-                      int ff_arith = 0);
+// classical Gram-Schmidt of w' against all k vectors, a second pass when the
+// first left less than ratio |w'|^2 (Daniel-Gragg-Kaufman-Stewart, decided on
+// the device), then beta_j = |w| and v_next = w / |w|.  y is overwritten.
+// partial: kLzPartial doubles; coef: 256 doubles; bar: two zeroed counters,
+// zero again afterwards; *err set if a wait ran out.  ff_arith != 0: dots
+// and updates in float-float arithmetic (the data stay FP64).
+struct LzStep {
+  const double* V;
+  long long ldq;
+  int k;
+  double* y;
+  long long n;
+  double* partial;
+  double* coef;
+  double ratio;
+  double* alpha_j;
+  const double* beta_prev;
+  double* beta_j;
+  double* v_next;
+  unsigned* bar;
+  int* err;
+};
+constexpr int kLzMaxBlocks = 1024;
+constexpr long long kLzPartial = 132LL * kLzMaxBlocks;
+int launch_lz_step(const LzStep& p, int ff_arith, cudaStream_t s);
 // out[0] = sqrt(max(in[0], 0))
 void launch_sqrt(const double* in, double* out, cudaStream_t s);
 // y = a*x + b*y with a, b read from device scalars (nullable -> constants)
