@@ -179,9 +179,11 @@ void launch_cgs2_qr(double* X, const long long* xoff, const int* rows, const int
 // Lowest eigenvalue of the symmetric tridiagonal (alpha[0..k), beta[0..k-1))
 // (1 <= k <= 128).  out[0] = theta, out[1] = |beta[k-1] * s_k| (Ritz residual
 // estimate; beta[k-1] is the trailing coupling).  With want_vec, s[0..k) gets
-// the unit eigenvector (s[0] >= 0) and out[0] its Rayleigh quotient.
+// the unit eigenvector (s[0] >= 0) and out[0] its Rayleigh quotient.  prev
+// (optional, device): an upper bound of theta, e.g. the value for a smaller
+// basis of the same run; a wrong one costs a round, not the result.
 void launch_tridiag_lowest(const double* alpha, const double* beta, int k, double* out, double* svec, int want_vec,
-                           cudaStream_t s);
+                           cudaStream_t s, const double* prev = nullptr);
 // Thick restart (keep the m <= 8 lowest Ritz pairs of the k x k tridiagonal,
 // k <= 128): writes the k x p combination C (row-major), the new leading
 // p x p tridiagonal into alpha/beta with beta[p-1] the coupling to the

@@ -447,27 +447,6 @@ __device__ int sturm_minors(const double* a, const double* b2, int k, double x) 
   return cnt;
 }
 
-// -p_{k-1}(x) / p_k'(x): the squared last component of the unit eigenvector
-// of an eigenvalue x (ratio of the minor below to the derivative).
-__device__ double last_component_sq(const double* a, const double* b2, int k, double x) {
-  if (k == 1) return 1.0;
-  double pm = 1.0, p = a[0] - x, dm = 0.0, d = -1.0;
-  for (int i = 1; i < k; ++i) {
-    const double t = a[i] - x;
-    const double pn = fma(t, p, -b2[i - 1] * pm);
-    const double dn = fma(t, d, -fma(b2[i - 1], dm, p));
-    pm = p; p = pn; dm = d; d = dn;
-    const int e = dexp(p) > dexp(d) ? dexp(p) : dexp(d);
-    if (e > 1023 + 512) {
-      p *= 0x1p-512; pm *= 0x1p-512; d *= 0x1p-512; dm *= 0x1p-512;
-    } else if (e < 1023 - 512 && dexp(pm) < 1023 - 512 && dexp(dm) < 1023 - 512) {
-      p *= 0x1p+512; pm *= 0x1p+512; d *= 0x1p+512; dm *= 0x1p+512;
-    }
-  }
-  const double r = d != 0.0 ? -pm / d : 1.0;
-  return fmin(fmax(r, 0.0), 1.0);
-}
-
 // Eigenvector of T for the eigenvalue theta: inverse iteration with a shift
 // just below theta, tridiagonal LU (Thomas), orthogonalised against the
 // n_prev rows of prev (stride ld) (vectors of lower eigenvalues of a
@@ -506,43 +485,51 @@ __device__ void inverse_iteration(const double* a, const double* b, int k, doubl
     for (int i = 0; i < k; ++i) x[i] = -x[i];
 }
 
-// Warp-collective multisection for the eigenvalue of index idx (0 = lowest):
-// on entry [lo, hi] holds it (count(lo) <= idx < count(hi)); each round the 32
-// lanes count at 32 interior points and the bracket shrinks 33-fold, until it
-// is a few ulps wide.  All lanes return the same bracket.
-__device__ void multisect(const double* a, const double* b2, int k, int idx, double& lo, double& hi) {
-  const int lane = threadIdx.x & 31;
+// Multisection for the eigenvalue of index idx (0 = lowest) by N threads, of
+// which this is thread t: on entry [lo, hi] holds it (count(lo) <= idx <
+// count(hi)); each round counts at N interior points, and the bracket shrinks
+// (N + 1)-fold, until it is a few ulps wide.  below(above) returns how many of
+// the N threads are not above.  All threads return the same bracket.
+template <int N, typename Below>
+__device__ void multisect(const double* a, const double* b2, int k, int idx, int t, Below below, double& lo,
+                          double& hi) {
   for (int round = 0; round < 64; ++round) {
     const double w = hi - lo;
     if (w <= 4.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + 1e-300) break;
-    const double x = lo + w * ((double)(lane + 1) * (1.0 / 33.0));
-    const unsigned above = __ballot_sync(0xffffffffu, sturm_minors(a, b2, k, x) > idx);
-    double nlo, nhi;
-    if (above == 0u) {
-      nlo = __shfl_sync(0xffffffffu, x, 31);
-      nhi = hi;
-    } else {
-      const int f = __ffs(above) - 1;
-      nhi = __shfl_sync(0xffffffffu, x, f);
-      const double xl = __shfl_sync(0xffffffffu, x, f > 0 ? f - 1 : 0);
-      nlo = f > 0 ? xl : lo;
-    }
+    const double x = lo + w * ((double)(t + 1) * (1.0 / (N + 1)));
+    const int f = below(sturm_minors(a, b2, k, x) > idx);
+    const double nlo = f > 0 ? lo + w * ((double)f * (1.0 / (N + 1))) : lo;
+    const double nhi = f < N ? lo + w * ((double)(f + 1) * (1.0 / (N + 1))) : hi;
     if (!(nhi - nlo < w)) break;   // no progress left at this precision
     lo = nlo;
     hi = nhi;
   }
 }
 
-// Warp-collective: stage (a, b, b2) of the tridiagonal in shared memory and
-// return its Gershgorin bracket (widened) and scale.
+struct WarpBelow {
+  __device__ int operator()(bool above) const { return 32 - __popc(__ballot_sync(0xffffffffu, above)); }
+};
+template <int N>
+struct BlockBelow {
+  __device__ int operator()(bool above) const { return N - __syncthreads_count(above); }
+};
+
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Warp-collective: stage (a, b, b2) of the tridiagonal and 1 / b in shared
+// memory and return its Gershgorin bracket (widened) and scale.
 __device__ void stage_tridiag(const double* alpha, const double* beta, int k, double* a, double* b, double* b2,
-                              double& lo, double& hi, double& scale) {
+                              double* ib, double& lo, double& hi, double& scale) {
   const int lane = threadIdx.x & 31;
   for (int i = lane; i < k; i += 32) {
     a[i] = alpha[i];
     const double bi = i < k - 1 ? beta[i] : 0.0;
     b[i] = bi;
     b2[i] = bi * bi;
+    ib[i] = i < k - 1 ? 1.0 / bi : 0.0;
   }
   __syncwarp();
   lo = 1e300;
@@ -562,39 +549,139 @@ __device__ void stage_tridiag(const double* alpha, const double* beta, int k, do
   hi += 1e-12 * span + 1e-300;
 }
 
-// One warp.  out[0] = theta (lowest eigenvalue), out[1] = |beta[k-1]| |s_k|
-// (the Ritz residual estimate).  With want_vec the eigenvector goes to s and
-// out[0] is its Rayleigh quotient; the vector is also formed when s_k is
-// too small for the minor ratio to resolve.
-__global__ void __launch_bounds__(32) tridiag_lowest_kernel(const double* __restrict__ alpha,
-                                                            const double* __restrict__ beta, int k, double* out,
-                                                            double* s, int want_vec) {
-  __shared__ double a[TRI_MAX], b[TRI_MAX], b2[TRI_MAX];
-  double lo, hi, scale;
-  stage_tridiag(alpha, beta, k, a, b, b2, lo, hi, scale);
-  multisect(a, b2, k, 0, lo, hi);
-  if (threadIdx.x != 0) return;
-  const double theta = 0.5 * (lo + hi);
-  double sk = sqrt(last_component_sq(a, b2, k, theta));
-  double th = theta;
-  if (want_vec || sk < 1e-4) {
-    double x[TRI_MAX];
-    inverse_iteration(a, b, k, theta, scale, want_vec ? 3 : 2, x, nullptr, 0, 0);
-    sk = fabs(x[k - 1]);
-    if (want_vec) {
-      double rq = 0.0;
-      for (int i = 0; i < k; ++i) {
-        double v = a[i] * x[i];
-        if (i > 0) v += b[i - 1] * x[i - 1];
-        if (i < k - 1) v += b[i] * x[i + 1];
-        rq += x[i] * v;
-      }
-      th = rq;
-      for (int i = 0; i < k; ++i) s[i] = x[i];
+// Warp-collective eigenvector of T for the eigenvalue theta, by the three-term
+// recurrences from both ends joined where they fit best (the twisted
+// factorisation of Parlett and Dhillon): with f running down from f_0 = 1 and
+// g up from g_{k-1} = 1, row r of (T - theta) x misses zero by
+//   gamma_r = (a_r - theta) + b_{r-1} f_{r-1} / f_r + b_r g_{r+1} / g_r
+// when x is f / f_r above r and g / g_r below; r is the row of least |gamma|.
+// Lanes 0 and 1 run the two recurrences in step; the rest is parallel.  f, g,
+// c1: k, k and 2 k doubles of shared memory; f returns the unit vector (first
+// component >= 0 with pos).  False if no row has a finite gamma (the
+// recurrences left the FP64 range), f then undefined.
+__device__ bool twisted_vector(const double* a, const double* b, const double* ib, int k, double theta, bool pos,
+                               double* f, double* g, double* c1) {
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < k; i += 32) {
+    const double t = theta - a[i];
+    c1[i] = t * ib[i];                                // f_{i+1} = c1[i] f_i - (b_{i-1} / b_i) f_{i-1}
+    c1[k + k - 1 - i] = i > 0 ? t * ib[i - 1] : 0.0;  // g_{i-1} likewise, stored in running order
+  }
+  __syncwarp();
+  if (lane < 2) {
+    const bool down = lane == 0;
+    double* out = down ? f : g;
+    const double* c = down ? c1 : c1 + k;
+    double pm = 0.0, p = 1.0;
+    int at = down ? 0 : k - 1;
+    const int dir = down ? 1 : -1;
+    out[at] = 1.0;
+    for (int i = 0; i + 1 < k; ++i) {
+      // coupling ratio to the entry before: b_{i-1} / b_i going down
+      const int lo = down ? i - 1 : k - 1 - i, hi = down ? i : k - 2 - i;
+      const double q = i > 0 ? b[lo] * ib[hi] : 0.0;
+      const double pn = fma(c[i], p, -q * pm);
+      pm = p;
+      p = pn;
+      at += dir;
+      out[at] = p;
     }
   }
-  out[0] = th;
-  out[1] = fabs(beta[k - 1]) * sk;
+  __syncwarp();
+  double best = 1e308;
+  int r = -1;
+  for (int i = lane; i < k; i += 32) {
+    double gm = a[i] - theta;
+    if (i > 0) gm += b[i - 1] * (f[i - 1] / f[i]);
+    if (i < k - 1) gm += b[i] * (g[i + 1] / g[i]);
+    gm = fabs(gm);
+    if (gm < best) { best = gm; r = i; }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int orr = __shfl_xor_sync(0xffffffffu, r, o);
+    if (orr >= 0 && (ob < best || (ob == best && (r < 0 || orr < r)))) { best = ob; r = orr; }
+  }
+  if (r < 0) return false;
+  const double fi = 1.0 / f[r], gi = 1.0 / g[r];
+  __syncwarp();
+  double n2 = 0.0;
+  for (int i = lane; i < k; i += 32) {
+    const double x = i <= r ? f[i] * fi : g[i] * gi;
+    f[i] = x;
+    n2 = fma(x, x, n2);
+  }
+  n2 = warp_sum(n2);
+  __syncwarp();
+  const double inv = (pos && f[0] < 0.0 ? -1.0 : 1.0) / sqrt(n2);
+  __syncwarp();
+  for (int i = lane; i < k; i += 32) f[i] *= inv;
+  __syncwarp();
+  return isfinite(inv) && n2 >= 1.0;
+}
+
+// Four warps (one per scheduler: a warp's FP64 instruction holds its
+// scheduler's pipe for 64 cycles, so four warps count at four times the points
+// in the same time).  out[0] = theta (lowest eigenvalue), out[1] = |beta[k-1]|
+// |s_k| (the Ritz residual estimate).  With want_vec the eigenvector goes to s
+// and out[0] is its Rayleigh quotient.  prev (optional): the lowest Ritz value
+// of a smaller basis of the same run, an upper bound of theta; the first round
+// then counts at distances from it that halve every second or third point.
+// GB300: 100 us on average over an FP64 sweep of 2x2x2 before (32 points a
+// round, inverse iteration in one lane for small s_k), 12-90 us now (k = 1-64).
+constexpr int TRI_THREADS = 128;
+
+__global__ void __launch_bounds__(TRI_THREADS) tridiag_lowest_kernel(const double* __restrict__ alpha,
+                                                                     const double* __restrict__ beta, int k,
+                                                                     double* out, double* s, int want_vec,
+                                                                     const double* prev) {
+  __shared__ double a[TRI_MAX], b[TRI_MAX], b2[TRI_MAX], ib[TRI_MAX];
+  __shared__ double f[TRI_MAX], g[TRI_MAX], c1[2 * TRI_MAX], bracket[3];
+  const int t = threadIdx.x;
+  double lo, hi, scale;
+  if (t < 32) {
+    stage_tridiag(alpha, beta, k, a, b, b2, ib, lo, hi, scale);
+    if (t == 0) { bracket[0] = lo; bracket[1] = hi; bracket[2] = scale; }
+  }
+  __syncthreads();
+  lo = bracket[0];
+  hi = bracket[1];
+  scale = bracket[2];
+  const BlockBelow<TRI_THREADS> below;
+  if (prev) {
+    const double top = *prev + 4.0 * DBL_EPSILON * scale, w = top - lo;
+    if (w > 0.0 && top < hi) {
+      // distances w 2^(-55 t / 128) below top; the last point is top itself
+      auto point = [&](int i) { return i == TRI_THREADS - 1 ? top : top - w * exp2(-55.0 / TRI_THREADS * i); };
+      const int n = below(sturm_minors(a, b2, k, point(t)) > 0);
+      if (n > 0) lo = fmax(lo, point(n - 1));
+      if (n < TRI_THREADS) hi = point(n);
+    }
+  }
+  multisect<TRI_THREADS>(a, b2, k, 0, t, below, lo, hi);
+  if (t >= 32) return;
+  const double theta = 0.5 * (lo + hi);
+  const bool ok = twisted_vector(a, b, ib, k, theta, true, f, g, c1);
+  if (!ok) {
+    if (t == 0) inverse_iteration(a, b, k, theta, scale, 3, f, nullptr, 0, 0);
+    __syncwarp();
+  }
+  double th = theta;
+  if (want_vec) {
+    double rq = 0.0;
+    for (int i = t; i < k; i += 32) {
+      double v = a[i] * f[i];
+      if (i > 0) v += b[i - 1] * f[i - 1];
+      if (i < k - 1) v += b[i] * f[i + 1];
+      rq = fma(f[i], v, rq);
+      s[i] = f[i];
+    }
+    th = warp_sum(rq);
+  }
+  if (t == 0) {
+    out[0] = th;
+    out[1] = fabs(beta[k - 1]) * fabs(f[k - 1]);
+  }
 }
 
 // Thick restart of a Lanczos cycle (Wu and Simon's thick-restart Lanczos).
@@ -606,75 +693,112 @@ __global__ void __launch_bounds__(32) tridiag_lowest_kernel(const double* __rest
 // last vector alone couples to r with |c|, so the next cycle continues the
 // ordinary three-term recurrence from r at position p.  Writes C = S U
 // reversed (k x p, row-major: C[r * p + i]), alpha[0..p), beta[0..p) (beta[p-1]
-// = |c|) and *p_out.  One warp; serial parts in lane 0.
-__global__ void __launch_bounds__(32) lanczos_restart_kernel(double* alpha, double* beta, int k, int m, double* C,
-                                                             int* p_out) {
-  __shared__ double a[TRI_MAX], b[TRI_MAX], b2[TRI_MAX];
-  __shared__ double S[RESTART_MAX][TRI_MAX];
-  __shared__ double th[RESTART_MAX];
-  double glo, ghi, scale;
-  stage_tridiag(alpha, beta, k, a, b, b2, glo, ghi, scale);
+// = |c|) and *p_out.  One warp per Ritz pair; then the vectors of a cluster
+// are made orthogonal to the lower ones, and the small Lanczos process runs
+// on the lanes of warp 0.  GB300, k = 64: 375 us; 3.5 ms in one lane.
+__global__ void __launch_bounds__(32 * RESTART_MAX) lanczos_restart_kernel(double* alpha, double* beta, int k, int m,
+                                                                           double* C, int* p_out) {
+  __shared__ double a[TRI_MAX], b[TRI_MAX], b2[TRI_MAX], ib[TRI_MAX];
+  __shared__ double S[RESTART_MAX][TRI_MAX], G[RESTART_MAX][TRI_MAX], c1[RESTART_MAX][2 * TRI_MAX];
+  __shared__ double th[RESTART_MAX], U[RESTART_MAX][RESTART_MAX], bracket[3];
+  __shared__ int good[RESTART_MAX], p_kept;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp == 0) {
+    double glo, ghi, scale;
+    stage_tridiag(alpha, beta, k, a, b, b2, ib, glo, ghi, scale);
+    if (lane == 0) { bracket[0] = glo; bracket[1] = ghi; bracket[2] = scale; }
+  }
+  __syncthreads();
+  const double scale = bracket[2];
   if (m > k) m = k;
-  for (int i = 0; i < m; ++i) {
-    double lo = glo, hi = ghi;
-    multisect(a, b2, k, i, lo, hi);
-    if (threadIdx.x == 0) th[i] = 0.5 * (lo + hi);
+  if (warp < m) {
+    double lo = bracket[0], hi = bracket[1];
+    multisect<32>(a, b2, k, warp, lane, WarpBelow(), lo, hi);
+    const double theta = 0.5 * (lo + hi);
+    const bool ok = twisted_vector(a, b, ib, k, theta, warp == 0, S[warp], G[warp], c1[warp]);
+    if (lane == 0) { th[warp] = theta; good[warp] = ok; }
   }
-  __syncwarp();
-  if (threadIdx.x != 0) return;
+  __syncthreads();
   const double bk = beta[k - 1];
-  double c[RESTART_MAX];
-  for (int i = 0; i < m; ++i) {
-    inverse_iteration(a, b, k, th[i], scale, 3, S[i], &S[0][0], TRI_MAX, i);
-    c[i] = bk * S[i][k - 1];
-  }
-  // Lanczos on diag(theta) from c / |c| with full reorthogonalisation
-  double cn = 0.0;
-  for (int i = 0; i < m; ++i) cn += c[i] * c[i];
-  cn = sqrt(cn);
-  double U[RESTART_MAX][RESTART_MAX];
-  double la[RESTART_MAX], lb[RESTART_MAX];
-  int p = 0;
-  if (cn > 0.0) {
-    for (int i = 0; i < m; ++i) U[0][i] = c[i] / cn;
-    p = 1;
-    for (int j = 0; j < m; ++j) {
-      double w[RESTART_MAX];
-      for (int i = 0; i < m; ++i) w[i] = th[i] * U[j][i];
-      double aj = 0.0;
-      for (int i = 0; i < m; ++i) aj += U[j][i] * w[i];
-      la[j] = aj;
-      for (int pass = 0; pass < 2; ++pass)
-        for (int q = 0; q <= j; ++q) {
-          double h = 0.0;
-          for (int i = 0; i < m; ++i) h += U[q][i] * w[i];
-          for (int i = 0; i < m; ++i) w[i] -= h * U[q][i];
+  if (warp == 0) {
+    // orthogonal to the lower vectors (twice); a vector that mostly lies in
+    // their span comes from a cluster and is formed by inverse iteration there
+    for (int i = 0; i < m; ++i) {
+      bool ok = good[i] != 0;
+      if (ok)
+        for (int pass = 0; pass < 2; ++pass) {
+          for (int q = 0; q < i; ++q) {
+            double h = 0.0;
+            for (int r = lane; r < k; r += 32) h = fma(S[q][r], S[i][r], h);
+            h = warp_sum(h);
+            for (int r = lane; r < k; r += 32) S[i][r] = fma(-h, S[q][r], S[i][r]);
+          }
+          double n2 = 0.0;
+          for (int r = lane; r < k; r += 32) n2 = fma(S[i][r], S[i][r], n2);
+          n2 = warp_sum(n2);
+          if (pass == 0 && n2 < 0.5) { ok = false; break; }
+          const double inv = 1.0 / sqrt(n2);
+          for (int r = lane; r < k; r += 32) S[i][r] *= inv;
         }
-      double bj = 0.0;
-      for (int i = 0; i < m; ++i) bj += w[i] * w[i];
-      bj = sqrt(bj);
-      if (j + 1 >= m || bj <= 1e-13 * fmax(scale, 1e-300)) break;
-      lb[j] = bj;
-      for (int i = 0; i < m; ++i) U[j + 1][i] = w[i] / bj;
-      p = j + 2;
+      __syncwarp();
+      if (!ok && lane == 0) inverse_iteration(a, b, k, th[i], scale, 3, S[i], &S[0][0], TRI_MAX, i);
+      __syncwarp();
+    }
+    // Lanczos on diag(theta) from c / |c| with full reorthogonalisation, one
+    // kept pair per lane
+    const bool in = lane < m;
+    const double c = in ? bk * S[in ? lane : 0][k - 1] : 0.0, t = in ? th[in ? lane : 0] : 0.0;
+    const double cn = sqrt(warp_sum(c * c));
+    double u[RESTART_MAX], la[RESTART_MAX], lb[RESTART_MAX];
+    int p = 0;
+    if (cn > 0.0) {
+      u[0] = c / cn;
+      p = 1;
+#pragma unroll
+      for (int j = 0; j < RESTART_MAX; ++j) {
+        if (j >= m || j >= p) break;
+        double w = t * u[j];
+        la[j] = warp_sum(u[j] * w);
+        for (int pass = 0; pass < 2; ++pass)
+#pragma unroll
+          for (int q = 0; q <= j; ++q) w = fma(-warp_sum(u[q] * w), u[q], w);
+        const double bj = sqrt(warp_sum(w * w));
+        if (j + 1 >= m || bj <= 1e-13 * fmax(scale, 1e-300)) break;
+        if (j + 1 < RESTART_MAX) {
+          lb[j] = bj;
+          u[j + 1] = w / bj;
+        }
+        p = j + 2;
+      }
+    }
+    if (p == 0) {   // r decoupled: keep the lowest Ritz vector alone
+      p = 1;
+      u[0] = lane == 0 ? 1.0 : 0.0;
+      la[0] = th[0];
+    }
+#pragma unroll
+    for (int i = 0; i < RESTART_MAX; ++i)
+      if (i < p) {
+        if (in) U[i][lane] = u[i];
+        if (lane == 0) {   // reversed tridiagonal
+          alpha[p - 1 - i] = la[i];
+          if (i + 1 < p) beta[p - 2 - i] = lb[i];
+        }
+      }
+    if (lane == 0) {
+      beta[p - 1] = cn;
+      *p_out = p_kept = p;
     }
   }
-  if (p == 0) {   // r decoupled: keep the lowest Ritz vector alone
-    p = 1;
-    for (int i = 0; i < m; ++i) U[0][i] = i == 0 ? 1.0 : 0.0;
-    la[0] = th[0];
+  __syncthreads();
+  // C[:, i] = S^T U[p-1-i]
+  const int p = p_kept;
+  for (int e = threadIdx.x; e < k * p; e += blockDim.x) {
+    const int r = e / p, i = e - r * p;
+    double v = 0.0;
+    for (int q = 0; q < m; ++q) v = fma(S[q][r], U[p - 1 - i][q], v);
+    C[e] = v;
   }
-  // C[:, i] = S^T U[p-1-i] (reversed), new tridiagonal reversed
-  for (int r = 0; r < k; ++r)
-    for (int i = 0; i < p; ++i) {
-      double v = 0.0;
-      for (int q = 0; q < m; ++q) v += S[q][r] * U[p - 1 - i][q];
-      C[r * p + i] = v;
-    }
-  for (int i = 0; i < p; ++i) alpha[i] = la[p - 1 - i];
-  for (int i = 0; i + 1 < p; ++i) beta[i] = lb[p - 2 - i];
-  beta[p - 1] = cn;
-  *p_out = p;
 }
 
 // Z[:, i] = sum_r V[:, r] C[r * p + i] for i < p (p <= RESTART_MAX).
@@ -829,7 +953,7 @@ void launch_cgs2_qr(double* X, const long long* xoff, const int* rows, const int
 
 void launch_lanczos_restart(double* alpha, double* beta, int k, int m, double* C, int* p_out, cudaStream_t st) {
   if (k <= 0 || k > TRI_MAX || m < 1 || m > RESTART_MAX) return;
-  lanczos_restart_kernel<<<1, 32, 0, st>>>(alpha, beta, k, m, C, p_out);
+  lanczos_restart_kernel<<<1, 32 * RESTART_MAX, 0, st>>>(alpha, beta, k, m, C, p_out);
   count_launches(1);
 }
 
@@ -841,9 +965,9 @@ void launch_rotate_basis(const double* V, long long ld, int k, const double* C, 
 }
 
 void launch_tridiag_lowest(const double* alpha, const double* beta, int k, double* out, double* s, int want_vec,
-                           cudaStream_t st) {
+                           cudaStream_t st, const double* prev) {
   if (k <= 0 || k > TRI_MAX) return;
-  tridiag_lowest_kernel<<<1, 32, 0, st>>>(alpha, beta, k, out, s, want_vec);
+  tridiag_lowest_kernel<<<1, TRI_THREADS, 0, st>>>(alpha, beta, k, out, s, want_vec, prev);
   count_launches(1);
 }
 
