@@ -93,11 +93,11 @@ int BatchRunner::build(int node, const std::vector<int>& members, std::unique_pt
       const int o0 = (int)b.outs.size(), c0 = (int)b.chunks.size(), a0 = (int)b.adds.size();
       for (TcTile tl : t->tiles) {
         tl.out += o0;
+        tl.chunk_begin += c0;
+        tl.chunk_end += c0;
         b.tiles.push_back(tl);
       }
       for (TcOutput o : t->outs) {
-        o.chunk_begin += c0;
-        o.chunk_end += c0;
         o.add_begin += a0;
         o.add_end += a0;
         b.outs.push_back(o);
@@ -197,9 +197,9 @@ int BatchRunner::launch(Grouped& g) {
   if (g.tc) {
     const int elem = e0->precision_ == PREC_BF16 ? 2 : 4;
     const int split = e0->precision_ == PREC_TF32X3 ? 1 : 0;
-    launch_convert(elem, split, g.tcp.d_xjobs, (int)g.tcp.xjobs.size(), g.tcp.x_max_elems, s);
+    launch_convert(elem, g.tcp.d_xjobs, (int)g.tcp.xjobs.size(), g.tcp.x_max_elems, 0, s);
     const int rc = launch_tc_heff(elem, split, g.tcp.d_tiles, (int)g.tcp.tiles.size(), g.tcp.d_outs, g.tcp.d_chunks,
-                                  g.tcp.d_adds, g.tcp.max_kpad, g.tcp.max_npad, e0->d_err_, s);
+                                  g.tcp.d_adds, g.tcp.max_kpad, g.tcp.max_npad, 0, e0->d_err_, s);
     if (rc) e0->err_ = "tensor-core H_eff: tile shape outside the supported range";
     return rc;
   }

@@ -353,10 +353,10 @@ void KPlan::release() {
 }
 
 void TcPlan::release() {
-  void* ptrs[6] = {d_tiles, d_outs, d_chunks, d_adds, d_xjobs, d_wjobs};
+  void* ptrs[7] = {d_tiles, d_outs, d_chunks, d_adds, d_order, d_xjobs, d_wjobs};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  d_tiles = nullptr; d_outs = nullptr; d_chunks = nullptr; d_adds = nullptr; d_xjobs = nullptr; d_wjobs = nullptr;
+  d_tiles = nullptr; d_outs = nullptr; d_chunks = nullptr; d_adds = nullptr; d_order = nullptr; d_xjobs = nullptr; d_wjobs = nullptr;
   for (size_t& c : cap) c = 0;
 }
 
@@ -959,6 +959,58 @@ const std::vector<RowMap>& Engine::site_ham_map(int node, int leg, int cls) {
   for (size_t oc = 0; oc < layout_[node].leg[2].q.size(); ++oc)
     maps.push_back(build_rowmap_sector(node, leg == 0 ? &diag : nullptr, leg == 1 ? &diag : nullptr, (int)oc,
                                        nullptr));
+  return rowmaps_[key] = maps;
+}
+
+// Term of the two sites of a bottom node alone, diagonal in their basis?
+bool Engine::local_diagonal(int node, int term) {
+  for (auto& so : terms_[term].ops) {
+    if (so.first != leg_site(node, 0) && so.first != leg_site(node, 1)) return false;
+    const SiteOp* op = site_op(lat_.parity(so.first), so.second);
+    for (int r = 0; r < kLocalDim; ++r)
+      if (op->src[r] >= 0 && op->src[r] != r) return false;
+  }
+  return true;
+}
+
+// Every diagonal term of the two sites (site energies, the penalty of their
+// link), one class or all, as one factor per row: a product then reads x once
+// for all of them.
+const std::vector<RowMap>& Engine::diagonal_map(int node, int cls) {
+  auto key = std::make_pair(node, -1100 - (cls + 1));
+  auto it = rowmaps_.find(key);
+  if (it != rowmaps_.end()) return it->second;
+  const Layout& L = layout_[node];
+  const int sl = leg_site(node, 0);
+  std::vector<double> diag((size_t)kLocalDim * kLocalDim, 0.0);
+  for (int k = 0; k < (int)terms_.size(); ++k) {
+    if ((cls >= 0 && terms_[k].cls != cls) || !local_diagonal(node, k)) continue;
+    const SiteOp* A = nullptr;
+    const SiteOp* B = nullptr;
+    for (auto& so : terms_[k].ops) (so.first == sl ? A : B) = site_op(lat_.parity(so.first), so.second);
+    for (int a = 0; a < kLocalDim; ++a)
+      for (int b = 0; b < kLocalDim; ++b)
+        if ((!A || A->src[a] >= 0) && (!B || B->src[b] >= 0))
+          diag[(size_t)a * kLocalDim + b] += terms_[k].coef * (A ? A->val[a] : 1.0) * (B ? B->val[b] : 1.0);
+  }
+  std::vector<RowMap> maps(L.leg[2].q.size());
+  for (size_t oc = 0; oc < maps.size(); ++oc) {
+    const int rows = L.sec_rows[oc];
+    std::vector<double> val(rows, 0.0);
+    for (const Layout::Blk& b : L.blk) {
+      if (b.ic != (int)oc) continue;
+      const int a0 = L.leg[0].offset(b.ia), b0 = L.leg[1].offset(b.ib);
+      for (int i = 0; i < b.da; ++i)
+        for (int j = 0; j < b.db; ++j) val[b.row0 + i * b.db + j] = diag[(size_t)(a0 + i) * kLocalDim + b0 + j];
+    }
+    RowMap& rm = maps[oc];
+    for (double v : val) rm.nnz += v != 0.0;
+    if (!rm.nnz) continue;
+    rm.src_sector = (int)oc;
+    rm.val = (double*)dalloc(rows * sizeof(double));
+    cudaMemcpyAsync(rm.val, val.data(), rows * sizeof(double), cudaMemcpyHostToDevice, stream_);
+    cudaStreamSynchronize(stream_);
+  }
   return rowmaps_[key] = maps;
 }
 
@@ -1873,6 +1925,14 @@ void Engine::build_heff_terms(int node, int cls, std::vector<HTerm>* out) {
   }
 }
 
+// Part of diagonal_map (a term of the two sites of a bottom node, diagonal)?
+bool Engine::bottom_diagonal(int node, const HTerm& h) {
+  if (h.op[2].kind) return false;
+  for (int leg = 0; leg < 2; ++leg)
+    if (h.op[leg].kind == 2) return h.op[leg].term < 0 || local_diagonal(node, h.op[leg].term);
+  return false;
+}
+
 // H_eff plans of (node, class filter), built on first use and replayed.
 // Returns nullptr (err_ set) if validation fails.
 // adjoint: the transposed operator (every term applied as A^T (x) B^T (x) C^T),
@@ -1890,6 +1950,25 @@ Engine::HeffPlans* Engine::heff_plans(int node, int cls, bool adjoint) {
   KPlan& s3 = st[2];
   const int d2 = L.leg[2].total();
   const double cst = (cls < 0 || cls == CLS_NU) ? constant_ : 0.0;
+  // the diagonal terms of a bottom node's two sites are one valued add
+  auto in_diagonal = [&](const HTerm& h) { return bottom_diagonal(node, h); };
+  auto add_diagonal = [&](size_t oc) {
+    const RowMap& rm = diagonal_map(node, cls)[oc];
+    if (rm.src_sector < 0) return;
+    const int dc = L.leg[2].dim[oc];
+    KChunk c = make_chunk();
+    c.A = x_in_ + L.sec_off[oc]; c.a_m = dc; c.a_k = 1;
+    c.aval = rm.val; c.add = 1;
+    s3.add_output(y_out_ + L.sec_off[oc], dc, 1, L.sec_rows[oc], dc, 0);
+    s3.add_chunk(c);
+  };
+  if (bottom) {
+    // the row maps that ttn_apply_heff_device_noalloc looks up
+    for (int leg = 0; leg < 2; ++leg) site_ham_map(node, leg, cls);
+    for (const HTerm& h : hts)
+      for (int leg = 0; leg < 2; ++leg)
+        if (h.op[leg].kind == 2 && h.op[leg].term >= 0) rowmap(node, h.op[leg].term);
+  }
   if (bottom && adjoint) {
     // transposed terms: the forward chunk y_oc += x_ic[map] C[oc, ic]^T becomes
     // y_ic += x_oc[inverse map] C[oc, ic]
@@ -1908,13 +1987,13 @@ Engine::HeffPlans* Engine::heff_plans(int node, int cls, bool adjoint) {
     for (size_t oc = 0; oc < L.leg[2].q.size(); ++oc) {
       if (L.sec_rows[oc] == 0) continue;
       const int dco = L.leg[2].dim[oc];
+      add_diagonal(oc);
       for (const HTerm& h : hts) {
         const bool phys = h.op[0].kind == 2 || h.op[1].kind == 2;
         const RowMap* rm = nullptr;
         if (phys) {
-          if (h.op[0].kind == 2 && h.op[0].term < 0) rm = &site_ham_map(node, 0, h.op[0].cls)[oc];
-          else if (h.op[1].kind == 2 && h.op[1].term < 0) rm = &site_ham_map(node, 1, h.op[1].cls)[oc];
-          else rm = &rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term)[oc];
+          if (in_diagonal(h)) continue;
+          rm = &rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term)[oc];
           if (rm->src_sector < 0) continue;
         }
         const int ic = phys ? rm->src_sector : (int)oc;
@@ -1953,13 +2032,13 @@ Engine::HeffPlans* Engine::heff_plans(int node, int cls, bool adjoint) {
         c.add = 1; c.alpha = cst;
         s3.add_chunk(c);
       }
+      add_diagonal(oc);
       for (const HTerm& h : hts) {
         const bool phys = h.op[0].kind == 2 || h.op[1].kind == 2;
         const RowMap* rm = nullptr;
         if (phys) {
-          if (h.op[0].kind == 2 && h.op[0].term < 0) rm = &site_ham_map(node, 0, h.op[0].cls)[oc];
-          else if (h.op[1].kind == 2 && h.op[1].term < 0) rm = &site_ham_map(node, 1, h.op[1].cls)[oc];
-          else rm = &rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term)[oc];
+          if (in_diagonal(h)) continue;
+          rm = &rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term)[oc];
           if (rm->src_sector < 0) continue;
         }
         const int ic = phys ? rm->src_sector : (int)oc;
@@ -2080,10 +2159,8 @@ int Engine::apply_heff(const double* x, double* y, int cls) {
   const long long n = layout_[center_].size;
   const bool bottom = nodes_[center_].child_kind[0] == 0;
   if (use_mixed_ && cls < 0 && bottom) {
-    if (x != x_in_) launch_copy(x, x_in_, n, stream_);
-    int rc = apply_heff_mixed();
+    int rc = apply_heff_mixed(x, y);
     if (rc) return rc;
-    if (y != y_out_) launch_copy(y_out_, y, n, stream_);
     return check(cudaGetLastError(), "apply_heff (mixed)") ? 0 : -3;
   }
   if (use_mixed_ && cls < 0) {
@@ -2193,6 +2270,74 @@ int Engine::gradient_step(double eta, double* e_before, double* e_after) {
 }
 
 // ------------------------------------------------------------------ mixed precision
+// Tiles of one output sector.  A term reaches a row (a, b) only where its site
+// operators have a source for a and for b, so the rows are ordered by the sets
+// of terms that a and b allow (equal sets together, rows in their own order
+// inside), and each tile of 128 lists the terms that reach one of its rows.
+// At a corner pair of 4x4x4 that is 15 terms of 35 a tile on average; sites
+// with more links inside the lattice have more sets, smaller groups and a
+// smaller gain.  ops[i]: site operators of chunk i.
+void Engine::tc_tiles(int node, int oc, const std::vector<TcChunk>& sector_chunks,
+                      const std::vector<std::pair<const SiteOp*, const SiteOp*>>& ops, TcPlan* tc) {
+  const Layout& L = layout_[node];
+  const int rows = L.sec_rows[oc], words = (int)(sector_chunks.size() + 63) / 64 + 1;
+  using Set = std::vector<uint64_t>;
+  // per site and basis row: the set of terms it allows, and the set's class
+  std::vector<Set> allow[2];
+  std::vector<int> cls[2];
+  int n_cls[2];
+  for (int leg = 0; leg < 2; ++leg) {
+    allow[leg].assign(kLocalDim, Set(words, 0));
+    std::map<Set, int> ids;
+    for (int r = 0; r < kLocalDim; ++r) {
+      for (size_t i = 0; i < ops.size(); ++i) {
+        const SiteOp* op = leg == 0 ? ops[i].first : ops[i].second;
+        if (!op || (op->src[r] >= 0 && op->val[r] != 0.0)) allow[leg][r][i / 64] |= 1ull << (i % 64);
+      }
+      ids.emplace(allow[leg][r], 0);
+    }
+    n_cls[leg] = 0;
+    for (auto& kv : ids) kv.second = n_cls[leg]++;
+    for (int r = 0; r < kLocalDim; ++r) cls[leg].push_back(ids[allow[leg][r]]);
+  }
+  // counting sort of the sector's rows by (left class, right class)
+  std::vector<int> ra(rows), rb(rows), start((size_t)n_cls[0] * n_cls[1] + 1, 0);
+  for (const Layout::Blk& b : L.blk) {
+    if (b.ic != oc) continue;
+    const int a0 = L.leg[0].offset(b.ia), b0 = L.leg[1].offset(b.ib);
+    for (int i = 0; i < b.da; ++i)
+      for (int j = 0; j < b.db; ++j) {
+        const int r = b.row0 + i * b.db + j;
+        ra[r] = a0 + i;
+        rb[r] = b0 + j;
+        ++start[(size_t)cls[0][a0 + i] * n_cls[1] + cls[1][b0 + j] + 1];
+      }
+  }
+  for (size_t i = 1; i < start.size(); ++i) start[i] += start[i - 1];
+  const size_t base = tc->order.size();
+  tc->order.resize(base + rows);
+  for (int r = 0; r < rows; ++r) tc->order[base + start[(size_t)cls[0][ra[r]] * n_cls[1] + cls[1][rb[r]]]++] = r;
+  Set last;
+  int begin = 0, end = 0;
+  for (int r0 = 0; r0 < rows; r0 += 128) {
+    Set any(words, 0);
+    for (int i = r0; i < std::min(rows, r0 + 128); ++i) {
+      const int r = tc->order[base + i];
+      for (int w = 0; w < words; ++w) any[w] |= allow[0][ra[r]][w] & allow[1][rb[r]][w];
+    }
+    if (any != last || r0 == 0) {
+      begin = (int)tc->chunks.size();
+      for (size_t i = 0; i < sector_chunks.size(); ++i)
+        if (any[i / 64] >> (i % 64) & 1) tc->chunks.push_back(sector_chunks[i]);
+      end = (int)tc->chunks.size();
+      last = any;
+    }
+    tc->tiles.push_back(TcTile{(int)tc->outs.size() - 1, r0, begin, end});
+    for (int c = begin; c < end; ++c)
+      tc->flops_exec += 2.0 * 128 * tc->outs.back().npad * tc->chunks[c].kpad * (precision_ == PREC_TF32X3 ? 3 : 1);
+  }
+}
+
 // Tensor-core plan of a bottom node: environment-coupled terms (and the
 // environment block Hamiltonian) become GEMM chunks with their operator
 // blocks converted to BF16 / FP32 and scaled by the term coefficient; terms
@@ -2208,8 +2353,6 @@ TcPlan* Engine::tc_plan(int node) {
   const int d2 = P.total();
   const int elem = precision_ == PREC_BF16 ? 2 : 4;
   const bool split = precision_ == PREC_TF32X3;
-  const int xmul = split ? 2 : 1;   // staged row width in units of kpad
-  const int kmul = split ? 2 : 1;   // staged B row width in units of kpad
   std::unique_ptr<TcPlan> tp(new TcPlan);
   TcPlan& tc = *tp;
   std::vector<long long> soff(ns, 0);
@@ -2220,14 +2363,16 @@ TcPlan* Engine::tc_plan(int node) {
     soff[i] = xs;
     xs += (long long)L.sec_rows[i] * kpad[i];
   }
-  // operand staging holds xmul * xs elements; an FP32 copy (xs) serves the epilogue
-  if (xs > xstage_elems_) {
+  // FP32 rows serve as TF32 operands and the epilogue's adds; BF16 rows beside them
+  if (xs > xstage_elems_ || (elem == 2 && !xstage_)) {
     clear_tc_cache();   // cached plans point into the old staging
-    if (xstage_) { untrack(xstage_); cudaFree(xstage_); }
+    if (xstage_) { untrack(xstage_); cudaFree(xstage_); xstage_ = nullptr; }
     if (xstage32_) { untrack(xstage32_); cudaFree(xstage32_); xstage32_ = nullptr; }
-    xstage_elems_ = xs + xs / 4;
-    if (!check(cudaMalloc(&xstage_, 2 * xstage_elems_ * elem), "x staging")) return nullptr;
-    track(xstage_, 2 * xstage_elems_ * elem);
+    xstage_elems_ = std::max(xstage_elems_, xs + xs / 4);
+    if (elem == 2) {
+      if (!check(cudaMalloc(&xstage_, xstage_elems_ * 2), "x staging")) return nullptr;
+      track(xstage_, xstage_elems_ * 2);
+    }
     if (!check(cudaMalloc(&xstage32_, xstage_elems_ * 4), "x staging")) return nullptr;
     track(xstage32_, xstage_elems_ * 4);
   }
@@ -2237,13 +2382,11 @@ TcPlan* Engine::tc_plan(int node) {
     ConvJob j;
     j.src = x_in_ + L.sec_off[i];
     j.ld_src = P.dim[i];
-    j.cs_src = 1;
-    j.dst = (char*)xstage_ + xmul * soff[i] * elem;
+    j.dst = elem == 2 ? (char*)xstage_ + soff[i] * 2 : nullptr;
     j.dst32 = xstage32_ + soff[i];
     j.rows = L.sec_rows[i];
     j.cols = P.dim[i];
     j.kpad = kpad[i];
-    j.scale = 1.0;
     tc.xjobs.push_back(j);
     tc.x_max_elems = std::max(tc.x_max_elems, (long long)j.rows * j.kpad);
   }
@@ -2260,7 +2403,10 @@ TcPlan* Engine::tc_plan(int node) {
     o.rows = rows;
     o.n = P.dim[oc];
     o.npad = kpad[oc];
-    o.chunk_begin = (int)tc.chunks.size();
+    o.div = (unsigned)(((1ull << 32) + o.n - 1) / o.n);
+    o.order = (const int*)(intptr_t)tc.order.size();   // patched below once uploaded
+    std::vector<TcChunk> sector_chunks;
+    std::vector<std::pair<const SiteOp*, const SiteOp*>> sector_ops;   // its two site operators (null: identity)
     o.add_begin = (int)tc.adds.size();
     tc.max_npad = std::max(tc.max_npad, o.npad);
     if (cst != 0.0) {
@@ -2272,13 +2418,25 @@ TcPlan* Engine::tc_plan(int node) {
       a.ld = kpad[oc];
       tc.adds.push_back(a);
     }
+    const RowMap& diag = diagonal_map(node, -1)[oc];
+    if (diag.src_sector >= 0) {
+      TcAdd a;
+      a.X32 = x32 + soff[oc];
+      a.map = nullptr;
+      a.val = diag.val;
+      a.alpha = 1.0;
+      a.ld = kpad[oc];
+      tc.adds.push_back(a);
+    }
     for (const HTerm& h : hts) {
       const bool phys = h.op[0].kind == 2 || h.op[1].kind == 2;
       const RowMap* rm = nullptr;
       if (phys) {
-        if (h.op[0].kind == 2 && h.op[0].term < 0) rm = &site_ham_map(node, 0, h.op[0].cls)[oc];
-        else if (h.op[1].kind == 2 && h.op[1].term < 0) rm = &site_ham_map(node, 1, h.op[1].cls)[oc];
-        else rm = &rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term)[oc];
+        const std::vector<RowMap>& maps = h.op[0].kind == 2 && h.op[0].term < 0   ? site_ham_map(node, 0, h.op[0].cls)
+                                          : h.op[1].kind == 2 && h.op[1].term < 0 ? site_ham_map(node, 1, h.op[1].cls)
+                                                                                  : rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term);
+        if (bottom_diagonal(node, h)) continue;
+        rm = &maps[oc];
         if (rm->src_sector < 0) continue;
       }
       const int ic = phys ? rm->src_sector : oc;
@@ -2289,19 +2447,24 @@ TcPlan* Engine::tc_plan(int node) {
           return nullptr;
         }
         TcChunk c;
-        c.X = (char*)xstage_ + xmul * soff[ic] * elem;
+        c.X = elem == 2 ? (const void*)((char*)xstage_ + soff[ic] * 2) : (const void*)(xstage32_ + soff[ic]);
         c.map = rm ? rm->map : nullptr;
-        c.kpad = kmul * kpad[ic];
-        c.xstride = xmul * kpad[ic];
-        const long long welems = (long long)o.npad * c.kpad;
+        c.kpad = kpad[ic];
+        c.xstride = kpad[ic];
+        const long long welems = (long long)o.npad * c.kpad * (split ? 2 : 1);
         wj.push_back({oc, ic, h.op[2].ptr, h.coef, wtot});
         c.W = (const void*)(intptr_t)wtot;   // patched below once the buffer exists
         wtot += welems;
-        tc.chunks.push_back(c);
+        std::pair<const SiteOp*, const SiteOp*> ops{nullptr, nullptr};
+        if (rm)
+          for (auto& so : terms_[h.op[0].kind == 2 ? h.op[0].term : h.op[1].term].ops)
+            if (so.first == leg_site(node, 0) || so.first == leg_site(node, 1))
+              (so.first == leg_site(node, 0) ? ops.first : ops.second) = site_op(lat_.parity(so.first), so.second);
+        sector_chunks.push_back(c);
+        sector_ops.push_back(ops);
         tc.max_kpad = std::max(tc.max_kpad, c.kpad);
         const double nnz = rm ? (double)rm->nnz : (double)rows;
         tc.flops_alg += 2.0 * nnz * P.dim[oc] * P.dim[ic];
-        tc.flops_exec += 2.0 * ((rows + 127) / 128 * 128) * o.npad * kpad[ic] * (split ? 3 : 1);
       } else {
         if (ic != oc) continue;
         TcAdd a;
@@ -2313,36 +2476,39 @@ TcPlan* Engine::tc_plan(int node) {
         tc.adds.push_back(a);
       }
     }
-    o.chunk_end = (int)tc.chunks.size();
     o.add_end = (int)tc.adds.size();
     tc.outs.push_back(o);
-    for (int r0 = 0; r0 < rows; r0 += 128) tc.tiles.push_back({(int)tc.outs.size() - 1, r0});
+    tc_tiles(node, oc, sector_chunks, sector_ops, &tc);
   }
-  if (wtot > wbuf_elems_) {
+  if (wtot * elem > wbuf_bytes_) {
     clear_tc_cache();   // cached plans point into the old W buffer
     if (wbuf_) { untrack(wbuf_); cudaFree(wbuf_); }
-    wbuf_elems_ = wtot + wtot / 4 + 1024;
-    if (!check(cudaMalloc(&wbuf_, wbuf_elems_ * elem), "W staging")) return nullptr;
-    track(wbuf_, wbuf_elems_ * elem);
+    wbuf_bytes_ = (wtot + wtot / 4 + 1024) * elem;
+    if (!check(cudaMalloc(&wbuf_, wbuf_bytes_), "W staging")) return nullptr;
+    track(wbuf_, wbuf_bytes_);
   }
   for (TcChunk& c : tc.chunks) c.W = (char*)wbuf_ + (intptr_t)c.W * elem;
   tc.wtot = wtot;
   for (const WJ& w : wj) {
-    ConvJob j;
+    WJob j;
     j.src = w.op + P.offset(w.oc) * (long long)d2 + P.offset(w.ic);
     j.ld_src = d2;
-    j.cs_src = 1;
     j.dst = (char*)wbuf_ + w.off * elem;
-    j.dst32 = nullptr;
     j.rows = P.dim[w.oc];
     j.cols = P.dim[w.ic];
+    j.npad = kpad[w.oc];
     j.kpad = kpad[w.ic];
     j.scale = w.coef;
     tc.wjobs.push_back(j);
-    tc.w_max_elems = std::max(tc.w_max_elems, (long long)j.rows * j.kpad);
   }
   // algorithmic bytes: x staging read once, y written once (FP64), W read once
-  tc.bytes_alg = (double)xs * xmul * elem + (double)L.size * 8.0 + (double)wtot * elem;
+  tc.bytes_alg = (double)xs * elem + (double)L.size * 8.0 + (double)wtot * elem;
+  // longest tiles first: the last ones to start then end soon
+  std::stable_sort(tc.tiles.begin(), tc.tiles.end(), [](const TcTile& x, const TcTile& y) {
+    return x.chunk_end - x.chunk_begin > y.chunk_end - y.chunk_begin;
+  });
+  grow_upload(tc.d_order, tc.cap[6], tc.order, stream_);
+  for (TcOutput& o : tc.outs) o.order = tc.d_order + (intptr_t)o.order;
   grow_upload(tc.d_tiles, tc.cap[0], tc.tiles, stream_);
   grow_upload(tc.d_outs, tc.cap[1], tc.outs, stream_);
   grow_upload(tc.d_chunks, tc.cap[2], tc.chunks, stream_);
@@ -2370,23 +2536,22 @@ TcPlan* Engine::tc_prepare() {
   const int split = precision_ == PREC_TF32X3 ? 1 : 0;
   if (tc_w_node_ != center_) {
     // environment blocks of this centre (padding zero) into the shared W buffer
-    if (tc->wtot > 0) cudaMemsetAsync(wbuf_, 0, tc->wtot * elem, stream_);
-    launch_convert(elem, split ? 2 : 0, tc->d_wjobs, (int)tc->wjobs.size(), tc->w_max_elems, stream_);
+    launch_stage_w(elem, split, tc->d_wjobs, (int)tc->wjobs.size(), stream_);
     tc_w_node_ = center_;
   }
   return tc;
 }
 
-int Engine::apply_heff_mixed() {
+int Engine::apply_heff_mixed(const double* x, double* y) {
   TcPlan* tc = tc_prepare();
   if (!tc) return -1;
   const int elem = precision_ == PREC_BF16 ? 2 : 4;
   const int split = precision_ == PREC_TF32X3 ? 1 : 0;
-  launch_convert(elem, split, tc->d_xjobs, (int)tc->xjobs.size(), tc->x_max_elems, stream_);
+  launch_convert(elem, tc->d_xjobs, (int)tc->xjobs.size(), tc->x_max_elems, x - x_in_, stream_);
   cudaEvent_t e0 = nullptr;
   if (profiling_) ev_begin(&e0);
   int rc = launch_tc_heff(elem, split, tc->d_tiles, (int)tc->tiles.size(), tc->d_outs, tc->d_chunks, tc->d_adds,
-                          tc->max_kpad, tc->max_npad, d_err_, stream_, wait_polls);
+                          tc->max_kpad, tc->max_npad, y - y_out_, d_err_, stream_, wait_polls);
   if (rc) {
     err_ = "tensor-core H_eff: tile shape outside the supported range";
     return rc;

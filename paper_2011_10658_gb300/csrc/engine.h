@@ -175,21 +175,24 @@ struct TcPlan {
   std::vector<TcOutput> outs;
   std::vector<TcChunk> chunks;
   std::vector<TcAdd> adds;
-  std::vector<ConvJob> xjobs, wjobs;
+  std::vector<int> order;        // row orders of the outputs, one after another
+  std::vector<ConvJob> xjobs;
+  std::vector<WJob> wjobs;
   TcTile* d_tiles = nullptr;
   TcOutput* d_outs = nullptr;
   TcChunk* d_chunks = nullptr;
   TcAdd* d_adds = nullptr;
+  int* d_order = nullptr;
   ConvJob* d_xjobs = nullptr;
-  ConvJob* d_wjobs = nullptr;
-  size_t cap[6] = {0, 0, 0, 0, 0, 0};
-  long long x_max_elems = 0, w_max_elems = 0;
+  WJob* d_wjobs = nullptr;
+  size_t cap[7] = {0, 0, 0, 0, 0, 0, 0};
+  long long x_max_elems = 0;
   int max_kpad = 16, max_npad = 16;
   double flops_alg = 0, flops_exec = 0, bytes_alg = 0;
   long long wtot = 0;            // elements of the W buffer this plan uses
   void clear() {
-    tiles.clear(); outs.clear(); chunks.clear(); adds.clear(); xjobs.clear(); wjobs.clear();
-    x_max_elems = w_max_elems = wtot = 0; max_kpad = max_npad = 16; flops_alg = flops_exec = bytes_alg = 0;
+    tiles.clear(); outs.clear(); chunks.clear(); adds.clear(); order.clear(); xjobs.clear(); wjobs.clear();
+    x_max_elems = wtot = 0; max_kpad = max_npad = 16; flops_alg = flops_exec = bytes_alg = 0;
   }
   void release();
   ~TcPlan() { release(); }
@@ -438,11 +441,11 @@ class Engine {
   int apply_heff_tg();
   int tc_w_node_ = -1;          // node whose environment blocks are staged
   void clear_tc_cache();
-  void* xstage_ = nullptr;      // BF16 or FP32 padded staging of x
-  float* xstage32_ = nullptr;   // FP32 padded staging (BF16 path)
+  void* xstage_ = nullptr;      // BF16 padded staging of x (BF16 operands)
+  float* xstage32_ = nullptr;   // FP32 padded staging of x
   long long xstage_elems_ = 0;
   void* wbuf_ = nullptr;
-  long long wbuf_elems_ = 0;
+  long long wbuf_bytes_ = 0;
   int* d_err_ = nullptr;
   bool profiling_ = false;
   struct EvRec { cudaEvent_t a, b; int cls; double fa, fe, ba; };
@@ -453,10 +456,12 @@ class Engine {
   void ev_begin(cudaEvent_t* e);
   void ev_end(cudaEvent_t a, int cls, double fa, double fe, double ba);
   TcPlan* tc_plan(int node);
+  void tc_tiles(int node, int oc, const std::vector<TcChunk>& sector_chunks,
+                const std::vector<std::pair<const SiteOp*, const SiteOp*>>& ops, TcPlan* tc);
   TcPlan* tc_prepare();
   // bumped whenever cached plans are dropped (their device pointers go stale)
   uint64_t gen_ = 0;
-  int apply_heff_mixed();
+  int apply_heff_mixed(const double* x, double* y);
   bool mixed_node(int node) const;
   // Lanczos workspace
   double* V_ = nullptr;
@@ -504,6 +509,9 @@ class Engine {
   const std::vector<RowMap>& rowmap(int node, int term);
   RowMap build_rowmap_sector(int node, const SiteOp* A, const SiteOp* B, int out_sector, const std::vector<double>* vals);
   const std::vector<RowMap>& site_ham_map(int node, int leg, int cls);
+  bool local_diagonal(int node, int term);
+  bool bottom_diagonal(int node, const HTerm& h);
+  const std::vector<RowMap>& diagonal_map(int node, int cls);
   void build_heff_terms(int node, int cls_filter, std::vector<HTerm>* out);
   int run_plan(KPlan& pl);
   void plan_leg_apply(KPlan& pl, const Layout& LX, const double* X, const Layout& LY, double* Y, int leg,

@@ -205,8 +205,8 @@ namespace qed {
 struct TcChunk {
   const void* X;      // staging source sector matrix (BF16 or FP32), row stride xstride
   const int* map;     // sign-encoded row map (nullable: identity)
-  const void* W;      // npad x kpad K-major B operand (alpha folded in)
-  int kpad;           // K of the staged rows, multiple of 16 (split: [hi | lo], 2 x part)
+  const void* W;      // B operand in core-matrix order (alpha folded in; split: [hi | lo])
+  int kpad;           // K of the staged rows, multiple of 16
   int xstride;        // elements per staged source row
 };
 struct TcAdd {
@@ -218,34 +218,46 @@ struct TcAdd {
 };
 struct TcOutput {
   double* y;
+  const int* order;   // row of the sector that row i of the tiles' order is
   int rows, n, npad;
-  int chunk_begin, chunk_end;
   int add_begin, add_end;
+  unsigned div;       // ceil(2^32 / n)
 };
+// 128 rows of an output, and the chunks that reach one of them.
 struct TcTile {
   int out;
   int row0;
+  int chunk_begin, chunk_end;
 };
-// One conversion job: dst (rows x kpad, zero padded) <- scale * src (rows x cols, ld_src), FP64 source.
+// Staging of x: dst32 (and, for BF16 operands, dst), rows x kpad, zero padded,
+// <- src (rows x cols, ld_src), FP64 source.
 struct ConvJob {
   const double* src;
   long long ld_src;   // row stride of the source
-  long long cs_src;   // column stride of the source
-  void* dst;          // BF16 or FP32
-  float* dst32;       // optional second FP32 copy (same padded layout)
+  void* dst;          // BF16 copy (BF16 operands only)
+  float* dst32;       // FP32 copy
   int rows, cols, kpad;
+};
+// Staging of one environment block: dst (npad x kpad, core-matrix order) <-
+// scale * src (rows x cols, ld_src).
+struct WJob {
+  const double* src;
+  long long ld_src;
+  void* dst;
+  int rows, cols, npad, kpad;
   double scale;
 };
 
 // elem: 2 = BF16 operands (kind::f16), 4 = TF32 operands (kind::tf32).
-// split (TF32 only): A rows staged as [x_hi | x_lo] and B rows as [W_hi |
-// W_lo]; three sub-products x_hi W_hi + x_hi W_lo + x_lo W_hi whose sum
-// carries about 21 bits (x_lo W_lo dropped).
+// split (TF32 only): both operands as hi + lo TF32 parts; three sub-products
+// x_hi W_hi + x_hi W_lo + x_lo W_hi whose sum carries about 21 bits (x_lo W_lo
+// dropped).  y_shift: added to every output pointer (elements), so that one
+// plan serves any y.
 // err: device flag set to 1 if a wait timed out (results then invalid).
 // polls: bound of each mbarrier wait in polls (< 0: the default, 2^22).
 int launch_tc_heff(int elem, int split, const TcTile* tiles, int n_tiles, const TcOutput* outs,
-                   const TcChunk* chunks, const TcAdd* adds, int max_kpad, int max_npad, int* err, cudaStream_t s,
-                   long long polls = -1);
+                   const TcChunk* chunks, const TcAdd* adds, int max_kpad, int max_npad, long long y_shift, int* err,
+                   cudaStream_t s, long long polls = -1);
 // ---- grouped leg contractions on the tensor cores (tcgen05) ----
 // One contribution D[r, j] += alpha * sum_{k < K} A(r, k) B(j, k):
 //   A(r, k) = A[(r / R2) * s1 + (r % R2) * s2 + k * sk]  (float if a_f32, else double)
@@ -336,9 +348,8 @@ struct OzOut {
 int launch_oz_gram(const OzTile* tiles, int n_tiles, const OzJob* jobs, const void* planes, int npad, double* partial,
                    const OzOut* outs, int n_outs, const OzSum* sums, int* err, cudaStream_t s, long long polls = -1);
 
-// mode 0: plain (BF16 or FP32 by elem); mode 1: split x rows [hi | lo] of
-// width 2 kpad; mode 2: split W rows [hi | lo] of width 2 kpad.  hi is
-// the value with its 13 low mantissa bits cleared (what the TF32 units read).
-void launch_convert(int elem, int mode, const ConvJob* jobs, int n_jobs, long long max_elems, cudaStream_t s);
+// Staging for launch_tc_heff; shift: added to every source pointer (elements).
+void launch_convert(int elem, const ConvJob* jobs, int n_jobs, long long max_elems, long long shift, cudaStream_t s);
+void launch_stage_w(int elem, int split, const WJob* jobs, int n_jobs, cudaStream_t s);
 
 }  // namespace qed

@@ -1,36 +1,60 @@
 // Mixed-precision H_eff x for bottom TTN nodes on the sm_103a tensor cores.
 //
-// y[r, :] = sum_chunks s_c(r) X_c[map_c(r), :] W_c^T  +  sum_adds alpha val(r) X32[map(r), :]
+// y[r, :] = sum_chunks s_c(r) X[map_c(r), :] W_c^T  +  sum_adds alpha val(r) X[map(r), :]
 //
 // The physical legs of a bottom node carry monomial site operators
 // (Eq. (15) and the plaquette factors: at most one +-1 per row), so each
 // product term becomes a row gather of the node tensor followed by one
 // dense contraction with the environment operator on the parent leg.  The
-// gather feeds the A operand of tcgen05.mma directly: every thread copies
-// one gathered row into the no-swizzle K-major shared-memory layout (8-row
-// x 16-byte core matrices), the environment block is the B operand, and
-// all product terms of an output tile accumulate in one TMEM accumulator.
-// Terms without an environment factor (site energies, the internal link of
-// the pair, the constant) are added in FP64 in the epilogue.
+// gather feeds the A operand of tcgen05.mma (no-swizzle K-major core matrices
+// of 8 rows x 16 bytes), the environment block is the B operand, and all
+// product terms of an output tile accumulate in one TMEM accumulator.  Terms
+// without an environment factor (the diagonal of the two sites, the internal
+// hopping) are added in float-float arithmetic when the tile is written.
 //
-// One CTA = one 128-row tile of one output charge sector; 128 threads; two
-// shared-memory stages so the gather of term j+1 overlaps the MMAs of term
-// j.  Every mbarrier wait is bounded (polls, a launch argument); a timeout
-// sets *err, and the CTA then drains its MMAs through a commit to a fresh
-// barrier (waited on with the default bound, so the MMAs still in flight
-// finish before TMEM is read or freed), frees its TMEM and returns.
+// One CTA = one 128-row tile of one output charge sector.  The rows of a
+// sector are ordered by the terms that reach them, so a tile walks only some
+// of the terms (Engine::tc_tiles).  Eight gather warps feed two stages of A,
+// one thread of a ninth warp copies the blocks of W (staged in core-matrix
+// order, bulk copies two terms ahead) and issues the MMAs; they meet on
+// mbarriers only.  x is staged once per product as FP32 (and BF16) rows; the
+// hi and lo TF32 parts of a split product are cut from the FP32 row on its way
+// to shared memory, so a gather moves 4 bytes per entry.  A warp's load takes
+// 8 rows x 64 bytes: eight cache lines instead of one per lane, and stores
+// that fill all banks.  The rows of term j + 1 and the map of term j + 2 are
+// read while term j waits for its stage; rows two terms ahead in registers
+// measured the same.
+//
+// Bound by the round trip gather -> MMA -> free stage of each term (two CTAs
+// an SM for split TF32).  Product at bottom node 0 of 4x4x4, whole call, GB300:
+// chi=64 split TF32 287 -> 108 us, chi=48 BF16 132 -> 77 us.  On the way: FP64
+// arithmetic out of the epilogue and the staging (two operations per clock and
+// SM; 40 % of the kernel) and coalesced gathers 203 us; gather and issue on
+// separate warps, 16-byte pieces at compile-time places 132 us; rows ordered
+// by their terms 108 us.
+//
+// Every mbarrier wait is bounded (polls, a launch argument); a timeout sets
+// *err, and the CTA then drains its MMAs through a commit to a fresh barrier
+// and its bulk copies through their own barriers (waited on with the default
+// bound, so that nothing is in flight when TMEM is freed), and returns.
 #include <algorithm>
 #include <cuda_bf16.h>
 
 #include <cstdio>
 
+#include "ffloat.cuh"
 #include "kernels.cuh"
 
 namespace qed {
 
 namespace {
 
-constexpr int TC_THREADS = 128;
+constexpr int TC_GATHER_WARPS = 8;
+constexpr int TC_THREADS = 32 * (TC_GATHER_WARPS + 1);   // and the warp that issues copies and MMAs
+constexpr int TC_WARP_ROWS = 16;                  // rows of A a warp gathers
+constexpr int TC_ADDS = 8;                        // terms without environment factor whose row factors are held
+constexpr int TC_UNROLL = 4;                      // outputs a thread writes at a time
+constexpr int TC_PRE = 6;                         // 16-byte pieces of a chunk a thread holds
 constexpr long long kWaitPolls = 1LL << 22;   // default bound of one mbarrier wait
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -61,9 +85,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, long l
         : "r"(addr), "r"(parity)
         : "memory");
     if (done) return true;
-    __nanosleep(32);
+    if (it > 32) __nanosleep(32);
   }
   return false;
+}
+
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar));
 }
 
 template <int ELEM>
@@ -78,21 +106,96 @@ __device__ __forceinline__ void mma(uint32_t tmem, uint64_t ad, uint64_t bd, uin
         "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
 }
 
+__device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
+
+// One thread's share of a chunk's A tile: KQ / 2 pieces of 16 bytes.  Piece `it`
+// is piece q of row r of the warp's 16 rows, the eight rows of a core matrix on
+// neighbouring lanes.  mp: lane l holds the map entry of row l (mod 16).
+template <int KQ>
+struct Gather {
+  static constexpr int N = KQ / 2;
+  static __device__ __forceinline__ int group(int it, int lane) { return it * 4 + (lane >> 3) >= KQ ? 1 : 0; }
+  static __device__ __forceinline__ int piece(int it, int lane) { return it * 4 + (lane >> 3) - group(it, lane) * KQ; }
+  template <int ELEM>
+  static __device__ __forceinline__ void load(uint4* v, const void* X, int row_bytes, int mp, int lane) {
+    const int s0 = __shfl_sync(0xffffffffu, mp, lane & 7), s1 = __shfl_sync(0xffffffffu, mp, 8 + (lane & 7));
+    const uint8_t* x0 = (const uint8_t*)X + (long long)(s0 >> 1) * row_bytes;
+    const uint8_t* x1 = (const uint8_t*)X + (long long)(s1 >> 1) * row_bytes;
+#pragma unroll
+    for (int it = 0; it < N; ++it) {
+      const bool g = group(it, lane);
+      v[it] = make_uint4(0u, 0u, 0u, 0u);
+      if ((g ? s1 : s0) >= 0) v[it] = __ldg((const uint4*)((g ? x1 : x0) + piece(it, lane) * 16));
+    }
+#pragma unroll
+    for (int it = 0; it < N; ++it) {
+      const int s = group(it, lane) ? s1 : s0;
+      const uint32_t flip = s < 0 ? 0u : (ELEM == 2 ? (uint32_t)(s & 1) * 0x80008000u : (uint32_t)s << 31);
+      v[it].x ^= flip; v[it].y ^= flip; v[it].z ^= flip; v[it].w ^= flip;
+    }
+  }
+  template <bool SPLIT>
+  static __device__ __forceinline__ void store(uint8_t* A, const uint4* v, int warp, int lane) {
+    constexpr int KCH = SPLIT ? 2 * KQ : KQ;
+#pragma unroll
+    for (int it = 0; it < N; ++it) {
+      uint8_t* d = A + ((warp * 2 + group(it, lane)) * KCH + piece(it, lane)) * 128 + (lane & 7) * 16;
+      if (SPLIT) {
+        const float4 x = make_float4(__uint_as_float(v[it].x), __uint_as_float(v[it].y), __uint_as_float(v[it].z),
+                                     __uint_as_float(v[it].w));
+        const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+        *(float4*)d = h;
+        *(float4*)(d + KQ * 128) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+      } else {
+        *(uint4*)d = v[it];
+      }
+    }
+  }
+};
+
+// The same for a width without a specialisation: straight to shared memory.
 template <int ELEM, bool SPLIT>
-__global__ void __launch_bounds__(TC_THREADS) tc_heff_kernel(const TcTile* __restrict__ tiles,
-                                                              const TcOutput* __restrict__ outs,
-                                                              const TcChunk* __restrict__ chunks,
-                                                              const TcAdd* __restrict__ adds, int a_bytes,
-                                                              int b_bytes, int* err, long long polls) {
+__device__ __noinline__ void gather_any(uint8_t* A, const void* X, int row_bytes, int kq, int mp, int warp, int lane) {
+  for (int it = 0; it < kq / 2; ++it) {
+    const int rest = it * 4 + (lane >> 3), g = rest >= kq ? 1 : 0, q = rest - g * kq;
+    const int s = __shfl_sync(0xffffffffu, mp, g * 8 + (lane & 7));
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (s >= 0) {
+      v = __ldg((const uint4*)((const uint8_t*)X + (long long)(s >> 1) * row_bytes + q * 16));
+      const uint32_t flip = ELEM == 2 ? (uint32_t)(s & 1) * 0x80008000u : (uint32_t)s << 31;
+      v.x ^= flip; v.y ^= flip; v.z ^= flip; v.w ^= flip;
+    }
+    uint8_t* d = A + ((warp * 2 + g) * (SPLIT ? 2 : 1) * kq + q) * 128 + (lane & 7) * 16;
+    if (SPLIT) {
+      const float4 x = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+      const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+      *(float4*)d = h;
+      *(float4*)(d + kq * 128) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+    } else {
+      *(uint4*)d = v;
+    }
+  }
+}
+
+template <int ELEM, bool SPLIT>
+__global__ void __launch_bounds__(TC_THREADS, SPLIT ? 2 : 3) tc_heff_kernel(const TcTile* __restrict__ tiles,
+                                                                             const TcOutput* __restrict__ outs,
+                                                                             const TcChunk* __restrict__ chunks,
+                                                                             const TcAdd* __restrict__ adds,
+                                                                             int a_bytes, int b_bytes, int b_stages,
+                                                                             long long y_shift, int* err,
+                                                                             long long polls) {
+  constexpr int PARTS = SPLIT ? 2 : 1;
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ uint32_t tmem_slot;
-  __shared__ __align__(8) uint64_t mbar[3];   // two stages, one drain
+  // MMAs of the two A stages, drain, the gathers of the two A stages, the
+  // copies of up to four B stages
+  __shared__ __align__(8) uint64_t mbar[9];
   __shared__ int s_fail;
   const TcTile tile = tiles[blockIdx.x];
   const TcOutput out = outs[tile.out];
-  const int tid = threadIdx.x, warp = tid >> 5;
-  uint8_t* Abuf[2] = {smem, smem + a_bytes};
-  uint8_t* Bbuf[2] = {smem + 2 * a_bytes, smem + 2 * a_bytes + b_bytes};
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint8_t* const B0 = smem + 2 * a_bytes;
   uint32_t ncols = 32;
   while ((int)ncols < out.npad) ncols <<= 1;
   if (warp == 0) {
@@ -101,9 +204,8 @@ __global__ void __launch_bounds__(TC_THREADS) tc_heff_kernel(const TcTile* __res
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar[0])), "r"(1));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar[1])), "r"(1));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar[2])), "r"(1));
+    for (int i = 0; i < 9; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar[i])), "r"(i == 3 || i == 4 ? TC_GATHER_WARPS : 1));
     asm volatile("fence.mbarrier_init.release.cluster;");
     s_fail = 0;
   }
@@ -111,159 +213,258 @@ __global__ void __launch_bounds__(TC_THREADS) tc_heff_kernel(const TcTile* __res
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_slot;
-  const int row = tile.row0 + tid;
-  const bool row_ok = row < out.rows;
-  const int nchunks = out.chunk_end - out.chunk_begin;
-  // idesc: D = F32, A/B = BF16 (kind::f16) or TF32 (kind::tf32), both K-major, M = 128
-  uint32_t idesc = (1u << 4) | ((uint32_t)(out.npad >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-  idesc |= ELEM == 4 ? ((2u << 7) | (2u << 10)) : ((1u << 7) | (1u << 10));
+  const int nchunks = tile.chunk_end - tile.chunk_begin;
+  const TcChunk* const ch = chunks + tile.chunk_begin;
 
-  auto load_chunk = [&](int ci, int b) {
-    const TcChunk c = chunks[ci];
-    const int kchunks = c.kpad * ELEM / 16;   // split: [hi | lo] for both A and B
-    int src = -1;
-    if (row_ok) src = c.map ? c.map[row] : (row << 1);
-    const uint8_t* xrow = src >= 0 ? (const uint8_t*)c.X + (long long)(src >> 1) * c.xstride * ELEM : nullptr;
-    const uint32_t flip = (src >= 0 && (src & 1)) ? (ELEM == 2 ? 0x80008000u : 0x80000000u) : 0u;
-    for (int q = 0; q < kchunks; ++q) {
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (xrow) {
-        v = __ldg((const uint4*)(xrow + q * 16));
-        v.x ^= flip;
-        v.y ^= flip;
-        v.z ^= flip;
-        v.w ^= flip;
+  if (warp < TC_GATHER_WARPS) {
+    // gather warps: lanes l and l + 16 hold the map entry of row l of 16
+    const int at = tile.row0 + warp * TC_WARP_ROWS + (lane & 15);
+    const int row = at < out.rows ? __ldg(out.order + at) : -1;
+    auto map_entry = [&](const TcChunk& c) { return row >= 0 ? (c.map ? __ldg(c.map + row) : (row << 1)) : -1; };
+    uint4 pre[TC_PRE];
+    auto load = [&](const TcChunk& c, int mp) {
+      const int rb = c.xstride * ELEM;
+      switch (c.kpad * ELEM / 16) {
+        case 2: Gather<2>::load<ELEM>(pre, c.X, rb, mp, lane); break;
+        case 4: Gather<4>::load<ELEM>(pre, c.X, rb, mp, lane); break;
+        case 6: Gather<6>::load<ELEM>(pre, c.X, rb, mp, lane); break;
+        case 8: Gather<8>::load<ELEM>(pre, c.X, rb, mp, lane); break;
+        case 12: Gather<12>::load<ELEM>(pre, c.X, rb, mp, lane); break;
+        default: break;
       }
-      *(uint4*)(Abuf[b] + core_off(tid, q, kchunks)) = v;
-    }
-    const uint8_t* w = (const uint8_t*)c.W;
-    for (int e = tid; e < out.npad * kchunks; e += TC_THREADS) {
-      const int n = e / kchunks, q = e - n * kchunks;
-      *(uint4*)(Bbuf[b] + core_off(n, q, kchunks)) = __ldg((const uint4*)(w + ((long long)n * kchunks + q) * 16));
-    }
-  };
-
-  uint32_t uses[2] = {0u, 0u};
-  if (nchunks > 0) {
-    load_chunk(out.chunk_begin, 0);
-    asm volatile("fence.proxy.async.shared::cta;");
-    __syncthreads();
+    };
+    TcChunk c, cn, cnn;
+    int mp = -1, mp_next = -1;
+    if (nchunks > 0) { c = ch[0]; mp = map_entry(c); }
+    if (nchunks > 1) { cn = ch[1]; mp_next = map_entry(cn); }
+    if (nchunks > 2) cnn = ch[2];
+    if (nchunks > 0) load(c, mp);
     for (int j = 0; j < nchunks; ++j) {
       const int b = j & 1;
-      if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const int kchunks = chunks[out.chunk_begin + j].kpad * ELEM / 16;
-        const uint32_t a0 = smem_u32(Abuf[b]), b0 = smem_u32(Bbuf[b]);
-        const uint32_t sbo = (uint32_t)kchunks * 128u;
-        if (!SPLIT) {
-          for (int ks = 0; ks < kchunks / 2; ++ks) {
-            const uint64_t ad = smem_desc(a0 + ks * 256, 128, sbo);
-            const uint64_t bd = smem_desc(b0 + ks * 256, 128, sbo);
-            mma<ELEM>(tmem, ad, bd, idesc, (j > 0 || ks > 0) ? 1u : 0u);
-          }
-        } else {
-          // x_hi W_hi + x_hi W_lo + x_lo W_hi; A and B tiles hold [hi | lo]
-          const int part = kchunks / 2;
-          const int pa[3] = {0, 0, part}, pb[3] = {0, part, 0};
-          for (int g = 0; g < 3; ++g)
-            for (int ks = 0; ks < part / 2; ++ks) {
-              const uint64_t ad = smem_desc(a0 + (pa[g] + 2 * ks) * 128, 128, sbo);
-              const uint64_t bd = smem_desc(b0 + (pb[g] + 2 * ks) * 128, 128, sbo);
-              mma<ELEM>(tmem, ad, bd, idesc, (j > 0 || g > 0 || ks > 0) ? 1u : 0u);
-            }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(&mbar[b])));
+      uint8_t* const A = smem + b * a_bytes;
+      // the MMAs that read this A stage (chunk j - 2) are done
+      const bool free = j < 2 || mbar_wait(smem_u32(&mbar[b]), (uint32_t)((j >> 1) - 1) & 1u, polls);
+      if (!__all_sync(0xffffffffu, free)) {
+        s_fail = 1;
+        break;
       }
-      uses[b] += 1;
-      if (j + 1 < nchunks) {
-        const int nb = b ^ 1;
-        if (uses[nb] > 0 && !mbar_wait(smem_u32(&mbar[nb]), (uses[nb] - 1) & 1, polls)) s_fail = 1;
-        load_chunk(out.chunk_begin + j + 1, nb);
-        asm volatile("fence.proxy.async.shared::cta;");
-        __syncthreads();
+      switch (c.kpad * ELEM / 16) {
+        case 2: Gather<2>::store<SPLIT>(A, pre, warp, lane); break;
+        case 4: Gather<4>::store<SPLIT>(A, pre, warp, lane); break;
+        case 6: Gather<6>::store<SPLIT>(A, pre, warp, lane); break;
+        case 8: Gather<8>::store<SPLIT>(A, pre, warp, lane); break;
+        case 12: Gather<12>::store<SPLIT>(A, pre, warp, lane); break;
+        default: gather_any<ELEM, SPLIT>(A, c.X, c.xstride * ELEM, c.kpad * ELEM / 16, mp, warp, lane); break;
       }
+      asm volatile("fence.proxy.async.shared::cta;");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&mbar[3 + b])) : "memory");
+      // rows of the next chunk, map of the one after, description of the third
+      c = cn;
+      mp = mp_next;
+      if (j + 1 < nchunks) load(c, mp);
+      cn = cnn;
+      if (j + 2 < nchunks) mp_next = map_entry(cn);
+      if (j + 3 < nchunks) cnn = ch[j + 3];
     }
-    // drain: one more commit from the issuing thread arrives on mbar[2] once
-    // every MMA it issued has completed (whatever happened to the stage
-    // barriers); the wait uses the caller's bound, and after a timeout the
-    // default bound, so TMEM is read and freed only after the MMAs are done
-    if (tid == 0)
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(&mbar[2])));
+  } else if (lane == 0) {
+    // the issuing thread: B copies, MMAs, commits
+    // idesc: D = F32, A/B = BF16 (kind::f16) or TF32 (kind::tf32), both K-major, M = 128
+    uint32_t idesc = (1u << 4) | ((uint32_t)(out.npad >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    idesc |= ELEM == 4 ? ((2u << 7) | (2u << 10)) : ((1u << 7) | (1u << 10));
+    auto copy_b = [&](int j) {
+      const int st = j % b_stages;
+      const uint32_t bar = smem_u32(&mbar[5 + st]);
+      const uint32_t bytes = (uint32_t)(out.npad * ch[j].kpad * ELEM * PARTS);
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                       smem_u32(B0 + st * b_bytes)),
+                   "l"(ch[j].W), "r"(bytes), "r"(bar)
+                   : "memory");
+    };
+    const int ahead = b_stages - 2;   // B copies run this many chunks ahead
+    int copies = 0;
+    bool fail = false;
+    for (; copies < ahead && copies < nchunks; ++copies) copy_b(copies);
+    for (int j = 0; j < nchunks; ++j) {
+      const int b = j & 1, st = j % b_stages;
+      // chunk j - 2 read the stage that the next copy takes
+      if (j >= 2 && !mbar_wait(smem_u32(&mbar[b]), (uint32_t)((j >> 1) - 1) & 1u, polls)) { fail = true; break; }
+      if (copies < nchunks) copy_b(copies++);
+      if (!mbar_wait(smem_u32(&mbar[3 + b]), (uint32_t)(j >> 1) & 1u, polls) ||
+          !mbar_wait(smem_u32(&mbar[5 + st]), (uint32_t)(j / b_stages) & 1u, polls)) {
+        fail = true;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const int kq = ch[j].kpad * ELEM / 16;
+      const uint32_t sbo = (uint32_t)(kq * PARTS) * 128u;
+      const uint64_t ad = smem_desc(smem_u32(smem + b * a_bytes), 128, sbo);
+      const uint64_t bd = smem_desc(smem_u32(B0 + st * b_bytes), 128, sbo);
+      // a K step is two core matrices: 256 bytes, 16 in the descriptor
+      if (!SPLIT) {
+        for (int ks = 0; ks < kq / 2; ++ks)
+          mma<ELEM>(tmem, ad + ks * 16, bd + ks * 16, idesc, (j > 0 || ks > 0) ? 1u : 0u);
+      } else {
+        // x_hi W_hi + x_hi W_lo + x_lo W_hi; A and B tiles hold [hi | lo]
+        for (int g = 0; g < 3; ++g) {
+          const int pa = g == 2 ? kq * 8 : 0, pb = g == 1 ? kq * 8 : 0;
+          for (int ks = 0; ks < kq / 2; ++ks)
+            mma<ELEM>(tmem, ad + pa + ks * 16, bd + pb + ks * 16, idesc, (j > 0 || g > 0 || ks > 0) ? 1u : 0u);
+        }
+      }
+      tc_commit(smem_u32(&mbar[b]));
+    }
+    // drain: one more commit arrives on mbar[2] once every MMA issued has
+    // completed; after a timeout the default bound, here and for the copies
+    // whose wait was given up, so that TMEM and shared memory are read and
+    // freed only when nothing is in flight
+    tc_commit(smem_u32(&mbar[2]));
     if (!mbar_wait(smem_u32(&mbar[2]), 0, polls)) {
-      s_fail = 1;
+      fail = true;
       mbar_wait(smem_u32(&mbar[2]), 0);
     }
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (fail) {
+      s_fail = 1;
+      for (int j = max(0, copies - b_stages); j < copies; ++j)
+        mbar_wait(smem_u32(&mbar[5 + j % b_stages]), (uint32_t)(j / b_stages) & 1u);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
   }
   __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
   const bool ok = s_fail == 0;
   if (!ok && tid == 0) atomicExch(err, 1);
-  // epilogue: TMEM lanes 32*warp .. +31 hold rows row0 + 32*warp + lane
-  for (int c0 = 0; c0 < out.n; c0 += 16) {
+  // accumulator to shared memory (the A stages are free): warps w and w + 4
+  // read TMEM lanes 32 (w % 4) .. + 31, alternate groups of 16 columns
+  const int ld = out.npad + 1;
+  float* const D = (float*)smem;
+  for (int c0 = 16 * (warp >> 2); warp < TC_GATHER_WARPS && c0 < out.npad; c0 += 32) {
     uint32_t v[16];
     if (nchunks > 0) {
-      const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0;
+      const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
           : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
             "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
           : "r"(taddr));
       asm volatile("tcgen05.wait::ld.sync.aligned;");
-    } else {
-      for (int j = 0; j < 16; ++j) v[j] = 0u;
     }
-    if (!row_ok) continue;
-    double acc[16];
-    for (int j = 0; j < 16; ++j) acc[j] = ok ? (double)__uint_as_float(v[j]) : 0.0;
-    for (int ai = out.add_begin; ai < out.add_end; ++ai) {
-      const TcAdd a = adds[ai];
-      const int src = a.map ? a.map[row] : (row << 1);
-      if (src < 0) continue;
-      double s = (src & 1) ? -a.alpha : a.alpha;
-      if (a.val) s *= a.val[row];
-      const float* xr = a.X32 + (long long)(src >> 1) * a.ld + c0;
-      for (int j = 0; j < 16; ++j)
-        if (c0 + j < out.n) acc[j] += s * (double)xr[j];
-    }
-    double* yr = out.y + (long long)row * out.n + c0;
-    for (int j = 0; j < 16; ++j)
-      if (c0 + j < out.n) yr[j] = acc[j];
+    float* d = D + (32 * (warp & 3) + lane) * ld + c0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) d[j] = nchunks > 0 && ok ? __uint_as_float(v[j]) : 0.f;
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+  // lanes along the rows of y, adds in float-float with the factor and source
+  // row of the first TC_ADDS formed once per row
+  const int rows = min(128, out.rows - tile.row0), total = rows * out.n;
+  const int n_add = out.add_end - out.add_begin, held = min(n_add, TC_ADDS);
+  float2* const F = (float2*)(smem + ((size_t)128 * ld * 4 + 15) / 16 * 16);
+  int* const S = (int*)(F + TC_ADDS * 128);
+  int* const R = S + TC_ADDS * 128;
+  if (tid < rows) R[tid] = __ldg(out.order + tile.row0 + tid);
+  __syncthreads();
+  auto factor = [&](const TcAdd& a, int r, ff& f) {
+    const int g = R[r];
+    const int src = a.map ? __ldg(a.map + g) : (g << 1);
+    f = d2ff(a.alpha);
+    if (a.val) f = f * d2ff(__ldg(a.val + g));
+    if (src & 1) f = ff(-f.hi, -f.lo);
+    return src < 0 ? -1 : src >> 1;
+  };
+  for (int e = tid; e < held * 128; e += TC_THREADS) {
+    const int r = e & 127;
+    ff f;
+    S[e] = r < rows ? factor(adds[out.add_begin + (e >> 7)], r, f) : -1;
+    F[e] = make_float2(f.hi, f.lo);
+  }
+  __syncthreads();
+  double* const y = out.y + y_shift;
+  for (int e0 = tid; e0 < total; e0 += TC_UNROLL * TC_THREADS) {
+    ff acc[TC_UNROLL];
+    int r[TC_UNROLL], n[TC_UNROLL];
+#pragma unroll
+    for (int u = 0; u < TC_UNROLL; ++u) {
+      const int e = min(e0 + u * TC_THREADS, total - 1);
+      r[u] = out.n == 1 ? e : (int)__umulhi((unsigned)e, out.div);
+      n[u] = e - r[u] * out.n;
+      acc[u] = ff(D[r[u] * ld + n[u]]);
+    }
+    for (int i = 0; i < n_add; ++i) {
+      const TcAdd a = adds[out.add_begin + i];
+      ff f[TC_UNROLL];
+      float x[TC_UNROLL];
+#pragma unroll
+      for (int u = 0; u < TC_UNROLL; ++u) {
+        int src;
+        if (i < held) {
+          src = S[i * 128 + r[u]];
+          f[u] = ff(F[i * 128 + r[u]].x, F[i * 128 + r[u]].y);
+        } else {
+          src = factor(a, r[u], f[u]);
+        }
+        if (src < 0) f[u] = ff(0.f);
+        x[u] = src < 0 ? 0.f : __ldg(a.X32 + (long long)src * a.ld + n[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < TC_UNROLL; ++u) acc[u] = kc_fma(f[u], ff(x[u]), acc[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < TC_UNROLL; ++u)
+      if (e0 + u * TC_THREADS < total) y[(long long)R[r[u]] * out.n + n[u]] = to_d<ff>(acc[u]);
+  }
 }
 
-__device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
-
-// One warp per padded row, lanes along the row: coalesced reads of the
-// FP64 source and writes of the staged operand (no index division).
-template <int ELEM, int MODE>
-__global__ void __launch_bounds__(256) convert_kernel(const ConvJob* __restrict__ jobs) {
+// One warp per padded row, lanes along the row: coalesced reads of the FP64
+// source and writes of the FP32 copy (DST16: and of the BF16 one).  Converted
+// on the integer pipes: FP64 conversions run at the FP64 rate.
+template <bool DST16>
+__global__ void __launch_bounds__(256) convert_kernel(const ConvJob* __restrict__ jobs, long long shift) {
   const ConvJob j = jobs[blockIdx.y];
   const int lane = threadIdx.x & 31;
   const int warps = (int)(gridDim.x * (blockDim.x >> 5));
-  for (int r = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); r < j.rows; r += warps) {
-    const double* src = j.src + (long long)r * j.ld_src;
+  const double* src = j.src + shift;
+  for (int r = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 4; r < j.rows; r += warps * 4) {
     for (int c = lane; c < j.kpad; c += 32) {
-      const double v = c < j.cols ? j.scale * src[(long long)c * j.cs_src] : 0.0;
-      const long long e = (long long)r * j.kpad + c;
-      if (MODE == 0) {
-        if (ELEM == 2)
-          ((__nv_bfloat16*)j.dst)[e] = __double2bfloat16(v);
-        else
-          ((float*)j.dst)[e] = (float)v;
-      } else {
-        // [hi | lo] rows: hi = TF32-truncated, lo = FP32 residual
-        const float hi = tf32_hi((float)v);
-        const float lo = (float)(v - (double)hi);
-        float* d = (float*)j.dst + (long long)r * 2 * j.kpad;
-        d[c] = hi;
-        d[j.kpad + c] = lo;
+      double x[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        x[i] = c < j.cols && r + i < j.rows ? __ldg(src + (long long)(r + i) * j.ld_src + c) : 0.0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (r + i >= j.rows) break;
+        const float v = d2f_bits(x[i]);
+        const long long e = (long long)(r + i) * j.kpad + c;
+        j.dst32[e] = v;
+        if (DST16) ((__nv_bfloat16*)j.dst)[e] = __float2bfloat16(v);
       }
-      if (j.dst32) j.dst32[e] = (float)v;
+    }
+  }
+}
+
+// One environment block, scaled, as the B operand in core-matrix order (rows
+// padded with zeros to npad, columns to kpad): BF16, TF32, or TF32 [hi | lo].
+template <int ELEM, bool SPLIT>
+__global__ void __launch_bounds__(256) stage_w_kernel(const WJob* __restrict__ jobs) {
+  const WJob j = jobs[blockIdx.x];
+  const int kq = j.kpad * ELEM / 16, kchunks = SPLIT ? 2 * kq : kq;
+  uint8_t* dst = (uint8_t*)j.dst;
+  for (int e = threadIdx.x; e < j.npad * j.kpad; e += blockDim.x) {
+    const int n = e / j.kpad, k = e - n * j.kpad;
+    const double v = n < j.rows && k < j.cols ? j.scale * j.src[(long long)n * j.ld_src + k] : 0.0;
+    const int q = k * ELEM / 16, in = k * ELEM % 16;
+    if (ELEM == 2) {
+      *(__nv_bfloat16*)(dst + core_off(n, q, kchunks) + in) = __double2bfloat16(v);
+    } else if (!SPLIT) {
+      *(float*)(dst + core_off(n, q, kchunks) + in) = (float)v;
+    } else {
+      // hi = TF32-truncated, lo = FP32 residual
+      const float hi = tf32_hi((float)v);
+      *(float*)(dst + core_off(n, q, kchunks) + in) = hi;
+      *(float*)(dst + core_off(n, kq + q, kchunks) + in) = (float)(v - (double)hi);
     }
   }
 }
@@ -271,59 +472,55 @@ __global__ void __launch_bounds__(256) convert_kernel(const ConvJob* __restrict_
 }  // namespace
 
 int launch_tc_heff(int elem, int split, const TcTile* tiles, int n_tiles, const TcOutput* outs,
-                   const TcChunk* chunks, const TcAdd* adds, int max_kpad, int max_npad, int* err, cudaStream_t s,
-                   long long polls) {
+                   const TcChunk* chunks, const TcAdd* adds, int max_kpad, int max_npad, long long y_shift, int* err,
+                   cudaStream_t s, long long polls) {
   if (n_tiles <= 0) return 0;
   if (polls < 0) polls = kWaitPolls;
-  const int a_bytes = 128 * max_kpad * elem;
-  const int b_bytes = max_npad * max_kpad * elem;
-  const int smem = 2 * (a_bytes + b_bytes);
-  if (smem > 200 * 1024 || max_npad > 256 || max_npad % 16 || max_kpad % 16) return -7;
+  const int parts = split ? 2 : 1;
+  const int a_bytes = 128 * max_kpad * parts * elem;
+  const int b_bytes = max_npad * max_kpad * parts * elem;
+  if (2 * (a_bytes + b_bytes) > 200 * 1024 || max_npad > 256 || max_npad % 16 || max_kpad % 16) return -7;
   if (split && elem != 4) return -7;
-  if (elem == 2) {
-    static bool attr_2f = false;   // set once: host attribute calls cost as much as a launch
-    if (!attr_2f) {
-      cudaFuncSetAttribute(tc_heff_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      attr_2f = true;
-    }
-    tc_heff_kernel<2, false><<<n_tiles, TC_THREADS, smem, s>>>(tiles, outs, chunks, adds, a_bytes, b_bytes, err, polls);
-    count_launches(1);
-  } else if (!split) {
-    static bool attr_4f = false;   // set once: host attribute calls cost as much as a launch
-    if (!attr_4f) {
-      cudaFuncSetAttribute(tc_heff_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      attr_4f = true;
-    }
-    tc_heff_kernel<4, false><<<n_tiles, TC_THREADS, smem, s>>>(tiles, outs, chunks, adds, a_bytes, b_bytes, err, polls);
-    count_launches(1);
-  } else {
-    static bool attr_4t = false;   // set once: host attribute calls cost as much as a launch
-    if (!attr_4t) {
-      cudaFuncSetAttribute(tc_heff_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      attr_4t = true;
-    }
-    tc_heff_kernel<4, true><<<n_tiles, TC_THREADS, smem, s>>>(tiles, outs, chunks, adds, a_bytes, b_bytes, err, polls);
-    count_launches(1);
+  // three or four B stages where that costs no CTA of the SM
+  const int sm = 226 * 1024, fit = std::max(1, sm / (2 * (a_bytes + b_bytes) + 1024));
+  int b_stages = 2;
+  while (b_stages < 4 && sm / (2 * a_bytes + (b_stages + 1) * b_bytes + 1024) >= std::min(fit, 2)) ++b_stages;
+  const int smem = std::max(2 * a_bytes + b_stages * b_bytes, 128 * (max_npad + 1) * 4 + 16 + TC_ADDS * 128 * 12 + 128 * 4);
+  auto kern = elem == 2 ? tc_heff_kernel<2, false> : (split ? tc_heff_kernel<4, true> : tc_heff_kernel<4, false>);
+  static bool attr[3] = {false, false, false};   // set once: host attribute calls cost as much as a launch
+  bool& set = attr[elem == 2 ? 0 : (split ? 2 : 1)];
+  if (!set) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    set = true;
   }
+  kern<<<n_tiles, TC_THREADS, smem, s>>>(tiles, outs, chunks, adds, a_bytes, b_bytes, b_stages, y_shift, err, polls);
+  count_launches(1);
   return 0;
 }
 
-void launch_convert(int elem, int mode, const ConvJob* jobs, int n_jobs, long long max_elems, cudaStream_t s) {
+void launch_convert(int elem, const ConvJob* jobs, int n_jobs, long long max_elems, long long shift, cudaStream_t s) {
   if (n_jobs <= 0) return;
-  // rows <= max_elems / 16 (kpad >= 16); 8 rows per block, about 4 blocks per SM in total
-  long long gx = (max_elems / 16 + 7) / 8;
-  const long long cap = std::max(1LL, 608LL / n_jobs);
+  // rows <= max_elems / 16 (kpad >= 16); 32 rows per block, about 8 blocks per SM in total
+  long long gx = (max_elems / 16 + 31) / 32;
+  const long long cap = std::max(1LL, 1216LL / n_jobs);
   if (gx > cap) gx = cap;
   if (gx < 1) gx = 1;
   dim3 grid((unsigned)gx, (unsigned)n_jobs);
-  if (mode == 1)
-    convert_kernel<4, 1><<<grid, 256, 0, s>>>(jobs);
-  else if (mode == 2)
-    convert_kernel<4, 2><<<grid, 256, 0, s>>>(jobs);
-  else if (elem == 2)
-    convert_kernel<2, 0><<<grid, 256, 0, s>>>(jobs);
+  if (elem == 2)
+    convert_kernel<true><<<grid, 256, 0, s>>>(jobs, shift);
   else
-    convert_kernel<4, 0><<<grid, 256, 0, s>>>(jobs);
+    convert_kernel<false><<<grid, 256, 0, s>>>(jobs, shift);
+  count_launches(1);
+}
+
+void launch_stage_w(int elem, int split, const WJob* jobs, int n_jobs, cudaStream_t s) {
+  if (n_jobs <= 0) return;
+  if (elem == 2)
+    stage_w_kernel<2, false><<<n_jobs, 256, 0, s>>>(jobs);
+  else if (split)
+    stage_w_kernel<4, true><<<n_jobs, 256, 0, s>>>(jobs);
+  else
+    stage_w_kernel<4, false><<<n_jobs, 256, 0, s>>>(jobs);
   count_launches(1);
 }
 
