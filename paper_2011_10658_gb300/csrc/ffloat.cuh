@@ -101,8 +101,13 @@ __device__ __forceinline__ double to_t<double>(double v) { return v; }
 template <>
 __device__ __forceinline__ float to_t<float>(double v) { return d2f_bits(v); }
 
+// hi rounded to nearest: the lo lo product that a multiply-add drops is then
+// a quarter of what two truncated parts leave, and of either sign.
 template <>
-__device__ __forceinline__ ff to_t<ff>(double v) { return d2ff(v); }
+__device__ __forceinline__ ff to_t<ff>(double v) {
+  const ff t = d2ff(v);
+  return ff_norm(t.hi, t.lo);
+}
 
 // Values outside the range of the short form below: zeros, magnitudes below
 // 2^-103 (whose lo part nears the FP32 subnormals) or past the FP32 range,

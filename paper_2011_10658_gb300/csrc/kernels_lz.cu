@@ -35,6 +35,12 @@ constexpr int LZ_MAX_K = 128;
 constexpr int LZ_DIRECT = 64;                    // grids up to this size: every block adds all partial sums itself
 constexpr long long kLzPolls = 1LL << 22;        // bound of a grid barrier's wait (seconds)
 
+// Operands as they come: the sums' own rounding is above what to_t would save.
+template <typename A>
+__device__ __forceinline__ A lz_in(double v) { return v; }
+template <>
+__device__ __forceinline__ ff lz_in<ff>(double v) { return d2ff(v); }
+
 template <typename A>
 __device__ __forceinline__ A lz_xor(A v, int m);
 template <>
@@ -113,19 +119,19 @@ __device__ __forceinline__ void lz_dots(const LzStep& p, double (*sh)[LZ_COLS], 
         double v[LZ_COLS];
 #pragma unroll
         for (int t = 0; t < LZ_COLS; ++t) v[t] = __ldg(col[t] + i);
-        const A ya = to_t<A>(p.y[i]);
+        const A ya = lz_in<A>(p.y[i]);
 #pragma unroll
-        for (int t = 0; t < LZ_COLS; ++t) acc[t] = kc_fma(to_t<A>(v[t]), ya, acc[t]);
+        for (int t = 0; t < LZ_COLS; ++t) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
       }
     } else {
       for (long long i = i0; i < p.n; i += step) {
         double v[LZ_COLS];
 #pragma unroll
         for (int t = 0; t < LZ_COLS; ++t) v[t] = t < cols ? __ldg(col[t] + i) : 0.0;
-        const A ya = to_t<A>(p.y[i]);
+        const A ya = lz_in<A>(p.y[i]);
 #pragma unroll
         for (int t = 0; t < LZ_COLS; ++t) {
-          if (t < cols) acc[t] = kc_fma(to_t<A>(v[t]), ya, acc[t]);
+          if (t < cols) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
           else if (t == cols) acc[t] = kc_fma(ya, ya, acc[t]);
         }
       }
@@ -181,12 +187,12 @@ __device__ __forceinline__ void lz_columns(const LzStep& p, int ncol, double* co
 // y -= V c; returns this thread's part of |y|^2.
 template <typename A>
 __device__ __forceinline__ A lz_update(const LzStep& p, const double* c, A* cs, long long i0, long long step) {
-  for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = to_t<A>(-c[j]);
+  for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = lz_in<A>(-c[j]);
   __syncthreads();
   A nrm = A(0);
 #pragma unroll 2
   for (long long i = i0; i < p.n; i += step) {
-    A v = to_t<A>(p.y[i]);
+    A v = lz_in<A>(p.y[i]);
     const double* q = p.V + i;
     int j = 0;
     for (; j + LZ_COLS <= p.k; j += LZ_COLS) {
@@ -194,9 +200,9 @@ __device__ __forceinline__ A lz_update(const LzStep& p, const double* c, A* cs, 
 #pragma unroll
       for (int t = 0; t < LZ_COLS; ++t) x[t] = __ldg(q + (long long)(j + t) * p.ldq);
 #pragma unroll
-      for (int t = 0; t < LZ_COLS; ++t) v = kc_fma(cs[j + t], to_t<A>(x[t]), v);
+      for (int t = 0; t < LZ_COLS; ++t) v = kc_fma(cs[j + t], lz_in<A>(x[t]), v);
     }
-    for (; j < p.k; ++j) v = kc_fma(cs[j], to_t<A>(__ldg(q + (long long)j * p.ldq)), v);
+    for (; j < p.k; ++j) v = kc_fma(cs[j], lz_in<A>(__ldg(q + (long long)j * p.ldq)), v);
     p.y[i] = to_d<A>(v);
     nrm = kc_fma(v, v, nrm);
   }
