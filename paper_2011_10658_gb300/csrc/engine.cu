@@ -99,24 +99,28 @@ void device_alloc(void** p, size_t bytes, const char* what) {
 }
 
 // ------------------------------------------------------------------ KPlan
-int KPlan::add_output(double* C, long long c_m, long long c_n, int M, int N, int accumulate) {
+// ceil(2^32 / d): e / d = umulhi(e, that) for the e d < 2^32 that occur (d = 1
+// and d = 0 are not divided by)
+static unsigned reciprocal(int d) { return d > 1 ? (unsigned)(((1ull << 32) + d - 1) / d) : 0u; }
+
+int KPlan::add_output(double* C, long long c_m, long long c_n, int M, int N, int accumulate, int nin, long long c_no) {
   auto key = std::make_tuple((uintptr_t)C, c_m, c_n, M, N);
   auto it = out_index.find(key);
   if (it != out_index.end()) {
     current = it->second;
     return current;
   }
-  KOutput o;
+  KOutput o{};
   o.C = C;
   o.c_m = c_m;
   o.c_n = c_n;
   o.M = M;
   o.N = N;
-  o.chunk_begin = 0;
-  o.chunk_end = 0;
   o.accumulate = accumulate;
   o.n_parts = 1;
-  o.part_off = 0;
+  o.nin = nin;
+  o.ndiv = reciprocal(nin);
+  o.c_no = c_no;
   outs.push_back(o);
   out_chunks.emplace_back();
   current = (int)outs.size() - 1;
@@ -196,16 +200,18 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
           nc.push_back(ch);
           acc += 1;
         } else {
-          for (int k0 = 0; k0 < ch.K; k0 += (int)kp) {
+          // a two-level K is cut between its inner runs
+          const int step = ch.kin ? std::max(ch.kin, (int)kp / ch.kin * ch.kin) : (int)kp;
+          for (int k0 = 0; k0 < ch.K; k0 += step) {
             KChunk sc = ch;
-            sc.K = std::min<int>((int)kp, ch.K - k0);
+            sc.K = std::min<int>(step, ch.K - k0);
             if (ch.bmap) {
               sc.bmap = ch.bmap + k0;
               if (ch.bval) sc.bval = ch.bval + k0;
             } else {
-              sc.B = ch.B + (long long)k0 * ch.b_k;
+              sc.B = ch.B + (ch.kin ? (long long)(k0 / ch.kin) * ch.b_ko : (long long)k0 * ch.b_k);
             }
-            sc.A = ch.A + (long long)k0 * ch.a_k;
+            sc.A = ch.A + (ch.kin ? (long long)(k0 / ch.kin) * ch.a_ko : (long long)k0 * ch.a_k);
             nc.push_back(sc);
             acc += sc.K;
             if (acc >= kp) {
@@ -271,13 +277,12 @@ BhPlan& KPlan::bh_plan(cudaStream_t s) {
   b.tiles.clear(); b.outs.clear(); b.chunks.clear(); b.jobs.clear();
   b.w_elems = 0;
   b.max_n = b.max_k = 1;
-  auto recip = [](int d) { return (unsigned)(((1ull << 32) + d - 1) / d); };   // ceil(2^32 / d), unused for d = 1
   for (const KOutput& o : outs) {
     BhOut bo{};
     bo.C = o.C;
     bo.M = o.M;
     bo.N = o.N;
-    bo.div = recip(o.N);
+    bo.div = reciprocal(o.N);
     bo.chunk_begin = (int)b.chunks.size();
     b.max_n = std::max(b.max_n, o.N);
     for (int ci = o.chunk_begin; ci < o.chunk_end; ++ci) {
@@ -290,7 +295,7 @@ BhPlan& KPlan::bh_plan(cudaStream_t s) {
       bc.ld = (int)c.a_m;
       if (!c.add) {
         bc.K = c.K;
-        bc.div = recip(c.K);
+        bc.div = reciprocal(c.K);
         bc.w = b.w_elems;
         b.max_k = std::max(b.max_k, c.K);
         BhJob j{};
@@ -511,8 +516,12 @@ bool Engine::in_own_range(const void* p, long long lo_bytes, long long hi_bytes)
 // known device allocation (enabled by QED_VALIDATE=1).  Row-mapped operands
 // are checked over their whole source sector by the row-map builder.
 bool Engine::validate_plan(const KPlan& pl, const KVariant* v, const char* what) {
+  // largest offset of a one- or two-level index of n values
+  auto reach = [](int n, int in, long long inner, long long outer) {
+    return in ? (long long)((n - 1) / in) * outer + (long long)(std::min(n, in) - 1) * inner : (long long)(n - 1) * inner;
+  };
   for (const KOutput& o : pl.outs) {
-    const long long hi = (long long)(o.M - 1) * o.c_m + (long long)(o.N - 1) * o.c_n;
+    const long long hi = (long long)(o.M - 1) * o.c_m + reach(o.N, o.nin, o.c_n, o.c_no);
     if (o.M <= 0 || o.N <= 0 || !in_range(o.C, 0, hi * 8 + 8)) {
       err_ = std::string(what) + ": output out of range";
       return false;
@@ -522,7 +531,7 @@ bool Engine::validate_plan(const KPlan& pl, const KVariant* v, const char* what)
       const int K = c.add ? o.N : c.K;
       if (K <= 0) { err_ = std::string(what) + ": empty chunk"; return false; }
       if (!c.amap) {
-        const long long ahi = (long long)(o.M - 1) * c.a_m + (long long)(K - 1) * c.a_k;
+        const long long ahi = (long long)(o.M - 1) * c.a_m + reach(K, c.kin, c.a_k, c.a_ko);
         if (!in_range(c.A, 0, ahi * 8 + 8)) {
           err_ = std::string(what) + ": A operand out of range";
           return false;
@@ -533,7 +542,7 @@ bool Engine::validate_plan(const KPlan& pl, const KVariant* v, const char* what)
       }
       if (!c.add) {
         if (!c.bmap) {
-          const long long bhi = (long long)(K - 1) * c.b_k + (long long)(o.N - 1) * c.b_n;
+          const long long bhi = reach(K, c.kin, c.b_k, c.b_ko) + reach(o.N, o.nin, c.b_n, c.b_no);
           if (!in_range(c.B, 0, bhi * 8 + 8)) {
             err_ = std::string(what) + ": B operand out of range";
             return false;
@@ -1045,14 +1054,13 @@ void Engine::plan_leg_apply(KPlan& pl, const Layout& LX, const double* X, const 
       c.K = b.da; c.alpha = alpha;
       pl.add_chunk(c);
     } else if (leg == 1) {
-      for (int a = 0; a < b.da; ++a) {
-        pl.add_output(Y + yb.off + (long long)a * yb.db * yb.dc, yb.dc, 1, yb.db, yb.dc, 0);
-        KChunk c = make_chunk();
-        c.A = Pblk; c.a_m = p_r; c.a_k = p_c;
-        c.B = X + b.off + (long long)a * b.db * b.dc; c.b_k = b.dc; c.b_n = 1;
-        c.K = b.db; c.alpha = alpha;
-        pl.add_chunk(c);
-      }
+      // columns (a, c): one output per block
+      pl.add_output(Y + yb.off, yb.dc, 1, yb.db, b.da * yb.dc, 0, yb.dc, (long long)yb.db * yb.dc);
+      KChunk c = make_chunk();
+      c.A = Pblk; c.a_m = p_r; c.a_k = p_c;
+      c.B = X + b.off; c.b_k = b.dc; c.b_n = 1; c.b_no = (long long)b.db * b.dc;
+      c.K = b.db; c.alpha = alpha;
+      pl.add_chunk(c);
     } else {
       pl.add_output(Y + yb.off, yb.dc, 1, yb.da * yb.db, yb.dc, 0);
       KChunk c = make_chunk();
@@ -1104,13 +1112,13 @@ void Engine::plan_contract_but(KPlan& pl, const Layout& LT, const double* T, con
         c.K = tb.db * tb.dc; c.alpha = alpha;
         acc[{tb.ia, zb.ia}].push_back(c);
       } else {
-        for (int a = 0; a < tb.da; ++a) {
-          KChunk c = make_chunk();
-          c.A = T + tb.off + (long long)a * tb.db * tb.dc; c.a_m = tb.dc; c.a_k = 1;
-          c.B = Z + zb.off + (long long)a * zb.db * zb.dc; c.b_k = 1; c.b_n = zb.dc;
-          c.K = tb.dc; c.alpha = alpha;
-          acc[{tb.ib, zb.ib}].push_back(c);
-        }
+        // K = (a, c): one chunk per block
+        KChunk c = make_chunk();
+        c.A = T + tb.off; c.a_m = tb.dc; c.a_k = 1; c.a_ko = (long long)tb.db * tb.dc;
+        c.B = Z + zb.off; c.b_k = 1; c.b_n = zb.dc; c.b_ko = (long long)zb.db * zb.dc;
+        c.kin = tb.dc; c.kdiv = reciprocal(tb.dc);
+        c.K = tb.da * tb.dc; c.alpha = alpha;
+        acc[{tb.ib, zb.ib}].push_back(c);
       }
     }
   }
@@ -2403,7 +2411,7 @@ TcPlan* Engine::tc_plan(int node) {
     o.rows = rows;
     o.n = P.dim[oc];
     o.npad = kpad[oc];
-    o.div = (unsigned)(((1ull << 32) + o.n - 1) / o.n);
+    o.div = reciprocal(o.n);
     o.order = (const int*)(intptr_t)tc.order.size();   // patched below once uploaded
     std::vector<TcChunk> sector_chunks;
     std::vector<std::pair<const SiteOp*, const SiteOp*>> sector_ops;   // its two site operators (null: identity)
@@ -3349,6 +3357,7 @@ int Engine::noalloc_worklist(const double* x, double* y, KTile* tiles, int max_t
     const int dc = P.dim[oc];
     if (no >= max_outs) { err_ = "work list: too many outputs"; return -2; }
     KOutput& o = outs[no];
+    o = KOutput{};
     o.C = y + L.sec_off[oc];
     o.c_m = dc;
     o.c_n = 1;

@@ -123,7 +123,7 @@ struct KPlan {
     for (KVariant& v : var) v.ready = false;
     gather = bh.ready = false;
   }
-  int add_output(double* C, long long c_m, long long c_n, int M, int N, int accumulate);
+  int add_output(double* C, long long c_m, long long c_n, int M, int N, int accumulate, int nin = 0, long long c_no = 0);
   void add_chunk(const KChunk& c);
   void finalize(long long k_part);
   KVariant& variant(int shape, cudaStream_t s);

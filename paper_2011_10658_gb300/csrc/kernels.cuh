@@ -13,6 +13,10 @@ void count_launches(int n);
 //   A[m,k] = sA * aval[m] * A[row*a_m + k*a_k],  amap[m] = (row << 1) | negate, -1 = zero row
 //   B[k,n] = sB * bval[k] * B[row*b_k + n*b_n],  bmap[k] likewise (maps and vals optional)
 // With add != 0 there is no B:  C[m,n] += alpha * A[m,n] (A[m,n] addressed as A[m,k=n]).
+// Two-level K (kin > 0): k stands for (k / kin, k % kin) and adds (k / kin) *
+// a_ko + (k % kin) * a_k (b_ko, b_k in B), so that a contraction over two legs
+// around a third is one chunk.  Two-level N (nin > 0 in the output) likewise,
+// with b_no in B and c_no in C.  kdiv, ndiv: ceil(2^32 / kin), ceil(2^32 / nin).
 struct KChunk {
   const double* A;
   long long a_m, a_k;
@@ -25,6 +29,9 @@ struct KChunk {
   int K;
   int add;
   double alpha;
+  long long a_ko, b_ko, b_no;
+  int kin;
+  unsigned kdiv;
 };
 
 // An output C (MxN, C[m,n] at C + m*c_m + n*c_n) = sum of its chunks
@@ -37,6 +44,9 @@ struct KOutput {
   int accumulate;
   int n_parts;        // > 1: split over chunk ranges, partial sums in scratch
   long long part_off; // scratch offset (doubles) of this output's partials
+  long long c_no;
+  int nin;
+  unsigned ndiv;
 };
 
 // One CTA's work: a BM x BN tile of an output over a chunk range.

@@ -22,6 +22,13 @@ namespace {
 constexpr int BK = 16;
 constexpr int THREADS = 256;
 
+// Two-level index e -> (e / in) * outer + (e % in) * inner (in = 0: one level).
+__device__ __forceinline__ long long two_level(int e, int in, unsigned div, long long inner, long long outer) {
+  if (in == 0) return (long long)e * inner;
+  const int o = in == 1 ? e : (int)__umulhi((unsigned)e, div);
+  return (long long)o * outer + (long long)(e - o * in) * inner;
+}
+
 // Row maps are sign-encoded: -1 = zero row, otherwise (row << 1) | negate.
 // Arithmetic in T (FP64, or FP32 with the operands converted first).
 template <typename T>
@@ -35,21 +42,17 @@ __device__ __forceinline__ T load_a(const KChunk& c, int m, int k) {
     if (r & 1) scale = T(-1);
   }
   if (c.aval) scale *= to_t<T>(c.aval[m]);
-  return scale * to_t<T>(c.A[row * c.a_m + (long long)k * c.a_k]);
+  return scale * to_t<T>(c.A[row * c.a_m + two_level(k, c.kin, c.kdiv, c.a_k, c.a_ko)]);
 }
 
 template <typename T>
-__device__ __forceinline__ T load_b(const KChunk& c, int k, int n) {
-  long long row = k;
-  T scale = T(1);
-  if (c.bmap) {
-    int r = c.bmap[k];
-    if (r < 0) return T(0);
-    row = r >> 1;
-    if (r & 1) scale = T(-1);
-  }
+__device__ __forceinline__ T load_b(const KChunk& c, int k, long long n_off) {
+  if (!c.bmap) return to_t<T>(c.B[two_level(k, c.kin, c.kdiv, c.b_k, c.b_ko) + n_off]);
+  const int r = c.bmap[k];
+  if (r < 0) return T(0);
+  T scale = (r & 1) ? T(-1) : T(1);
   if (c.bval) scale *= to_t<T>(c.bval[k]);
-  return scale * to_t<T>(c.B[row * c.b_k + (long long)n * c.b_n]);
+  return scale * to_t<T>(c.B[(long long)(r >> 1) * c.b_k + n_off]);
 }
 
 // One CTA computes a BM x BN tile of one output (16 x 16 threads, each a
@@ -94,7 +97,7 @@ __global__ void __launch_bounds__(THREADS) kc_gemm_kernel(const KTile* __restric
       for (int e = tid; e < BN * BK; e += THREADS) {
         const int kk = e / BN, nn = e % BN;
         const int n = tile.n0 + nn, k = k0 + kk;
-        Bs[kk][nn] = (n < out.N && k < c.K) ? load_b<T>(c, k, n) : T(0);
+        Bs[kk][nn] = (n < out.N && k < c.K) ? load_b<T>(c, k, two_level(n, out.nin, out.ndiv, c.b_n, c.b_no)) : T(0);
       }
       __syncthreads();
 #pragma unroll
@@ -122,7 +125,7 @@ __global__ void __launch_bounds__(THREADS) kc_gemm_kernel(const KTile* __restric
       if (tile.part >= 0) {
         scratch[out.part_off + (long long)tile.part * out.M * out.N + (long long)m * out.N + n] = v;
       } else {
-        double* p = out.C + (long long)m * out.c_m + (long long)n * out.c_n;
+        double* p = out.C + (long long)m * out.c_m + two_level(n, out.nin, out.ndiv, out.c_n, out.c_no);
         *p = out.accumulate ? (*p + v) : v;
       }
     }
@@ -136,7 +139,7 @@ __global__ void kc_reduce_kernel(const KOutput* __restrict__ outs, const int* __
     double s = 0.0;
     for (int p = 0; p < out.n_parts; ++p) s += scratch[out.part_off + p * mn + e];
     int m = (int)(e / out.N), n = (int)(e % out.N);
-    double* c = out.C + (long long)m * out.c_m + (long long)n * out.c_n;
+    double* c = out.C + (long long)m * out.c_m + two_level(n, out.nin, out.ndiv, out.c_n, out.c_no);
     *c = out.accumulate ? (*c + s) : s;
   }
 }
@@ -249,63 +252,89 @@ __global__ void fill_uniform_kernel(double* __restrict__ x, long long n, uint64_
   }
 }
 
-// Upper Cholesky G = R^T R in shared memory, then R^{-1} by back substitution.
-// One CTA per matrix; n <= 256.
-__global__ void cholesky_inv_kernel(double* G, double* Rinv, const long long* off, const int* nn, const int* ldd,
-                                    int* status, double ill_cond) {
+// Upper Cholesky G = R^T R and X = R^{-1}, one CTA per matrix, in one n x n
+// array of shared memory: U = D^{1/2} R above the diagonal, X transposed below
+// it.  A column of the root-free form costs one reciprocal where a square root
+// and a division stood (the serial chain of an FP64 operation is 65 cycles
+// and more here), the square roots follow side by side, and X grows by outer
+// products, a row finished and spread over the rows above it in each step.
+// 32 columns: 64 us before (column solves in one thread each), see the centre
+// moves in the engine for the whole.
+__global__ void __launch_bounds__(256) cholesky_inv_kernel(double* G, double* Rinv, const long long* off,
+                                                           const int* nn, const int* ldd, int* status,
+                                                           double ill_cond) {
   extern __shared__ double sh[];
   const int idx = blockIdx.x;
   const int n = nn[idx], ld = ldd[idx];
   double* g = G + off[idx];
   double* ri = Rinv + off[idx];
-  double* R = sh;                // n x n
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) R[e] = g[(e / n) * ld + (e % n)];
-  __syncthreads();
+  double* R = sh;              // n x n
+  __shared__ double inv, rs[160], row[160], gmax;
   __shared__ int bad;
-  if (threadIdx.x == 0) bad = 0;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < n * n; e += blockDim.x) R[e] = g[(e / n) * ld + (e % n)];
+  if (tid == 0) bad = 0;
   __syncthreads();
   // largest original diagonal = squared largest column norm of the factored matrix
-  __shared__ double gmax;
-  if (threadIdx.x == 0) {
+  if (tid < 32) {
     double mx = 0.0;
-    for (int j = 0; j < n; ++j) mx = fmax(mx, R[j * n + j]);
-    gmax = mx;
+    for (int j = tid; j < n; j += 32) mx = fmax(mx, R[j * n + j]);
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (tid == 0) gmax = mx;
   }
   __syncthreads();
-  // right-looking: for column j, R[j][j] = sqrt(G[j][j]), R[j][i] = G[j][i]/R[j][j], trailing update
+  // u_jb (row j) with d_j = u_jj; trailing a_ab -= u_ja u_jb / d_j
   for (int j = 0; j < n; ++j) {
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       double d = R[j * n + j];
-      if (!(d > 0.0)) { bad = 1; d = 1.0; }
+      if (!(d > 0.0)) { bad = 1; d = 1.0; R[j * n + j] = 1.0; }
       else if (d <= ill_cond * gmax) bad = bad ? bad : 2;
-      R[j * n + j] = sqrt(d);
+      inv = 1.0 / d;
     }
     __syncthreads();
-    const double rjj = R[j * n + j];
-    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) R[j * n + i] /= rjj;
+    const int w = n - j - 1;
+    for (int i = tid; i < w; i += blockDim.x) row[i] = -R[j * n + j + 1 + i] * inv;
     __syncthreads();
-    for (int e = threadIdx.x; e < (n - j - 1) * (n - j - 1); e += blockDim.x) {
-      int a = j + 1 + e / (n - j - 1), b = j + 1 + e % (n - j - 1);
-      if (b >= a) R[a * n + b] -= R[j * n + a] * R[j * n + b];
+    for (int e = tid; e < w * w; e += blockDim.x) {
+      const int a = e / w, b = e - a * w;
+      if (b >= a) {
+        double* p = R + (j + 1 + a) * n + j + 1 + b;
+        *p = fma(row[a], R[j * n + j + 1 + b], *p);
+      }
     }
     __syncthreads();
   }
-  // write R (upper) back to G, zero below
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    int a = e / n, b = e % n;
-    g[a * ld + b] = b >= a ? R[e] : 0.0;
+  for (int j = tid; j < n; j += blockDim.x) rs[j] = 1.0 / sqrt(R[j * n + j]);
+  __syncthreads();
+  // R = D^{-1/2} U in place and to G; the transposed sums of X start at zero
+  for (int e = tid; e < n * n; e += blockDim.x) {
+    const int a = e / n, b = e - a * n;
+    const double v = b >= a ? R[e] * rs[a] : 0.0;
+    R[e] = v;
+    g[a * ld + b] = v;
   }
   __syncthreads();
-  // Rinv: solve R X = I column by column (thread per column)
-  for (int col = threadIdx.x; col < n; col += blockDim.x) {
-    for (int a = n - 1; a >= 0; --a) {
-      double v = (a == col) ? 1.0 : 0.0;
-      for (int b = a + 1; b <= col; ++b) v -= R[a * n + b] * ri[b * ld + col];
-      ri[a * ld + col] = (a <= col) ? v / R[a * n + a] : 0.0;
+  // X_ij = -rs_i sum_{i < k <= j} R_ik X_kj (X_ii = rs_i): row i is finished,
+  // then added to the sums of the rows above
+  for (int i = n - 1; i >= 0; --i) {
+    for (int j = i + tid; j < n; j += blockDim.x) {
+      const double x = j == i ? rs[i] : -R[j * n + i] * rs[i];
+      row[j] = x;
+      if (j > i) R[j * n + i] = x;
     }
-    for (int a = col + 1; a < n; ++a) ri[a * ld + col] = 0.0;
+    __syncthreads();
+    const int w = n - i;
+    for (int e = tid; e < i * w; e += blockDim.x) {
+      const int k = e / w, j = i + e - k * w;
+      R[j * n + k] = fma(R[k * n + i], row[j], R[j * n + k]);
+    }
+    __syncthreads();
   }
-  if (threadIdx.x == 0) status[idx] = bad;
+  for (int e = tid; e < n * n; e += blockDim.x) {
+    const int a = e / n, b = e - a * n;
+    ri[a * ld + b] = b > a ? R[b * n + a] : (b == a ? rs[a] : 0.0);
+  }
+  if (tid == 0) status[idx] = bad;
 }
 
 

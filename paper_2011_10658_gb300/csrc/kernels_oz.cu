@@ -358,22 +358,36 @@ __global__ void __launch_bounds__(OZ_THREADS) oz_gram_kernel(const OzTile* __res
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOLS));
 }
 
-// O[c', c] (+)= sum over the output's entries (partial block, alpha) in order.
-__global__ void oz_reduce_kernel(const OzOut* __restrict__ outs, const OzSum* __restrict__ sums,
-                                 const double* __restrict__ partial) {
+// O[c', c] += sum over the output's entries (partial block, alpha).  A CTA takes
+// 64 elements of one output, neighbouring lanes along c' (the contiguous index
+// of a partial block); four lanes share an element, each adding every fourth
+// partial sum, and are combined in a fixed order.
+constexpr int OZ_RED = 64;
+
+__global__ void __launch_bounds__(4 * OZ_RED) oz_reduce_kernel(const OzOut* __restrict__ outs,
+                                                               const OzSum* __restrict__ sums,
+                                                               const double* __restrict__ partial) {
+  __shared__ double sh[4][OZ_RED];
   const OzOut o = outs[blockIdx.x];
-  const int mn = o.rows * o.cols;
-  for (int e = threadIdx.x; e < mn; e += blockDim.x) {
-    const int cp = e / o.cols, cc = e % o.cols;   // O row c' (output sector), column c (source sector)
+  const int mn = o.rows * o.cols, el = threadIdx.x & (OZ_RED - 1), share = threadIdx.x / OZ_RED;
+  for (int e0 = blockIdx.y * OZ_RED; e0 < mn; e0 += gridDim.y * OZ_RED) {
+    const int e = e0 + el;
     double s = 0.0;
-    for (int k = o.sum_begin; k < o.sum_end; ++k) {
-      const OzSum t = sums[k];
-      double v = 0.0;
-      for (int p = 0; p < t.n_parts; ++p) v += partial[t.off + (long long)p * t.part_stride + (long long)cc * o.rows + cp];
-      s += t.alpha * v;
+    if (e < mn)
+      for (int k = o.sum_begin; k < o.sum_end; ++k) {
+        const OzSum t = sums[k];
+        double v = 0.0;
+#pragma unroll 4
+        for (int p = share; p < t.n_parts; p += 4) v += __ldg(partial + t.off + (long long)p * t.part_stride + e);
+        s = fma(t.alpha, v, s);
+      }
+    sh[share][el] = s;
+    __syncthreads();
+    if (share == 0 && e < mn) {
+      const int cc = e / o.rows, cp = e - cc * o.rows;   // O row c' (output sector), column c (source sector)
+      o.O[(long long)cp * o.ld + cc] += (sh[0][el] + sh[1][el]) + (sh[2][el] + sh[3][el]);
     }
-    double* dst = o.O + (long long)cp * o.ld + cc;
-    *dst += s;
+    __syncthreads();
   }
 }
 
@@ -414,7 +428,7 @@ int launch_oz_gram(const OzTile* tiles, int n_tiles, const OzJob* jobs, const vo
   kern<<<grid, OZ_THREADS, smem, s>>>(tiles, n_tiles, jobs, (const uint4*)planes, partial, err, polls);
   count_launches(1);
   if (n_outs > 0) {
-    oz_reduce_kernel<<<n_outs, 256, 0, s>>>(outs, sums, partial);
+    oz_reduce_kernel<<<dim3(n_outs, 8), 4 * OZ_RED, 0, s>>>(outs, sums, partial);
     count_launches(1);
   }
   return 0;
