@@ -166,8 +166,12 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
   v.chunks.reserve(chunks.size());
   v.outs = outs;
   v.scratch_need = 0;
-  // K per part: small enough that the launch has about four tiles per SM
-  // when the plan has few, long contractions (a Gram matrix), at most k_part
+  // K per part: small enough that the launch has about eight tiles per SM
+  // when the plan has few, long contractions (a Gram matrix), at most k_part.
+  // A slab of 16 is one trip to L2, so long sums are cut down to 192 (GB300,
+  // 4x4x4: centre move chi=64 15.6 ms at 4 tiles and 256, 14.7 ms at 8 and 192,
+  // 14.4 ms at 16 and 128, where the short sums of an upper-node update at
+  // chi=32 lose more to the reduction: 8.4, 8.5, 9.0 ms)
   long long work = 0, base_tiles = 0;
   for (const KOutput& o : outs) {
     long long ktot = 0;
@@ -176,8 +180,8 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
     work += t * ktot;
     base_tiles += t;
   }
-  const long long kp = std::max(256LL, std::min(k_part, work / (4 * 152)));
-  const bool few_tiles = base_tiles < 4 * 152;
+  const long long kp = std::max(192LL, std::min(k_part, work / (8 * 152)));
+  const bool few_tiles = base_tiles < 8 * 152;
   std::vector<KChunk>& nc = v.chunks;
   for (size_t oi = 0; oi < outs.size(); ++oi) {
     KOutput& o = v.outs[oi];
