@@ -209,7 +209,7 @@ int BatchRunner::launch(Grouped& g) {
     for (int i = 0; i < 3; ++i) {
       TgPlan& p = g.tgs[i];
       const int rc = launch_tg_gemm(elem, split, p.d_tiles, (int)p.tiles.size(), p.d_outs, p.d_chunks, p.max_npad,
-                                    g.tg_scratch, p.d_red, (int)p.red.size(), e0->d_err_, s, e0->wait_polls);
+                                    g.tg_scratch, p.d_red, (int)p.red.size(), 0, 0, e0->d_err_, s, e0->wait_polls);
       if (rc) {
         e0->err_ = "tensor-core contraction: output width outside the supported range";
         return rc;

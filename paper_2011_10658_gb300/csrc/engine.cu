@@ -2177,11 +2177,7 @@ int Engine::apply_heff(const double* x, double* y, int cls) {
   }
   if (use_mixed_ && cls < 0) {
     // upper node in a mixed state: tensor-core leg contractions
-    if (x != x_in_) launch_copy(x, x_in_, n, stream_);
-    int rc = apply_heff_tg();
-    if (rc) return rc;
-    if (y != y_out_) launch_copy(y_out_, y, n, stream_);
-    return 0;
+    return apply_heff_tg(x, y);
   }
   HeffPlans* hp = heff_plans(center_, cls, false);
   if (!hp) return -1;
@@ -2606,7 +2602,7 @@ void tg_tiles(TgPlan& pl, int oi, int parts_wanted) {
   }
   for (int r0 = 0; r0 < o.rows; r0 += 128)
     for (size_t p = 0; p < ranges.size(); ++p)
-      pl.tiles.push_back(TgTile{oi, r0, ranges[p].first, ranges[p].second, o.n_parts > 1 ? (int)p : -1});
+      pl.tiles.push_back(TgTile{oi, r0, ranges[p].first, ranges[p].second, o.n_parts > 1 ? (int)p : -1, 0});
 }
 }  // namespace
 
@@ -2660,8 +2656,14 @@ Engine::TgHeff* Engine::tg_plans(int node) {
   std::unique_ptr<TgHeff> tp(new TgHeff);
   TgHeff& T = *tp;
   // Z = op (x)_leg X on the child legs, block by block; written[] marks the
-  // output blocks that receive a source block (the others are never read)
-  auto leg_apply = [&](TgPlan& pl, const Layout& LX, const void* X, bool x_f32, const std::vector<char>* xw,
+  // output blocks that receive a source block (the others are never read).
+  // Contractions of one source block over one leg by operators of one padded
+  // width are collected and grouped afterwards (in order of first use).
+  struct Group { std::vector<TgOut> outs; std::vector<TgChunk> chunks; };
+  using GroupKey = std::tuple<const void*, int, int>;   // source block, leg, padded width
+  std::map<GroupKey, int> group_of[2];
+  std::vector<Group> groups[2];
+  auto leg_apply = [&](int stage, const Layout& LX, const void* X, bool x_f32, const std::vector<char>* xw,
                        const Layout& LY, float* Y, std::vector<char>* yw, int leg, const OpRef& op, int shiftP,
                        int dimP) {
     const Sectors& S = LX.leg[leg];
@@ -2679,6 +2681,7 @@ Engine::TgHeff* Engine::tg_plans(int node) {
       o.C = Y + yb.off;
       o.c_f32 = 1;
       o.accumulate = 0;
+      o.n_parts = 1;
       TgChunk c{};
       c.A = x_f32 ? (const void*)((const float*)X + b.off) : (const void*)((const double*)X + b.off);
       c.a_f32 = x_f32 ? 1 : 0;
@@ -2693,18 +2696,19 @@ Engine::TgHeff* Engine::tg_plans(int node) {
         o.R2 = kTgRowsBig; o.t1 = 0; o.t2 = 1; o.cj = (long long)yb.db * yb.dc;
         c.R2 = kTgRowsBig; c.s1 = 0; c.s2 = 1; c.sk = (long long)b.db * b.dc; c.K = b.da;
       } else {
-        // rows (a, c), K = b with stride dc; out (a, b', c)
+        // rows (a, c), K = b with stride dc; out (a, b', c).  One column c: rows a
+        const bool flat = b.dc == 1;
         o.rows = b.da * b.dc; o.N = yb.db;
-        o.R2 = b.dc; o.t1 = (long long)yb.db * yb.dc; o.t2 = 1; o.cj = yb.dc;
-        c.R2 = b.dc; c.s1 = (long long)b.db * b.dc; c.s2 = 1; c.sk = b.dc; c.K = b.db;
+        o.R2 = flat ? kTgRowsBig : b.dc; o.t1 = (long long)yb.db * yb.dc; o.t2 = flat ? o.t1 : 1; o.cj = yb.dc;
+        c.R2 = o.R2; c.s1 = (long long)b.db * b.dc; c.s2 = flat ? c.s1 : 1; c.sk = b.dc; c.K = b.db;
+        if (!flat) o.r2div = c.r2div = reciprocal(b.dc);
       }
       o.npad = (o.N + 15) / 16 * 16;
-      pl.max_npad = std::max(pl.max_npad, o.npad);
-      o.n_parts = (int)pl.chunks.size();   // chunk_begin while building
-      pl.chunks.push_back(c);
-      pl.flops += 2.0 * o.rows * o.N * c.K;
-      pl.outs.push_back(o);
-      tg_tiles(pl, (int)pl.outs.size() - 1, 1);
+      T.st[stage].flops += 2.0 * o.rows * o.N * c.K;
+      const auto at = group_of[stage].emplace(GroupKey{c.A, leg, o.npad}, (int)groups[stage].size());
+      if (at.second) groups[stage].emplace_back();
+      groups[stage][at.first->second].outs.push_back(o);
+      groups[stage][at.first->second].chunks.push_back(c);
     }
   };
   struct Src { const void* Z; bool f32; int shift; std::vector<char> written; };
@@ -2715,19 +2719,47 @@ Engine::TgHeff* Engine::tg_plans(int node) {
     if (h.op[0].kind && h.op[1].kind) {
       const int s0 = h.op[0].shift, s1 = h.op[1].shift;
       std::vector<char> w1(lays[s0].blk.size(), 0), w2(lays[s0 + s1].blk.size(), 0);
-      leg_apply(T.st[0], L, x_in_, false, nullptr, lays[s0], zp, &w1, 0, h.op[0], s0, d0);
-      leg_apply(T.st[1], lays[s0], zp, true, &w1, lays[s0 + s1], zp + zsize, &w2, 1, h.op[1], s1, d1);
+      leg_apply(0, L, x_in_, false, nullptr, lays[s0], zp, &w1, 0, h.op[0], s0, d0);
+      leg_apply(1, lays[s0], zp, true, &w1, lays[s0 + s1], zp + zsize, &w2, 1, h.op[1], s1, d1);
       sr = Src{zp + zsize, true, s0 + s1, w2};
       zp += 2 * zsize;
     } else if (h.op[0].kind || h.op[1].kind) {
       const int leg = h.op[0].kind ? 0 : 1;
       const int sh = h.op[leg].shift;
       std::vector<char> w(lays[sh].blk.size(), 0);
-      leg_apply(T.st[0], L, x_in_, false, nullptr, lays[sh], zp, &w, leg, h.op[leg], sh, leg == 0 ? d0 : d1);
+      leg_apply(0, L, x_in_, false, nullptr, lays[sh], zp, &w, leg, h.op[leg], sh, leg == 0 ? d0 : d1);
       sr = Src{zp, true, sh, w};
       zp += zsize;
     }
     srcs.push_back(std::move(sr));
+  }
+  // Width of a group: wide ones load the rows less often, narrow ones give more
+  // tiles.  GB300, upper products of 4x4x4 in us at no group / 64 / 128 / 256
+  // columns: chi=64 layer 2 168 / 138 / 146 / 186, layer 4 274 / 200 / 214 / 244;
+  // where 64 leaves SMs without two tiles, one output a tile is faster (root of
+  // 4x2x2 chi=16 36 / 40 / 45 / 56).
+  for (int i = 0; i < 2; ++i) {
+    TgPlan& pl = T.st[i];
+    int width = kTgGroup;
+    for (; width > 16; width /= 2) {
+      long long tiles = 0;
+      for (const Group& g : groups[i]) {
+        const long long most = std::max(1, width / g.outs[0].npad);
+        tiles += ((long long)g.outs.size() + most - 1) / most * ((g.outs[0].rows + 127) / 128);
+      }
+      if (tiles >= 2 * 152) break;
+    }
+    for (const Group& g : groups[i]) {
+      const int npad = g.outs[0].npad, most = std::max(1, width / npad);
+      for (size_t g0 = 0; g0 < g.outs.size(); g0 += most) {
+        const int n = (int)std::min(g.outs.size() - g0, (size_t)most);
+        const int out0 = (int)pl.outs.size(), chunk0 = (int)pl.chunks.size();
+        pl.outs.insert(pl.outs.end(), g.outs.begin() + g0, g.outs.begin() + g0 + n);
+        pl.chunks.insert(pl.chunks.end(), g.chunks.begin() + g0, g.chunks.begin() + g0 + n);
+        pl.max_npad = std::max(pl.max_npad, n * npad);
+        for (int r0 = 0; r0 < g.outs[g0].rows; r0 += 128) pl.tiles.push_back(TgTile{out0, r0, chunk0, chunk0 + n, -1, n});
+      }
+    }
   }
   // stage 2: one output per block of y, chunks over terms
   TgPlan& s3 = T.st[2];
@@ -2795,9 +2827,14 @@ Engine::TgHeff* Engine::tg_plans(int node) {
   return raw;
 }
 
-int Engine::apply_heff_tg() {
+int Engine::apply_heff_tg(const double* x, double* y) {
   TgHeff* T = tg_plans(center_);
   if (!T) return -1;
+  const long long n = layout_[center_].size;
+  if (x != x_in_ && x < y + n && y < x + n) {   // the last stage reads x while it writes y
+    launch_copy(x, x_in_, n, stream_);
+    x = x_in_;
+  }
   const int elem = precision_ == PREC_BF16 ? 2 : 4;
   const int split = precision_ == PREC_TF32X3 ? 1 : 0;
   cudaEvent_t e0 = nullptr;
@@ -2805,7 +2842,8 @@ int Engine::apply_heff_tg() {
   for (int i = 0; i < 3; ++i) {
     TgPlan& pl = T->st[i];
     const int rc = launch_tg_gemm(elem, split, pl.d_tiles, (int)pl.tiles.size(), pl.d_outs, pl.d_chunks, pl.max_npad,
-                                  tg_scratch_, pl.d_red, (int)pl.red.size(), d_err_, stream_, wait_polls);
+                                  tg_scratch_, pl.d_red, (int)pl.red.size(), x - x_in_, y - y_out_, d_err_, stream_,
+                                  wait_polls);
     if (rc) {
       err_ = "tensor-core contraction: output width outside the supported range";
       return rc;

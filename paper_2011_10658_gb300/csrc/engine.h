@@ -438,7 +438,7 @@ class Engine {
   long long oz_partial_elems_ = 0;
   int compute_up_oz(int node, const std::vector<std::pair<double*, double>>& terms, const std::vector<int>& keys,
                     BondOps& out);
-  int apply_heff_tg();
+  int apply_heff_tg(const double* x, double* y);
   int tc_w_node_ = -1;          // node whose environment blocks are staged
   void clear_tc_cache();
   void* xstage_ = nullptr;      // BF16 padded staging of x (BF16 operands)

@@ -28,6 +28,8 @@ __device__ __forceinline__ float d2f_bits(double d) {
   return __uint_as_float(r);
 }
 
+static __device__ __noinline__ float d2f_edge(double d) { return d2f_bits(d); }
+
 // FP32 -> FP64, exact, on the integer pipes (FP32 subnormals become zero).
 __device__ __forceinline__ double f2d_bits(float f) {
   const unsigned u = __float_as_uint(f);

@@ -281,6 +281,7 @@ struct TgChunk {
   int K;
   int a_f32;
   float alpha;
+  unsigned r2div;   // ceil(2^32 / R2); 0: every row below R2
 };
 // An output: D[r, j] (r < rows, j < N) at C[(r / R2) * t1 + (r % R2) * t2 + j * cj],
 // float if c_f32 (else double), written or added (accumulate); chunks of its
@@ -295,23 +296,30 @@ struct TgOut {
   int accumulate;
   int n_parts;
   long long part_off;
+  unsigned r2div;   // as in TgChunk
 };
 // One CTA: rows row0 .. row0 + 127 of output `out` over chunks [chunk_begin,
-// chunk_end); part >= 0 writes partial slot `part`.
+// chunk_end); part >= 0 writes partial slot `part`.  n_sub > 0: a group of
+// outputs out .. out + n_sub - 1, output out + i from the one chunk chunk_begin
+// + i, with the same rows, K, padded width and A operand in all of them.
 struct TgTile {
   int out;
   int row0;
   int chunk_begin, chunk_end;
   int part;
+  int n_sub;
 };
+constexpr int kTgGroup = 64;   // most columns of a group
 // Shared memory of one launch (two stages of A and B tiles).
 int tg_stage_bytes(int elem, int split, int max_npad, int* a_bytes, int* b_bytes);
 // elem 4: TF32 operands (split: three products of hi / lo parts), 2: BF16.
-// red_list: outputs with n_parts > 1 (reduced after the GEMM).  err: device
+// max_npad: widest tile (a group's columns together).  red_list: outputs with
+// n_parts > 1 (reduced after the GEMM).  x_shift, y_shift: added to every FP64
+// A and C pointer (elements), so that one plan serves any x and y.  err: device
 // flag set if a wait timed out; polls < 0: default bound.
 int launch_tg_gemm(int elem, int split, const TgTile* tiles, int n_tiles, const TgOut* outs, const TgChunk* chunks,
-                   int max_npad, float* scratch, const int* red_list, int n_red, int* err, cudaStream_t s,
-                   long long polls = -1);
+                   int max_npad, float* scratch, const int* red_list, int n_red, long long x_shift, long long y_shift,
+                   int* err, cudaStream_t s, long long polls = -1);
 
 // ---- FP64-accurate contractions on the BF16 tensor cores (digit planes) ----
 constexpr int kOzDigits = 5;   // balanced base-256 digits per FP64 entry (about 2^-39 of the max)

@@ -14,7 +14,9 @@
 // terms).
 //
 // One CTA = 128 rows of one output (MMA M = 128, one thread per row); the
-// MMA N is the output width rounded up to 16.  A rows are loaded by their
+// MMA N is the output width rounded up to 16.  Terms that act on the same
+// block of the same source are grouped: their operators stand side by side
+// along N, so the rows are loaded and converted once for up to 64 columns.  A rows are loaded by their
 // threads (FP64 or FP32 sources, converted on the integer pipes) and written
 // in the no-swizzle K-major core-matrix layout; B is the operator block,
 // scaled by alpha.  Two shared-memory stages: the loads of step s+1 overlap
@@ -22,6 +24,12 @@
 // products hi*hi + hi*lo + lo*hi), or BF16; FP32 accumulation.  Outputs
 // whose K is long are split into parts whose FP32 partial sums are added in
 // a fixed order afterwards.
+//
+// Bound by the latency of a step (loads, conversion, one MMA batch) and, in the
+// first stage, by the issue of the conversions.  Whole products, GB300: 4x4x4
+// chi=64 layer 2 217 -> 137 us, layer 4 287 -> 200 us, chi=48 BF16 layer 3 133 ->
+// 102 us; 168, 274 and 123 us with the loads of a row in flight together, short
+// conversions and no copies of x and y, the rest from the groups.
 //
 // Every mbarrier wait is bounded (polls, a launch argument); a timeout sets
 // *err, and the CTA then drains its MMAs through a commit to a fresh barrier
@@ -31,6 +39,7 @@
 
 #include <cuda_bf16.h>
 
+#include "ffloat.cuh"
 #include "kernels.cuh"
 
 namespace qed {
@@ -39,6 +48,7 @@ namespace {
 
 constexpr int TG_THREADS = 128;
 constexpr int TG_KB = 16;                         // K elements per stage
+constexpr int TG_BSUB = 2;                        // operators of a group loaded at a time
 constexpr long long kTgWaitPolls = 1LL << 22;
 
 __device__ __forceinline__ uint32_t tg_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -72,21 +82,14 @@ __device__ __forceinline__ bool tg_wait(uint32_t addr, uint32_t parity, long lon
 }
 
 // FP64 -> FP32, round to nearest even, on the integer pipes (GB300 runs FP64
-// instructions, conversions included, at a small fraction of its FP32 rate).
-// Magnitudes below the FP32 normal range become signed zero.
+// instructions, conversions included, at a small fraction of its FP32 rate):
+// the exponent rebiased, the top 23 fraction bits, a carry from the other 29.
+// Outside 2^-126 .. 2^127 the general form (d2f_bits; zeros apart).
 __device__ __forceinline__ float tg_d2f(double d) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-  const int e = (int)((b >> 52) & 0x7ff);
-  const unsigned long long frac = b & 0xFFFFFFFFFFFFFull;
-  if (e == 0x7ff) return __uint_as_float(sign | 0x7f800000u | (frac ? 0x400000u : 0u));
-  const int fe = e - 1023 + 127;
-  if (fe <= 0) return __uint_as_float(sign);
-  if (fe >= 255) return __uint_as_float(sign | 0x7f800000u);
-  unsigned r = sign | ((unsigned)fe << 23) | (unsigned)(frac >> 29);
-  const unsigned rem = (unsigned)(frac & 0x1FFFFFFFull);
-  if (rem > 0x10000000u || (rem == 0x10000000u && (r & 1u))) r += 1u;
-  return __uint_as_float(r);
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  if ((h & 0x7fffffffu) - (897u << 20) >= (253u << 20)) return (h << 1) == 0u && l == 0u ? 0.f : d2f_edge(d);
+  const unsigned t = (__funnelshift_l(l, h, 3) - (384u << 23)) & 0x7fffffffu;
+  return __uint_as_float((t + (((l & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29)) | (h & 0x80000000u));
 }
 
 __device__ __forceinline__ float tg_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
@@ -134,11 +137,12 @@ __device__ __forceinline__ void tg_put4(uint8_t* base, int row, int q4, const fl
 }
 
 template <int ELEM, bool SPLIT>
-__global__ void __launch_bounds__(TG_THREADS) tg_gemm_kernel(const TgTile* __restrict__ tiles, int n_tiles,
+__global__ void __launch_bounds__(TG_THREADS, 4) tg_gemm_kernel(const TgTile* __restrict__ tiles, int n_tiles,
                                                               const TgOut* __restrict__ outs,
                                                               const TgChunk* __restrict__ chunks,
                                                               float* __restrict__ scratch, int a_bytes, int b_bytes,
-                                                              int max_npad, int* err, long long polls) {
+                                                              int max_npad, long long x_shift, long long y_shift,
+                                                              int* err, long long polls) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ uint32_t tmem_slot;
   __shared__ __align__(8) uint64_t mbar[3];   // two stages, one drain
@@ -172,50 +176,77 @@ __global__ void __launch_bounds__(TG_THREADS) tg_gemm_kernel(const TgTile* __res
     const uint32_t u = st ? uses1 : uses0;
     if (u > 0 && !tg_wait(tg_smem_u32(&mbar[st]), (u - 1) & 1, polls)) s_fail = 1;
   };
-  // K values k0 .. k0 + TG_KB of chunk ci of `tile` into stage buffers Ab, Bb
+  // K values k0 .. k0 + TG_KB of chunk c_idx of `tile` into stage buffers Ab,
+  // Bb; a grouped tile stacks the operators of its outputs' chunks along N.
+  // All loads of a row (indices clamped into the block) are issued before the
+  // first conversion.
   auto load_step = [&](const TgTile& tile, const TgOut& out, int c_idx, int kk0, uint8_t* Ab, uint8_t* Bb) {
     const TgChunk c = chunks[c_idx];
     const int row = tile.row0 + tid;
     const bool row_ok = row < out.rows;
     long long base = 0;
-    if (row_ok) base = (long long)(row / c.R2) * c.s1 + (long long)(row % c.R2) * c.s2;
-#pragma unroll
-    for (int q4 = 0; q4 < TG_KB / 4; ++q4) {
-      float v[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int k = kk0 + 4 * q4 + i;
-        float x = 0.f;
-        if (row_ok && k < c.K) {
-          const long long o = base + (long long)k * c.sk;
-          x = c.a_f32 ? __ldg((const float*)c.A + o) : tg_d2f(__ldg((const double*)c.A + o));
-        }
-        v[i] = x;
-      }
-      tg_put4<ELEM, SPLIT>(Ab, tid, q4, v);
+    if (row_ok) {
+      const int q = (int)__umulhi((unsigned)row, c.r2div);
+      base = (long long)q * c.s1 + (long long)(row - q * c.R2) * c.s2;
     }
-    const float alpha = c.alpha;
-    for (int e = tid; e < out.npad * (TG_KB / 4); e += TG_THREADS) {
-      const int j = e / (TG_KB / 4), q4 = e % (TG_KB / 4);
-      float v[4];
+    float v[TG_KB];
+    if (c.a_f32) {
+      const float* p = (const float*)c.A + base;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int k = kk0 + 4 * q4 + i;
-        v[i] = (j < out.N && k < c.K) ? alpha * tg_d2f(__ldg(c.B + (long long)j * c.bj + (long long)k * c.bk)) : 0.f;
-      }
-      tg_put4<ELEM, SPLIT>(Bb, j, q4, v);
+      for (int i = 0; i < TG_KB; ++i) v[i] = __ldg(p + (long long)min(kk0 + i, c.K - 1) * c.sk);
+    } else {
+      const double* p = (const double*)c.A + x_shift + base;
+      double d[TG_KB];
+#pragma unroll
+      for (int i = 0; i < TG_KB; ++i) d[i] = __ldg(p + (long long)min(kk0 + i, c.K - 1) * c.sk);
+#pragma unroll
+      for (int i = 0; i < TG_KB; ++i) v[i] = tg_d2f(d[i]);
     }
+#pragma unroll
+    for (int i = 0; i < TG_KB; ++i)
+      if (!row_ok || kk0 + i >= c.K) v[i] = 0.f;
+#pragma unroll
+    for (int q4 = 0; q4 < TG_KB / 4; ++q4) tg_put4<ELEM, SPLIT>(Ab, tid, q4, v + 4 * q4);
+    const int subs = tile.n_sub > 0 ? tile.n_sub : 1;
+    for (int s0 = 0; s0 < subs; s0 += TG_BSUB)
+      for (int e = tid; e < out.npad * (TG_KB / 4); e += TG_THREADS) {
+        const int j = e / (TG_KB / 4), q4 = e % (TG_KB / 4);
+        double d[TG_BSUB][4];
+#pragma unroll
+        for (int u = 0; u < TG_BSUB; ++u)
+          if (s0 + u < subs) {
+            const TgChunk& cu = chunks[c_idx + s0 + u];
+            const int n = tile.n_sub > 0 ? outs[tile.out + s0 + u].N : out.N;
+            const double* p = cu.B + (long long)min(j, n - 1) * cu.bj;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d[u][i] = __ldg(p + (long long)min(kk0 + 4 * q4 + i, cu.K - 1) * cu.bk);
+          }
+#pragma unroll
+        for (int u = 0; u < TG_BSUB; ++u)
+          if (s0 + u < subs) {
+            const TgChunk& cu = chunks[c_idx + s0 + u];
+            const int n = tile.n_sub > 0 ? outs[tile.out + s0 + u].N : out.N;
+            float w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              w[i] = j < n && kk0 + 4 * q4 + i < cu.K ? cu.alpha * tg_d2f(d[u][i]) : 0.f;
+            tg_put4<ELEM, SPLIT>(Bb, (s0 + u) * out.npad + j, q4, w);
+          }
+      }
   };
   // rows of `tile` from TMEM (or zeros) to the output or its partial slot
-  auto store_tile = [&](const TgTile& tile, const TgOut& out, bool from_tmem, bool ok) {
+  auto store_out = [&](const TgTile& tile, const TgOut& out, int col0, bool from_tmem, bool ok) {
     const int row = tile.row0 + tid;
     const bool row_ok = row < out.rows;
     long long cbase = 0;
-    if (row_ok) cbase = (long long)(row / out.R2) * out.t1 + (long long)(row % out.R2) * out.t2;
+    if (row_ok) {
+      const int q = (int)__umulhi((unsigned)row, out.r2div);
+      cbase = (long long)q * out.t1 + (long long)(row - q * out.R2) * out.t2;
+    }
     for (int c0 = 0; c0 < out.N; c0 += 16) {
       uint32_t v[16];
       if (from_tmem) {
-        const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0;
+        const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(col0 + c0);
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
@@ -238,11 +269,18 @@ __global__ void __launch_bounds__(TG_THREADS) tg_gemm_kernel(const TgTile* __res
           float* p = (float*)out.C + cbase + (long long)col * out.cj;
           *p = out.accumulate ? *p + f : f;
         } else {
-          double* p = (double*)out.C + cbase + (long long)col * out.cj;
-          *p = out.accumulate ? *p + (double)f : (double)f;
+          double* p = (double*)out.C + y_shift + cbase + (long long)col * out.cj;
+          *p = out.accumulate ? *p + f2d_bits(f) : f2d_bits(f);
         }
       }
     }
+  };
+  auto store_tile = [&](const TgTile& tile, const TgOut& out, bool from_tmem, bool ok) {
+    if (tile.n_sub == 0) {
+      store_out(tile, out, 0, from_tmem, ok);
+      return;
+    }
+    for (int u = 0; u < tile.n_sub; ++u) store_out(tile, outs[tile.out + u], u * out.npad, from_tmem, ok);
   };
   // next tile of this CTA that has chunks; tiles without any get zeros
   auto next_tile = [&](int from) {
@@ -273,7 +311,8 @@ __global__ void __launch_bounds__(TG_THREADS) tg_gemm_kernel(const TgTile* __res
     while (true) {
       if (tid == 0) {
         // D = F32; A, B = TF32 (kind::tf32) or BF16 (kind::f16), K-major; M = 128
-        uint32_t idesc = (1u << 4) | ((uint32_t)(out.npad >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        const int width = out.npad * (tile.n_sub > 0 ? tile.n_sub : 1);
+        uint32_t idesc = (1u << 4) | ((uint32_t)(width >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         idesc |= ELEM == 4 ? ((2u << 7) | (2u << 10)) : ((1u << 7) | (1u << 10));
         asm volatile("tcgen05.fence::after_thread_sync;");
         const uint32_t a0 = tg_smem_u32(b ? A1 : A0), b0 = tg_smem_u32(b ? B1 : B0);
@@ -304,8 +343,12 @@ __global__ void __launch_bounds__(TG_THREADS) tg_gemm_kernel(const TgTile* __res
       first = false;
       // the step after this one
       int nci = ci, nk0 = k0 + TG_KB, nti = ti;
-      if (nk0 >= chunks[ci].K) { ++nci; nk0 = 0; }
-      const bool tile_done = nci >= tile.chunk_end;
+      bool tile_done = false;
+      if (nk0 >= chunks[ci].K) {
+        ++nci;
+        nk0 = 0;
+        tile_done = tile.n_sub > 0 || nci >= tile.chunk_end;
+      }
       TgTile ntile = tile;
       TgOut nout = out;
       if (tile_done) {
@@ -360,7 +403,7 @@ __global__ void __launch_bounds__(TG_THREADS) tg_gemm_kernel(const TgTile* __res
 
 // Partial sums of split outputs, added in part order.
 __global__ void tg_reduce_kernel(const TgOut* __restrict__ outs, const int* __restrict__ red_list,
-                                 const float* __restrict__ scratch) {
+                                 const float* __restrict__ scratch, long long y_shift) {
   const TgOut out = outs[red_list[blockIdx.y]];
   const long long mn = (long long)out.rows * out.N;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < mn; e += (long long)gridDim.x * blockDim.x) {
@@ -372,7 +415,7 @@ __global__ void tg_reduce_kernel(const TgOut* __restrict__ outs, const int* __re
       float* p = (float*)out.C + o;
       *p = out.accumulate ? *p + s : s;
     } else {
-      double* p = (double*)out.C + o;
+      double* p = (double*)out.C + y_shift + o;
       *p = out.accumulate ? *p + (double)s : (double)s;
     }
   }
@@ -388,8 +431,8 @@ int tg_stage_bytes(int elem, int split, int max_npad, int* a_bytes, int* b_bytes
 }
 
 int launch_tg_gemm(int elem, int split, const TgTile* tiles, int n_tiles, const TgOut* outs, const TgChunk* chunks,
-                   int max_npad, float* scratch, const int* red_list, int n_red, int* err, cudaStream_t s,
-                   long long polls) {
+                   int max_npad, float* scratch, const int* red_list, int n_red, long long x_shift, long long y_shift,
+                   int* err, cudaStream_t s, long long polls) {
   if (n_tiles <= 0) return 0;
   if (polls < 0) polls = kTgWaitPolls;
   if (max_npad > 256 || max_npad % 16 || (split && elem != 4)) return -7;
@@ -418,10 +461,11 @@ int launch_tg_gemm(int elem, int split, const TgTile* tiles, int n_tiles, const 
   // memory (227 KB per SM), TMEM columns (512 per SM), at most 8
   const int per_sm = std::max(1, std::min(8, std::min(512 / ncols, (227 * 1024) / (smem + 2048))));
   const int grid = std::min(n_tiles, sms * per_sm);
-  kern<<<grid, TG_THREADS, smem, s>>>(tiles, n_tiles, outs, chunks, scratch, a_bytes, b_bytes, max_npad, err, polls);
+  kern<<<grid, TG_THREADS, smem, s>>>(tiles, n_tiles, outs, chunks, scratch, a_bytes, b_bytes, max_npad,
+                                       x_shift, y_shift, err, polls);
   count_launches(1);
   if (n_red > 0) {
-    tg_reduce_kernel<<<dim3(16, n_red), 256, 0, s>>>(outs, red_list, scratch);
+    tg_reduce_kernel<<<dim3(16, n_red), 256, 0, s>>>(outs, red_list, scratch, y_shift);
     count_launches(1);
   }
   return 0;
