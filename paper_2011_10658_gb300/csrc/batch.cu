@@ -246,6 +246,11 @@ int BatchRunner::product(int node, const std::vector<int>& active) {
     g = ng.get();
     cur_[node] = std::move(ng);
   }
+  // a plan kept from an earlier sweep: the environment blocks are those of this
+  // visit only after they are staged again
+  if (g->tc)
+    for (int m : g->members)
+      if (!es_[m]->tc_prepare()) return -1;
   Engine* e0 = es_[g->members[0]];
   cudaStream_t s = e0->stream_;
   if (g->exec && g->scratch != e0->scratch_) {
