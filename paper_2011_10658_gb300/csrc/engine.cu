@@ -166,29 +166,32 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
   v.chunks.reserve(chunks.size());
   v.outs = outs;
   v.scratch_need = 0;
-  // K per part: small enough that the launch has about eight tiles per SM
+  // K per part: small enough that the launch has about sixteen tiles per SM
   // when the plan has few, long contractions (a Gram matrix), at most k_part.
-  // A slab of 16 is one trip to L2, so long sums are cut down to 192 (GB300,
-  // 4x4x4: centre move chi=64 15.6 ms at 4 tiles and 256, 14.7 ms at 8 and 192,
-  // 14.4 ms at 16 and 128, where the short sums of an upper-node update at
-  // chi=32 lose more to the reduction: 8.4, 8.5, 9.0 ms)
+  // A slab of 16 is one trip to L2, so long sums are cut down to 192; parts of
+  // 128 cost an upper-node update more in the reduction than they save, and
+  // with 4 tiles per SM and parts of 256 the operator updates of a centre move
+  // ran 1.06 times as long (GB300, 4x4x4 chi=64).
   long long work = 0, base_tiles = 0;
+  // length of a chunk in the sum: whole slabs of 16 (a term that is only added
+  // is one trip to L2 as well: 160 of them in one sum took 280 us)
+  auto slabs = [](const KChunk& c) { return c.add ? 16 : (c.K + 15) / 16 * 16; };
   for (const KOutput& o : outs) {
     long long ktot = 0;
-    for (int c = o.chunk_begin; c < o.chunk_end; ++c) ktot += chunks[c].add ? 1 : chunks[c].K;
+    for (int c = o.chunk_begin; c < o.chunk_end; ++c) ktot += slabs(chunks[c]);
     const long long t = (long long)((o.M + BMs - 1) / BMs) * ((o.N + BNs - 1) / BNs);
     work += t * ktot;
     base_tiles += t;
   }
-  const long long kp = std::max(192LL, std::min(k_part, work / (8 * 152)));
-  const bool few_tiles = base_tiles < 8 * 152;
+  const long long kp = std::max(192LL, std::min(k_part, work / (16 * 152)));
+  const bool few_tiles = base_tiles < 16 * 152;
   std::vector<KChunk>& nc = v.chunks;
   for (size_t oi = 0; oi < outs.size(); ++oi) {
     KOutput& o = v.outs[oi];
     const KOutput& mo = outs[oi];
     const int tm = (o.M + BMs - 1) / BMs, tn = (o.N + BNs - 1) / BNs;
     long long ktot = 0;
-    for (int c = mo.chunk_begin; c < mo.chunk_end; ++c) ktot += chunks[c].add ? 1 : chunks[c].K;
+    for (int c = mo.chunk_begin; c < mo.chunk_end; ++c) ktot += slabs(chunks[c]);
     const bool split = ktot > 2 * kp && (tm * tn <= 16 || few_tiles);
     std::vector<std::pair<int, int>> parts;   // ranges in nc
     const int begin = (int)nc.size();
@@ -202,7 +205,12 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
         const KChunk& ch = chunks[c];
         if (ch.add) {
           nc.push_back(ch);
-          acc += 1;
+          acc += slabs(ch);
+          if (acc >= kp) {
+            parts.push_back({part_begin, (int)nc.size()});
+            part_begin = (int)nc.size();
+            acc = 0;
+          }
         } else {
           // a two-level K is cut between its inner runs
           const int step = ch.kin ? std::max(ch.kin, (int)kp / ch.kin * ch.kin) : (int)kp;
@@ -217,7 +225,7 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
             }
             sc.A = ch.A + (ch.kin ? (long long)(k0 / ch.kin) * ch.a_ko : (long long)k0 * ch.a_k);
             nc.push_back(sc);
-            acc += sc.K;
+            acc += slabs(sc);
             if (acc >= kp) {
               parts.push_back({part_begin, (int)nc.size()});
               part_begin = (int)nc.size();

@@ -86,11 +86,13 @@ __device__ __forceinline__ double lz_block_sum(A v, double* red) {
   return r;
 }
 
-// Sum of one value per block, in block order by lanes; valid in every thread.
-__device__ __forceinline__ double lz_grid_sum(const double* part, double* red) {
+// Sum of `count` values (one per block), in block order by lanes; valid in
+// every thread.
+__device__ __forceinline__ double lz_grid_sum(const double* part, int count, double* red) {
   if (threadIdx.x < 32) {
     double v = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) v += __ldcg(part + i);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < count; i += 32) v += __ldcg(part + i);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (threadIdx.x == 0) red[0] = v;
   }
@@ -209,6 +211,167 @@ __device__ __forceinline__ A lz_update(const LzStep& p, const double* c, A* cs, 
   return nrm;
 }
 
+// The last block to leave zeroes the counters for the next launch.
+__device__ __forceinline__ void lz_leave(const LzStep& p, double alpha, double nrm2) {
+  if (threadIdx.x == 0) {
+    if (blockIdx.x == 0) {
+      *p.alpha_j = alpha;
+      *p.beta_j = sqrt(fmax(nrm2, 0.0));
+    }
+    if (atomicAdd(p.bar + 1, 1u) == gridDim.x - 1) {
+      p.bar[0] = 0u;
+      p.bar[1] = 0u;
+    }
+  }
+}
+
+// ---- short vectors: the basis columns are shared out as well
+// (a step at n = 5104 with 1-46 vectors: 25-55 us in the long form, 22 here)
+// Block (rb, cg) of row_blocks x column_groups: rows rb * 256 .., column sweeps
+// cg, cg + column_groups, ..  A short vector leaves a thread a row or two, so
+// the time is the number of trips to L2 one after another; here a dot phase is
+// one sweep per block, and four lanes share a row of an update.
+// part[rb * (k + 1) + col]; `w` gives w' (or y) of a row.
+template <typename A, typename Row>
+__device__ __forceinline__ void lz_short_dots(const LzStep& p, int rb, int row_blocks, int cg, int column_groups,
+                                              double (*sh)[LZ_COLS], Row row) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int g = cg * LZ_COLS; g <= p.k; g += column_groups * LZ_COLS) {
+    A acc[LZ_COLS];
+#pragma unroll
+    for (int t = 0; t < LZ_COLS; ++t) acc[t] = A(0);
+    for (long long i = (long long)rb * LZ_THREADS + threadIdx.x; i < p.n; i += (long long)row_blocks * LZ_THREADS) {
+      double v[LZ_COLS];
+#pragma unroll
+      for (int t = 0; t < LZ_COLS; ++t) v[t] = g + t < p.k ? __ldg(p.V + (long long)(g + t) * p.ldq + i) : 0.0;
+      const A ya = lz_in<A>(row(i));
+#pragma unroll
+      for (int t = 0; t < LZ_COLS; ++t) {
+        if (g + t < p.k) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
+        else if (g + t == p.k) acc[t] = kc_fma(ya, ya, acc[t]);
+      }
+    }
+#pragma unroll
+    for (int h = LZ_COLS / 2, m = 16; h >= 1; h >>= 1, m >>= 1)
+#pragma unroll
+      for (int t = 0; t < h; ++t) {
+        const bool up = (lane & m) != 0;
+        const A keep = up ? acc[t + h] : acc[t];
+        const A give = up ? acc[t] : acc[t + h];
+        acc[t] = keep + lz_xor(give, m);
+      }
+    A r = acc[0];
+    r = r + lz_xor(r, 2);
+    r = r + lz_xor(r, 1);
+    if ((lane & 3) == 0) sh[warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = to_d<A>(r);
+    __syncthreads();
+    if (threadIdx.x < LZ_COLS && g + (int)threadIdx.x <= p.k) {
+      double v = 0.0;
+#pragma unroll
+      for (int u = 0; u < LZ_WARPS; ++u) v += sh[u][threadIdx.x];
+      __stcg(p.partial + (long long)rb * (p.k + 1) + g + threadIdx.x, v);
+    }
+    __syncthreads();
+  }
+}
+
+// c[col] = sum over the row blocks, one thread a column, in every block.
+__device__ __forceinline__ void lz_short_columns(const LzStep& p, int ncol, int row_blocks, double* c) {
+  if ((int)threadIdx.x < ncol) {
+    double v = 0.0;
+#pragma unroll 8
+    for (int b = 0; b < row_blocks; ++b) v += __ldcg(p.partial + (long long)b * (p.k + 1) + threadIdx.x);
+    c[threadIdx.x] = v;
+  }
+  __syncthreads();
+}
+
+// y = row - V c by quads of lanes; returns this thread's part of |y|^2.
+template <typename A, typename Row>
+__device__ __forceinline__ A lz_short_update(const LzStep& p, const double* c, A* cs, Row row) {
+  for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = lz_in<A>(-c[j]);
+  __syncthreads();
+  const int sub = threadIdx.x & 3;
+  const long long quads = (long long)gridDim.x * (LZ_THREADS / 4);
+  A nrm = A(0);
+  for (long long i0 = 0; i0 < p.n; i0 += quads) {   // uniform trip count: the quads exchange below
+    const long long i = i0 + blockIdx.x * (LZ_THREADS / 4) + (threadIdx.x >> 2);
+    const bool in = i < p.n;
+    const double* q = p.V + (in ? i : 0);
+    A v = A(0);
+    for (int j = sub; j < p.k; j += 32) {
+      double x[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) x[t] = j + 4 * t < p.k ? __ldg(q + (long long)(j + 4 * t) * p.ldq) : 0.0;
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (j + 4 * t < p.k) v = kc_fma(cs[j + 4 * t], lz_in<A>(x[t]), v);
+    }
+    v = v + lz_xor(v, 1);
+    v = v + lz_xor(v, 2);
+    if (in && sub == 0) {
+      v = lz_in<A>(row(i)) + v;
+      p.y[i] = to_d<A>(v);
+      nrm = kc_fma(v, v, nrm);
+    }
+  }
+  return nrm;
+}
+
+template <bool FF>
+__global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int row_blocks, int column_groups) {
+  using A = typename std::conditional<FF, ff, double>::type;
+  __shared__ double sh[LZ_WARPS][LZ_COLS];
+  __shared__ double c[LZ_MAX_K + 4];
+  __shared__ A cs[LZ_MAX_K];
+  double* red = &sh[0][0];
+  unsigned round = 0;
+  const int rb = blockIdx.x % row_blocks, cg = blockIdx.x / row_blocks;
+  const double* vj = p.V + (long long)(p.k - 1) * p.ldq;
+  const double* vp = vj - p.ldq;
+  double* part_a = p.partial + (long long)(LZ_MAX_K + 1) * row_blocks;
+  double* part_b = part_a + gridDim.x;
+  if (cg == 0) {
+    double a = 0.0;
+    for (long long i = (long long)rb * LZ_THREADS + threadIdx.x; i < p.n; i += (long long)row_blocks * LZ_THREADS)
+      a = fma(__ldg(vj + i), __ldcg(p.y + i), a);
+    a = lz_block_sum<double>(a, red);
+    if (threadIdx.x == 0) __stcg(part_a + rb, a);
+  }
+  grid_sync(p.bar, round, p.err);
+  const double alpha = lz_grid_sum(part_a, row_blocks, red);
+  const double beta = p.k >= 2 ? *p.beta_prev : 0.0;
+  // w' of a row, formed wherever it is needed: y is written in the update only
+  auto residual = [&](long long i) {
+    double v = fma(-alpha, __ldg(vj + i), __ldcg(p.y + i));
+    return p.k >= 2 ? fma(-beta, __ldg(vp + i), v) : v;
+  };
+  lz_short_dots<A>(p, rb, row_blocks, cg, column_groups, sh, residual);
+  grid_sync(p.bar, round, p.err);
+  lz_short_columns(p, p.k + 1, row_blocks, c);
+  const double before = c[p.k];
+  A t = lz_short_update<A>(p, c, cs, residual);
+  double s = lz_block_sum<A>(t, red);
+  if (threadIdx.x == 0) __stcg(part_b + blockIdx.x, s);
+  grid_sync(p.bar, round, p.err);
+  double nrm2 = lz_grid_sum(part_b, gridDim.x, red);
+  if (nrm2 < p.ratio * before) {
+    auto plain = [&](long long i) { return __ldcg(p.y + i); };
+    lz_short_dots<A>(p, rb, row_blocks, cg, column_groups, sh, plain);
+    grid_sync(p.bar, round, p.err);
+    lz_short_columns(p, p.k, row_blocks, c);
+    t = lz_short_update<A>(p, c, cs, plain);
+    s = lz_block_sum<A>(t, red);
+    if (threadIdx.x == 0) __stcg(part_a + blockIdx.x, s);
+    grid_sync(p.bar, round, p.err);
+    nrm2 = lz_grid_sum(part_a, gridDim.x, red);
+  }
+  const double inv = 1.0 / sqrt(nrm2);
+  for (long long i = blockIdx.x * (long long)LZ_THREADS + threadIdx.x; i < p.n; i += (long long)gridDim.x * LZ_THREADS)
+    p.v_next[i] = __ldcg(p.y + i) * inv;
+  lz_leave(p, alpha, nrm2);
+}
+
 template <bool FF>
 __global__ void __launch_bounds__(LZ_THREADS, 3) lz_step_kernel(LzStep p) {
   using A = typename std::conditional<FF, ff, double>::type;
@@ -230,7 +393,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_step_kernel(LzStep p) {
   a = lz_block_sum<double>(a, red);
   if (threadIdx.x == 0) __stcg(part_a + blockIdx.x, a);
   grid_sync(p.bar, round, p.err);
-  const double alpha = lz_grid_sum(part_a, red);
+  const double alpha = lz_grid_sum(part_a, gridDim.x, red);
   // w' = y - alpha_j v_j - beta_{j-1} v_{j-1}
   const double beta = p.k >= 2 ? *p.beta_prev : 0.0;
   for (long long i = i0; i < p.n; i += step) {
@@ -246,7 +409,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_step_kernel(LzStep p) {
   double s = lz_block_sum<A>(t, red);
   if (threadIdx.x == 0) __stcg(part_b + blockIdx.x, s);
   grid_sync(p.bar, round, p.err);
-  double nrm2 = lz_grid_sum(part_b, red);
+  double nrm2 = lz_grid_sum(part_b, gridDim.x, red);
   if (nrm2 < p.ratio * before) {
     lz_dots<A>(p, sh, i0, step);
     grid_sync(p.bar, round, p.err);
@@ -255,32 +418,24 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_step_kernel(LzStep p) {
     s = lz_block_sum<A>(t, red);
     if (threadIdx.x == 0) __stcg(part_a + blockIdx.x, s);
     grid_sync(p.bar, round, p.err);
-    nrm2 = lz_grid_sum(part_a, red);
+    nrm2 = lz_grid_sum(part_a, gridDim.x, red);
   }
   const double inv = 1.0 / sqrt(nrm2);
   for (long long i = i0; i < p.n; i += step) p.v_next[i] = p.y[i] * inv;
-  if (threadIdx.x == 0) {
-    if (blockIdx.x == 0) {
-      *p.alpha_j = alpha;
-      *p.beta_j = sqrt(fmax(nrm2, 0.0));
-    }
-    // the last block to leave zeroes the counters for the next launch
-    if (atomicAdd(p.bar + 1, 1u) == gridDim.x - 1) {
-      p.bar[0] = 0u;
-      p.bar[1] = 0u;
-    }
-  }
+  lz_leave(p, alpha, nrm2);
 }
 
 }  // namespace
 
-// Blocks: two rows a thread while that leaves SMs idle (small problems are
-// latency-bound), the resident maximum for large ones.
+// Vectors of up to 16384 rows: a row per thread in the dots, the column sweeps
+// on further blocks.  Longer ones: two rows a thread up to the resident maximum.
 int launch_lz_step(const LzStep& p, int ff_arith, cudaStream_t s) {
   if (p.k < 1 || p.k > LZ_MAX_K) return -7;
-  auto kern = ff_arith ? lz_step_kernel<true> : lz_step_kernel<false>;
-  static int resident[2] = {0, 0};
-  int& cap = resident[ff_arith ? 1 : 0];
+  const bool is_short = p.n <= 64 * LZ_THREADS;
+  const void* kern = is_short ? (ff_arith ? (const void*)lz_short_kernel<true> : (const void*)lz_short_kernel<false>)
+                              : (ff_arith ? (const void*)lz_step_kernel<true> : (const void*)lz_step_kernel<false>);
+  static int resident[4] = {0, 0, 0, 0};
+  int& cap = resident[(ff_arith ? 1 : 0) + (is_short ? 2 : 0)];
   if (!cap) {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
@@ -288,12 +443,13 @@ int launch_lz_step(const LzStep& p, int ff_arith, cudaStream_t s) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, LZ_THREADS, 0);
     cap = std::max(1, std::min(kLzMaxBlocks, std::min(3, per) * sms));
   }
-  const long long want = (p.n + 2 * LZ_THREADS - 1) / (2 * LZ_THREADS);
-  const int blocks = (int)std::max(1LL, std::min<long long>(cap, want));
   LzStep arg = p;
-  void* args[] = {&arg};
-  if (cudaLaunchCooperativeKernel((const void*)kern, dim3(blocks), dim3(LZ_THREADS), args, 0, s) != cudaSuccess)
-    return -3;
+  int row_blocks = (int)std::min<long long>(std::min(64, cap), (p.n + LZ_THREADS - 1) / LZ_THREADS);
+  int column_groups = std::max(1, std::min(cap / row_blocks, (p.k + LZ_COLS) / LZ_COLS));
+  const long long want = (p.n + 2 * LZ_THREADS - 1) / (2 * LZ_THREADS);
+  const int blocks = is_short ? row_blocks * column_groups : (int)std::max(1LL, std::min<long long>(cap, want));
+  void* args[] = {&arg, &row_blocks, &column_groups};
+  if (cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(LZ_THREADS), args, 0, s) != cudaSuccess) return -3;
   count_launches(1);
   return 0;
 }
