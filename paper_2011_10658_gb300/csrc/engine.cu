@@ -778,8 +778,12 @@ Engine::Engine(const Params& p, int chi, uint64_t seed, int precision, cudaStrea
     cudaEventCreateWithFlags(&ev_conv_[i], cudaEventDisableTiming);
   }
   ring_dev_ = (double*)dalloc(4 * (kMaxKrylov + 1) * sizeof(double));
-  if (!check(cudaMallocHost(&ring_host_, 4 * (kMaxKrylov + 1) * sizeof(double)), "pinned ring"))
+  size_t sectors = 2;   // of a site; of the widest bond below
+  for (const Sectors& b : bonds_) sectors = std::max(sectors, b.q.size());
+  if (!check(cudaMallocHost(&ring_host_, 4 * (kMaxKrylov + 1) * sizeof(double) + sectors * sizeof(int)), "pinned ring"))
     throw std::runtime_error(err_);
+  qr_status_ = (int*)(ring_host_ + 4 * (kMaxKrylov + 1));
+  if (!check(cudaEventCreateWithFlags(&ev_qr_, cudaEventDisableTiming), "QR event")) throw std::runtime_error(err_);
   cudaMemsetAsync(d_err_, 0, 8 * sizeof(int), stream_);
   long long dmax = 1;
   for (const Sectors& b : bonds_) dmax = std::max<long long>(dmax, b.total());
@@ -829,6 +833,7 @@ Engine::~Engine() {
     if (ev_iter_[i]) cudaEventDestroy(ev_iter_[i]);
     if (ev_conv_[i]) cudaEventDestroy(ev_conv_[i]);
   }
+  if (ev_qr_) cudaEventDestroy(ev_qr_);
   if (ring_host_) cudaFreeHost(ring_host_);
   for (void* p : allocs_) cudaFree(p);
 }
@@ -1209,11 +1214,17 @@ int Engine::qr_toward(int node, int leg, double* Rout) {
     if (rc) break;
     cudaMemsetAsync(Rinv, 0, dd * sizeof(double), stream_);
     launch_cholesky_inv(Gb, Rinv, d.off, d.n, d.ld, d.count, d.max_n, kQrFallback * kQrFallback, d.status, stream_);
-    std::vector<int> status(d.count);
-    cudaMemcpyAsync(status.data(), d.status, d.count * sizeof(int), cudaMemcpyDeviceToHost, stream_);
-    if (!check(cudaStreamSynchronize(stream_), "cholesky")) { rc = -3; break; }
-    for (int st : status)
-      if (st) fallback = true;
+    cudaMemcpyAsync(qr_status_, d.status, d.count * sizeof(int), cudaMemcpyDeviceToHost, stream_);
+    cudaEventRecord(ev_qr_, stream_);
+    // Q = X R^{-1} into the move buffer before the status is known: the GPU
+    // works on while the host waits, and an ill-conditioned sector leaves T
+    // as it was
+    cudaMemsetAsync(tmp_, 0, L.size * sizeof(double), stream_);
+    rc = launch_plan(apply);
+    if (rc) break;
+    if (!check(cudaEventSynchronize(ev_qr_), "cholesky")) { rc = -3; break; }
+    for (int i = 0; i < d.count; ++i)
+      if (qr_status_[i]) fallback = true;
     if (fallback) {
       if (pass == 0) break;
       // a second pass of a well-conditioned first pass cannot be ill-conditioned
@@ -1221,10 +1232,7 @@ int Engine::qr_toward(int node, int leg, double* Rout) {
       rc = -5;
       break;
     }
-    // T <- T (x)_leg Rinv^T  (Q = X R^{-1})
-    cudaMemsetAsync(tmp_, 0, L.size * sizeof(double), stream_);
-    rc = launch_plan(apply);
-    if (rc) break;
+    // T <- T (x)_leg Rinv^T
     launch_copy(tmp_, T, L.size, stream_);
     // R accumulation: Racc = R_pass * Racc (R of this pass in Gb, upper)
     if (pass == 0) {
@@ -1380,6 +1388,29 @@ int Engine::absorb(int node, int leg, const double* R) {
 
 // ------------------------------------------------------------------ bond operators
 
+// Storage of the operators of the bond above `node` (either direction): the
+// class Hamiltonians, their sum, and one operator per term that crosses it.
+void Engine::bond_slab(BondOps& out, int node, long long dd) {
+  if (out.slab) return;
+  long long n = N_CLASSES + 1;
+  for (int k = 0; k < (int)terms_.size(); ++k) n += crosses(k, node);
+  out.slab_elems = n * dd;
+  out.slab = (double*)dalloc(out.slab_elems * sizeof(double));
+  for (int c = 0; c < N_CLASSES; ++c) out.H[c] = out.slab + c * dd;
+  out.Htot = out.slab + N_CLASSES * dd;
+}
+
+double* Engine::bond_term(BondOps& out, int key, int shift, long long dd) {
+  auto it = out.term.find(key);
+  if (it == out.term.end()) {
+    BondOp b;
+    b.ptr = out.slab + (N_CLASSES + 1 + (long long)out.term.size()) * dd;
+    it = out.term.emplace(key, b).first;
+  }
+  it->second.shift = shift;
+  return it->second.ptr;
+}
+
 // Renormalized operators of the bond above `node` (subtree side), from
 // T[node] (isometric towards its parent) and the operators below it.
 int Engine::compute_up(int node) {
@@ -1390,20 +1421,8 @@ int Engine::compute_up(int node) {
   BondOps& out = up_[node];
   const bool bottom = nd.child_kind[0] == 0;
   const double* T = T_[node];
-  auto op_ptr = [&](int key, int shift) -> double* {
-    auto it = out.term.find(key);
-    if (it == out.term.end()) {
-      BondOp b;
-      b.ptr = (double*)dalloc(dd * sizeof(double));
-      b.shift = shift;
-      it = out.term.emplace(key, b).first;
-    }
-    it->second.shift = shift;
-    return it->second.ptr;
-  };
-  for (int c = 0; c < N_CLASSES; ++c)
-    if (!out.H[c]) out.H[c] = (double*)dalloc(dd * sizeof(double));
-  if (!out.Htot) out.Htot = (double*)dalloc(dd * sizeof(double));
+  bond_slab(out, node, dd);
+  auto op_ptr = [&](int key, int shift) { return bond_term(out, key, shift, dd); };
   // Contributions: (output matrix, alpha, op on leg 0, op on leg 1) where an
   // op is identified by (term or site-ham), shift.
   struct Contrib { double* O; double alpha; int term; int kind; int cls; };
@@ -1431,8 +1450,7 @@ int Engine::compute_up(int node) {
       if (tl && tr) cs.push_back({out.H[terms_[k].cls], terms_[k].coef, k, 1, terms_[k].cls});
     }
   }
-  for (int c = 0; c < N_CLASSES; ++c) cudaMemsetAsync(out.H[c], 0, dd * sizeof(double), stream_);
-  for (auto& kv : out.term) cudaMemsetAsync(kv.second.ptr, 0, dd * sizeof(double), stream_);
+  cudaMemsetAsync(out.slab, 0, out.slab_elems * sizeof(double), stream_);
   int rc = 0;
   int max_sector = 0;
   for (int d : L.leg[2].dim) max_sector = std::max(max_sector, d);
@@ -1532,8 +1550,7 @@ int Engine::compute_up(int node) {
     }
   }
   // Htot = sum of classes
-  cudaMemsetAsync(out.Htot, 0, dd * sizeof(double), stream_);
-  for (int c = 0; c < N_CLASSES; ++c) launch_add_scaled(out.H[c], out.Htot, dd, 1.0, stream_);
+  launch_sum_rows(out.slab, dd, N_CLASSES, out.Htot, stream_);
   return rc;
 }
 
@@ -1737,24 +1754,13 @@ int Engine::compute_down(int node) {
   const int dim = L.leg[leg].total();
   const long long dd = (long long)dim * dim;
   BondOps& out = down_[node];
-  for (int c = 0; c < N_CLASSES; ++c)
-    if (!out.H[c]) out.H[c] = (double*)dalloc(dd * sizeof(double));
-  if (!out.Htot) out.Htot = (double*)dalloc(dd * sizeof(double));
+  bond_slab(out, node, dd);
   std::vector<char> comp_par(lat_.n_sites(), 1);
   for (int s : pn.sites) comp_par[s] = 0;
   const bool par_root = pn.parent < 0;
   struct Job { double* O; double alpha; const double* S; int shS; const double* P; int shP; };
   std::vector<Job> jobs;
-  auto op_ptr = [&](int key, int shift) -> double* {
-    auto it = out.term.find(key);
-    if (it == out.term.end()) {
-      BondOp b;
-      b.ptr = (double*)dalloc(dd * sizeof(double));
-      it = out.term.emplace(key, b).first;
-    }
-    it->second.shift = shift;
-    return it->second.ptr;
-  };
+  auto op_ptr = [&](int key, int shift) { return bond_term(out, key, shift, dd); };
   for (int k = 0; k < (int)terms_.size(); ++k) {
     const bool ts = sib >= 0 ? touches(k, sib) : false;
     const bool tp = touches_sites(k, comp_par);
@@ -1776,8 +1782,7 @@ int Engine::compute_down(int node) {
     jobs.push_back({out.H[cl], 1.0, up_[sib].H[cl], 0, nullptr, 0});
     if (!par_root) jobs.push_back({out.H[cl], 1.0, nullptr, 0, down_[par].H[cl], 0});
   }
-  for (int c = 0; c < N_CLASSES; ++c) cudaMemsetAsync(out.H[c], 0, dd * sizeof(double), stream_);
-  for (auto& kv : out.term) cudaMemsetAsync(kv.second.ptr, 0, dd * sizeof(double), stream_);
+  cudaMemsetAsync(out.slab, 0, out.slab_elems * sizeof(double), stream_);
   long long zsize = 0;
   std::map<int, Layout> lays;
   for (int s = -2; s <= 2; ++s) {
@@ -1820,8 +1825,7 @@ int Engine::compute_down(int node) {
     });
     for (int i = 0; i < 3 && rc == 0; ++i) rc = launch_plan(st[i], ops_mode());
   }
-  cudaMemsetAsync(out.Htot, 0, dd * sizeof(double), stream_);
-  for (int c = 0; c < N_CLASSES; ++c) launch_add_scaled(out.H[c], out.Htot, dd, 1.0, stream_);
+  launch_sum_rows(out.slab, dd, N_CLASSES, out.Htot, stream_);
   return rc;
 }
 

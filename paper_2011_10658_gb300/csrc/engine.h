@@ -140,7 +140,11 @@ struct BondOp {
   int shift = 0;
 };
 
+// One allocation holds the class Hamiltonians, their sum and the term
+// operators, so that an update clears them in one go.
 struct BondOps {
+  double* slab = nullptr;
+  long long slab_elems = 0;
   std::unordered_map<int, BondOp> term;
   double* H[N_CLASSES] = {};
   double* Htot = nullptr;
@@ -414,6 +418,8 @@ class Engine {
     int max_n = 0;
   };
   std::map<std::pair<int, int>, QrDesc> qr_desc_;
+  int* qr_status_ = nullptr;      // pinned: factorisation status per sector
+  cudaEvent_t ev_qr_ = nullptr;
   // mixed-precision state: per-node plans; the staging buffers are shared
   // and the environment blocks are re-staged when the centre changes
   std::map<int, std::unique_ptr<TcPlan>> tc_cache_;
@@ -504,6 +510,8 @@ class Engine {
   int qr_toward(int node, int leg, double* Rout);
   int qr_gram_schmidt(int node, int leg, double* Rout);
   int absorb(int node, int leg, const double* R);
+  void bond_slab(BondOps& out, int node, long long dd);
+  double* bond_term(BondOps& out, int key, int shift, long long dd);
   int compute_up(int node);
   int compute_down(int node);
   const std::vector<RowMap>& rowmap(int node, int term);

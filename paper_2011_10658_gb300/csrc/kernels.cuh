@@ -167,6 +167,8 @@ void launch_scale_inv_sqrt(const double* x, double* y, long long n, const double
 void launch_copy(const double* x, double* y, long long n, cudaStream_t s);
 void launch_fill_uniform(double* x, long long n, uint64_t seed, uint64_t start, cudaStream_t s);
 void launch_add_scaled(const double* x, double* y, long long n, double a, cudaStream_t s);
+// y[i] = sum over r < rows of x[r * n + i]
+void launch_sum_rows(const double* x, long long n, int rows, double* y, cudaStream_t s);
 void launch_zero(double* x, long long n, cudaStream_t s);
 void launch_to_float(const double* x, float* y, long long n, cudaStream_t s);
 // *flag = 1 if any of x[0..n) is NaN or infinite (flag untouched otherwise).

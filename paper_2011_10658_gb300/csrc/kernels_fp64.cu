@@ -217,6 +217,15 @@ __global__ void add_scaled_kernel(const double* __restrict__ x, double* __restri
     y[i] = fma(a, x[i], y[i]);
 }
 
+// y[i] = sum of x[r * n + i] over the rows r.
+__global__ void sum_rows_kernel(const double* __restrict__ x, long long n, int rows, double* __restrict__ y) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    double v = 0.0;
+    for (int r = 0; r < rows; ++r) v += x[r * n + i];
+    y[i] = v;
+  }
+}
+
 __global__ void zero_kernel(double* __restrict__ x, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     x[i] = 0.0;
@@ -935,6 +944,11 @@ void launch_fill_uniform(double* x, long long n, uint64_t seed, uint64_t start, 
 
 void launch_add_scaled(const double* x, double* y, long long n, double a, cudaStream_t s) {
   add_scaled_kernel<<<grid_for(n), 256, 0, s>>>(x, y, n, a);
+  count_launches(1);
+}
+
+void launch_sum_rows(const double* x, long long n, int rows, double* y, cudaStream_t s) {
+  sum_rows_kernel<<<grid_for(n), 256, 0, s>>>(x, n, rows, y);
   count_launches(1);
 }
 
