@@ -418,6 +418,13 @@ __global__ void __launch_bounds__(TC_THREADS, SPLIT ? 2 : 3) tc_heff_kernel(cons
   }
 }
 
+// FP64 -> BF16, rounded once: the FP32 value rounded to odd (the last bit set
+// when something was cut off) rounds to the same BF16 as the FP64 one.
+__device__ __forceinline__ __nv_bfloat16 d2bf(double d) {
+  const ff t = d2ff(d);   // hi cut at 24 bits, lo the rest
+  return __float2bfloat16_rn(__uint_as_float(__float_as_uint(t.hi) | (t.lo != 0.f ? 1u : 0u)));
+}
+
 // One warp per padded row, lanes along the row: coalesced reads of the FP64
 // source and writes of the FP32 copy (DST16: and of the BF16 one).  Converted
 // on the integer pipes: FP64 conversions run at the FP64 rate.
@@ -439,7 +446,7 @@ __global__ void __launch_bounds__(256) convert_kernel(const ConvJob* __restrict_
         const float v = d2f_bits(x[i]);
         const long long e = (long long)(r + i) * j.kpad + c;
         j.dst32[e] = v;
-        if (DST16) ((__nv_bfloat16*)j.dst)[e] = __float2bfloat16(v);
+        if (DST16) ((__nv_bfloat16*)j.dst)[e] = d2bf(x[i]);
       }
     }
   }
