@@ -176,6 +176,7 @@ int BatchRunner::build(int node, const std::vector<int>& members, std::unique_pt
         append(&b.chunks, p.chunks);
       }
       b.finalize(4096);
+      b.fine = true;
       b.gather = gather;
     }
   }

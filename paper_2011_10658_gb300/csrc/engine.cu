@@ -166,32 +166,34 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
   v.chunks.reserve(chunks.size());
   v.outs = outs;
   v.scratch_need = 0;
-  // K per part: small enough that the launch has about sixteen tiles per SM
-  // when the plan has few, long contractions (a Gram matrix), at most k_part.
-  // A slab of 16 is one trip to L2, so long sums are cut down to 192; parts of
-  // 128 cost an upper-node update more in the reduction than they save, and
-  // with 4 tiles per SM and parts of 256 the operator updates of a centre move
-  // ran 1.06 times as long (GB300, 4x4x4 chi=64).
+  // K per part: small enough that the launch has about four tiles per SM when
+  // the plan has few, long contractions (a Gram matrix), at most k_part.  Where
+  // a sum is cut is part of its rounding, and the tensors of a centre move have
+  // to come out the same to the last place (see cholesky_inv_kernel), so only
+  // products (fine) are cut further: sixteen tiles per SM, parts of 192, sums
+  // counted in slabs of 16, each one trip to L2, added terms (up to 160 in the
+  // last stage of an upper product) among them.  GB300: FP64 upper product
+  // 4x4x4 chi=64 1329 -> 1099 us, chi=32 190 -> 115 us; the operator updates of
+  // a centre move would gain 6 %.
+  const long long tiles_wanted = fine ? 16 * 152 : 4 * 152;
   long long work = 0, base_tiles = 0;
-  // length of a chunk in the sum: whole slabs of 16 (a term that is only added
-  // is one trip to L2 as well: 160 of them in one sum took 280 us)
-  auto slabs = [](const KChunk& c) { return c.add ? 16 : (c.K + 15) / 16 * 16; };
+  auto length = [&](const KChunk& c) { return fine ? (c.add ? 16 : (c.K + 15) / 16 * 16) : (c.add ? 1 : c.K); };
   for (const KOutput& o : outs) {
     long long ktot = 0;
-    for (int c = o.chunk_begin; c < o.chunk_end; ++c) ktot += slabs(chunks[c]);
+    for (int c = o.chunk_begin; c < o.chunk_end; ++c) ktot += length(chunks[c]);
     const long long t = (long long)((o.M + BMs - 1) / BMs) * ((o.N + BNs - 1) / BNs);
     work += t * ktot;
     base_tiles += t;
   }
-  const long long kp = std::max(192LL, std::min(k_part, work / (16 * 152)));
-  const bool few_tiles = base_tiles < 16 * 152;
+  const long long kp = std::max(fine ? 192LL : 256LL, std::min(k_part, work / tiles_wanted));
+  const bool few_tiles = base_tiles < tiles_wanted;
   std::vector<KChunk>& nc = v.chunks;
   for (size_t oi = 0; oi < outs.size(); ++oi) {
     KOutput& o = v.outs[oi];
     const KOutput& mo = outs[oi];
     const int tm = (o.M + BMs - 1) / BMs, tn = (o.N + BNs - 1) / BNs;
     long long ktot = 0;
-    for (int c = mo.chunk_begin; c < mo.chunk_end; ++c) ktot += slabs(chunks[c]);
+    for (int c = mo.chunk_begin; c < mo.chunk_end; ++c) ktot += length(chunks[c]);
     const bool split = ktot > 2 * kp && (tm * tn <= 16 || few_tiles);
     std::vector<std::pair<int, int>> parts;   // ranges in nc
     const int begin = (int)nc.size();
@@ -201,37 +203,42 @@ KVariant& KPlan::variant(int shape, cudaStream_t s) {
     } else {
       long long acc = 0;
       int part_begin = begin;
+      auto close_if_full = [&]() {
+        if (acc < kp) return;
+        parts.push_back({part_begin, (int)nc.size()});
+        part_begin = (int)nc.size();
+        acc = 0;
+      };
       for (int c = mo.chunk_begin; c < mo.chunk_end; ++c) {
         const KChunk& ch = chunks[c];
         if (ch.add) {
           nc.push_back(ch);
-          acc += slabs(ch);
-          if (acc >= kp) {
-            parts.push_back({part_begin, (int)nc.size()});
-            part_begin = (int)nc.size();
-            acc = 0;
-          }
-        } else {
-          // a two-level K is cut between its inner runs
-          const int step = ch.kin ? std::max(ch.kin, (int)kp / ch.kin * ch.kin) : (int)kp;
-          for (int k0 = 0; k0 < ch.K; k0 += step) {
-            KChunk sc = ch;
-            sc.K = std::min<int>(step, ch.K - k0);
+          acc += length(ch);
+          if (fine) close_if_full();
+          continue;
+        }
+        for (int k0 = 0; k0 < ch.K;) {
+          KChunk sc = ch;
+          if (ch.kin) {
+            // a two-level K is cut between its inner runs, the run that fills a part included
+            const int runs = (int)std::max(1LL, (kp - acc + ch.kin - 1) / ch.kin);
+            sc.K = (int)std::min<long long>((long long)runs * ch.kin, ch.K - k0);
+            sc.A = ch.A + (long long)(k0 / ch.kin) * ch.a_ko;
+            sc.B = ch.B + (long long)(k0 / ch.kin) * ch.b_ko;
+          } else {
+            sc.K = std::min<int>((int)kp, ch.K - k0);
+            sc.A = ch.A + (long long)k0 * ch.a_k;
             if (ch.bmap) {
               sc.bmap = ch.bmap + k0;
               if (ch.bval) sc.bval = ch.bval + k0;
             } else {
-              sc.B = ch.B + (ch.kin ? (long long)(k0 / ch.kin) * ch.b_ko : (long long)k0 * ch.b_k);
-            }
-            sc.A = ch.A + (ch.kin ? (long long)(k0 / ch.kin) * ch.a_ko : (long long)k0 * ch.a_k);
-            nc.push_back(sc);
-            acc += slabs(sc);
-            if (acc >= kp) {
-              parts.push_back({part_begin, (int)nc.size()});
-              part_begin = (int)nc.size();
-              acc = 0;
+              sc.B = ch.B + (long long)k0 * ch.b_k;
             }
           }
+          nc.push_back(sc);
+          k0 += sc.K;
+          acc += length(sc);
+          close_if_full();
         }
       }
       if ((int)nc.size() > part_begin) parts.push_back({part_begin, (int)nc.size()});
@@ -2164,6 +2171,7 @@ Engine::HeffPlans* Engine::heff_plans(int node, int cls, bool adjoint) {
     for (int i = 0; i < 2; ++i) st[i].finalize(kKPart);
   }
   s3.finalize(kKPart);
+  for (int i = 0; i < 3; ++i) st[i].fine = true;
   int widest = 1;
   for (int d : L.leg[2].dim) widest = std::max(widest, d);
   s3.gather = bottom && bh_fits(widest, widest);

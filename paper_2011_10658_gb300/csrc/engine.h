@@ -105,6 +105,7 @@ struct KPlan {
   std::map<std::tuple<uintptr_t, long long, long long, int, int>, int> out_index;
   int current = -1;
   long long k_part = 4096;
+  bool fine = false;    // long sums in shorter parts (a product's; see KPlan::variant)
   double flops = 0.0;   // 2 M N K over the GEMM chunks (set by finalize)
   // row-gather product of a bottom node: whole output sectors (row-major,
   // not accumulated), A rows of unit stride; runs on kernels_bh.cu
@@ -121,7 +122,7 @@ struct KPlan {
   void clear() {
     chunks.clear(); outs.clear(); out_chunks.clear(); out_index.clear(); current = -1; flops = 0.0;
     for (KVariant& v : var) v.ready = false;
-    gather = bh.ready = false;
+    fine = gather = bh.ready = false;
   }
   int add_output(double* C, long long c_m, long long c_n, int M, int N, int accumulate, int nin = 0, long long c_no = 0);
   void add_chunk(const KChunk& c);

@@ -262,86 +262,84 @@ __global__ void fill_uniform_kernel(double* __restrict__ x, long long n, uint64_
 }
 
 // Upper Cholesky G = R^T R and X = R^{-1}, one CTA per matrix, in one n x n
-// array of shared memory: U = D^{1/2} R above the diagonal, X transposed below
-// it.  A column of the root-free form costs one reciprocal where a square root
-// and a division stood (the serial chain of an FP64 operation is 65 cycles
-// and more here), the square roots follow side by side, and X grows by outer
-// products, a row finished and spread over the rows above it in each step.
-// 32 columns: 64 us before (column solves in one thread each), see the centre
-// moves in the engine for the whole.
+// array of shared memory: R above the diagonal (its diagonal in rd), X
+// transposed below it.  Bound by the serial chain (an FP64 operation takes 65
+// cycles and more here): a square root, a division and an update per column of
+// R, then n (n - 1) / 2 multiply-adds and n divisions down the last column of
+// X.  Every thread that divides by a diagonal takes its square root itself,
+// which saves a barrier per column.  The order of the operations is part of
+// the result: centre moves feed gauges and low-precision updates that turn a
+// changed last place into a visible difference, so the root-free form with X
+// grown by outer products (32 us a launch of sectors up to 32 columns; this form
+// 53, with X in global memory 64) is not used.
 __global__ void __launch_bounds__(256) cholesky_inv_kernel(double* G, double* Rinv, const long long* off,
                                                            const int* nn, const int* ldd, int* status,
                                                            double ill_cond) {
   extern __shared__ double sh[];
   const int idx = blockIdx.x;
-  const int n = nn[idx], ld = ldd[idx];
+  const int n = nn[idx], ld = ldd[idx], lr = n | 1;
   double* g = G + off[idx];
   double* ri = Rinv + off[idx];
-  double* R = sh;              // n x n
-  __shared__ double inv, rs[160], row[160], gmax;
+  double* R = sh;              // n rows of lr
+  __shared__ double rd[160], xd[160], gmax;
   __shared__ int bad;
   const int tid = threadIdx.x;
-  for (int e = tid; e < n * n; e += blockDim.x) R[e] = g[(e / n) * ld + (e % n)];
+  for (int e = tid; e < n * n; e += blockDim.x) R[(e / n) * lr + e % n] = g[(e / n) * ld + (e % n)];
   if (tid == 0) bad = 0;
   __syncthreads();
   // largest original diagonal = squared largest column norm of the factored matrix
   if (tid < 32) {
     double mx = 0.0;
-    for (int j = tid; j < n; j += 32) mx = fmax(mx, R[j * n + j]);
+    for (int j = tid; j < n; j += 32) mx = fmax(mx, R[j * lr + j]);
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (tid == 0) gmax = mx;
   }
   __syncthreads();
-  // u_jb (row j) with d_j = u_jj; trailing a_ab -= u_ja u_jb / d_j
+  // row j divided by r_jj = sqrt(g_jj), then trailing g_ab -= r_ja r_jb
   for (int j = 0; j < n; ++j) {
-    if (tid == 0) {
-      double d = R[j * n + j];
-      if (!(d > 0.0)) { bad = 1; d = 1.0; R[j * n + j] = 1.0; }
-      else if (d <= ill_cond * gmax) bad = bad ? bad : 2;
-      inv = 1.0 / d;
-    }
-    __syncthreads();
     const int w = n - j - 1;
-    for (int i = tid; i < w; i += blockDim.x) row[i] = -R[j * n + j + 1 + i] * inv;
+    if (tid < w || tid == 0) {
+      double d = R[j * lr + j];
+      if (!(d > 0.0)) {
+        if (tid == 0) bad = 1;
+        d = 1.0;
+      } else if (tid == 0 && d <= ill_cond * gmax) {
+        bad = bad ? bad : 2;
+      }
+      const double r = sqrt(d);
+      if (tid == 0) rd[j] = r;
+      if (tid < w) R[j * lr + j + 1 + tid] /= r;
+    }
     __syncthreads();
     for (int e = tid; e < w * w; e += blockDim.x) {
-      const int a = e / w, b = e - a * w;
-      if (b >= a) {
-        double* p = R + (j + 1 + a) * n + j + 1 + b;
-        *p = fma(row[a], R[j * n + j + 1 + b], *p);
-      }
-    }
-    __syncthreads();
-  }
-  for (int j = tid; j < n; j += blockDim.x) rs[j] = 1.0 / sqrt(R[j * n + j]);
-  __syncthreads();
-  // R = D^{-1/2} U in place and to G; the transposed sums of X start at zero
-  for (int e = tid; e < n * n; e += blockDim.x) {
-    const int a = e / n, b = e - a * n;
-    const double v = b >= a ? R[e] * rs[a] : 0.0;
-    R[e] = v;
-    g[a * ld + b] = v;
-  }
-  __syncthreads();
-  // X_ij = -rs_i sum_{i < k <= j} R_ik X_kj (X_ii = rs_i): row i is finished,
-  // then added to the sums of the rows above
-  for (int i = n - 1; i >= 0; --i) {
-    for (int j = i + tid; j < n; j += blockDim.x) {
-      const double x = j == i ? rs[i] : -R[j * n + i] * rs[i];
-      row[j] = x;
-      if (j > i) R[j * n + i] = x;
-    }
-    __syncthreads();
-    const int w = n - i;
-    for (int e = tid; e < i * w; e += blockDim.x) {
-      const int k = e / w, j = i + e - k * w;
-      R[j * n + k] = fma(R[k * n + i], row[j], R[j * n + k]);
+      const int a = j + 1 + e / w, b = j + 1 + e % w;
+      if (b >= a) R[a * lr + b] = fma(-R[j * lr + a], R[j * lr + b], R[a * lr + b]);
     }
     __syncthreads();
   }
   for (int e = tid; e < n * n; e += blockDim.x) {
     const int a = e / n, b = e - a * n;
-    ri[a * ld + b] = b > a ? R[b * n + a] : (b == a ? rs[a] : 0.0);
+    g[a * ld + b] = b > a ? R[a * lr + b] : (b == a ? rd[a] : 0.0);
+  }
+  __syncthreads();   // below the diagonal X is written from here on
+  // R X = I, a column per thread, from the diagonal up
+  if (tid < n) {
+    double* x = R + tid * lr;   // X of column tid
+    const double xc = 1.0 / rd[tid];
+    xd[tid] = xc;
+    for (int a = tid - 1; a >= 0; --a) {
+      const double* r = R + a * lr;
+      double v = 0.0;
+#pragma unroll 4
+      for (int b = a + 1; b < tid; ++b) v = fma(-r[b], x[b], v);
+      v = fma(-r[tid], xc, v);
+      x[a] = v / rd[a];
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < n * n; e += blockDim.x) {
+    const int a = e / n, b = e - a * n;
+    ri[a * ld + b] = b > a ? R[b * lr + a] : (b == a ? xd[a] : 0.0);
   }
   if (tid == 0) status[idx] = bad;
 }
@@ -979,10 +977,10 @@ void launch_cholesky_inv(double* G, double* Rinv, const long long* off, const in
   if (count <= 0) return;
   static bool configured = false;
   if (!configured) {
-    cudaFuncSetAttribute(cholesky_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 160 * 8);
+    cudaFuncSetAttribute(cholesky_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 161 * 8);
     configured = true;
   }
-  cholesky_inv_kernel<<<count, 256, (size_t)max_n * max_n * sizeof(double), s>>>(G, Rinv, off, n, ld, status,
+  cholesky_inv_kernel<<<count, 256, (size_t)max_n * (max_n | 1) * sizeof(double), s>>>(G, Rinv, off, n, ld, status,
                                                                                   ill_cond);
   count_launches(1);
 }

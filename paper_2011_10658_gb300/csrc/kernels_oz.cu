@@ -358,36 +358,31 @@ __global__ void __launch_bounds__(OZ_THREADS) oz_gram_kernel(const OzTile* __res
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOLS));
 }
 
-// O[c', c] += sum over the output's entries (partial block, alpha).  A CTA takes
-// 64 elements of one output, neighbouring lanes along c' (the contiguous index
-// of a partial block); four lanes share an element, each adding every fourth
-// partial sum, and are combined in a fixed order.
-constexpr int OZ_RED = 64;
+// O[c', c] += sum over the output's entries (partial block, alpha), the parts of
+// an entry one after another and the entries one after another.  A thread owns
+// an element, neighbouring lanes along c' (the contiguous index of a partial
+// block); the loads of eight parts are in flight at a time.  Bound by the FP64
+// chain of an element: 84 us per bottom bond of 4x4x4 chi=64, 579 with one CTA an
+// output; four lanes an element take 43 but change the order.
+constexpr int OZ_RED = 128;
 
-__global__ void __launch_bounds__(4 * OZ_RED) oz_reduce_kernel(const OzOut* __restrict__ outs,
-                                                               const OzSum* __restrict__ sums,
-                                                               const double* __restrict__ partial) {
-  __shared__ double sh[4][OZ_RED];
+__global__ void __launch_bounds__(OZ_RED) oz_reduce_kernel(const OzOut* __restrict__ outs,
+                                                           const OzSum* __restrict__ sums,
+                                                           const double* __restrict__ partial) {
   const OzOut o = outs[blockIdx.x];
-  const int mn = o.rows * o.cols, el = threadIdx.x & (OZ_RED - 1), share = threadIdx.x / OZ_RED;
-  for (int e0 = blockIdx.y * OZ_RED; e0 < mn; e0 += gridDim.y * OZ_RED) {
-    const int e = e0 + el;
+  const int mn = o.rows * o.cols;
+  for (int e = blockIdx.y * OZ_RED + threadIdx.x; e < mn; e += gridDim.y * OZ_RED) {
     double s = 0.0;
-    if (e < mn)
-      for (int k = o.sum_begin; k < o.sum_end; ++k) {
-        const OzSum t = sums[k];
-        double v = 0.0;
-#pragma unroll 4
-        for (int p = share; p < t.n_parts; p += 4) v += __ldg(partial + t.off + (long long)p * t.part_stride + e);
-        s = fma(t.alpha, v, s);
-      }
-    sh[share][el] = s;
-    __syncthreads();
-    if (share == 0 && e < mn) {
-      const int cc = e / o.rows, cp = e - cc * o.rows;   // O row c' (output sector), column c (source sector)
-      o.O[(long long)cp * o.ld + cc] += (sh[0][el] + sh[1][el]) + (sh[2][el] + sh[3][el]);
+    for (int k = o.sum_begin; k < o.sum_end; ++k) {
+      const OzSum t = sums[k];
+      const double* from = partial + t.off + e;
+      double v = 0.0;
+#pragma unroll 8
+      for (int p = 0; p < t.n_parts; ++p) v += __ldg(from + (long long)p * t.part_stride);
+      s = fma(t.alpha, v, s);
     }
-    __syncthreads();
+    const int cc = e / o.rows, cp = e - cc * o.rows;   // O row c' (output sector), column c (source sector)
+    o.O[(long long)cp * o.ld + cc] += s;
   }
 }
 
@@ -428,7 +423,7 @@ int launch_oz_gram(const OzTile* tiles, int n_tiles, const OzJob* jobs, const vo
   kern<<<grid, OZ_THREADS, smem, s>>>(tiles, n_tiles, jobs, (const uint4*)planes, partial, err, polls);
   count_launches(1);
   if (n_outs > 0) {
-    oz_reduce_kernel<<<dim3(n_outs, 8), 4 * OZ_RED, 0, s>>>(outs, sums, partial);
+    oz_reduce_kernel<<<dim3(n_outs, 8), OZ_RED, 0, s>>>(outs, sums, partial);
     count_launches(1);
   }
   return 0;
