@@ -198,7 +198,7 @@ int BatchRunner::launch(Grouped& g) {
   if (g.tc) {
     const int elem = e0->precision_ == PREC_BF16 ? 2 : 4;
     const int split = e0->precision_ == PREC_TF32X3 ? 1 : 0;
-    launch_convert(elem, g.tcp.d_xjobs, (int)g.tcp.xjobs.size(), g.tcp.x_max_elems, 0, s);
+    launch_convert(elem, split, g.tcp.d_xjobs, (int)g.tcp.xjobs.size(), g.tcp.x_max_elems, 0, s);
     const int rc = launch_tc_heff(elem, split, g.tcp.d_tiles, (int)g.tcp.tiles.size(), g.tcp.d_outs, g.tcp.d_chunks,
                                   g.tcp.d_adds, g.tcp.max_kpad, g.tcp.max_npad, 0, e0->d_err_, s);
     if (rc) e0->err_ = "tensor-core H_eff: tile shape outside the supported range";

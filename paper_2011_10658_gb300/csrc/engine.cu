@@ -2391,18 +2391,23 @@ TcPlan* Engine::tc_plan(int node) {
     soff[i] = xs;
     xs += (long long)L.sec_rows[i] * kpad[i];
   }
-  // FP32 rows serve as TF32 operands and the epilogue's adds; BF16 rows beside them
-  if (xs > xstage_elems_ || (elem == 2 && !xstage_)) {
+  // FP32 rows serve as TF32 operands and the epilogue's adds; BF16 rows, or split
+  // rows [hi | lo], beside them
+  const int op_bytes = elem == 2 ? 2 : (split ? 8 : 0);   // operand row bytes per entry
+  if (xs > xstage_elems_ || xs * op_bytes > xstage_bytes_) {
     clear_tc_cache();   // cached plans point into the old staging
     if (xstage_) { untrack(xstage_); cudaFree(xstage_); xstage_ = nullptr; }
     if (xstage32_) { untrack(xstage32_); cudaFree(xstage32_); xstage32_ = nullptr; }
-    xstage_elems_ = std::max(xstage_elems_, xs + xs / 4);
-    if (elem == 2) {
-      if (!check(cudaMalloc(&xstage_, xstage_elems_ * 2), "x staging")) return nullptr;
-      track(xstage_, xstage_elems_ * 2);
+    const long long want = std::max(xstage_elems_, xs + xs / 4);
+    xstage_elems_ = xstage_bytes_ = 0;   // until both are there
+    if (!check(cudaMalloc(&xstage32_, want * 4), "x staging")) { xstage32_ = nullptr; return nullptr; }
+    track(xstage32_, want * 4);
+    if (op_bytes) {
+      if (!check(cudaMalloc(&xstage_, want * op_bytes), "x staging")) { xstage_ = nullptr; return nullptr; }
+      track(xstage_, want * op_bytes);
     }
-    if (!check(cudaMalloc(&xstage32_, xstage_elems_ * 4), "x staging")) return nullptr;
-    track(xstage32_, xstage_elems_ * 4);
+    xstage_elems_ = want;
+    xstage_bytes_ = want * op_bytes;
   }
   float* x32 = xstage32_;
   for (int i = 0; i < ns; ++i) {
@@ -2410,7 +2415,7 @@ TcPlan* Engine::tc_plan(int node) {
     ConvJob j;
     j.src = x_in_ + L.sec_off[i];
     j.ld_src = P.dim[i];
-    j.dst = elem == 2 ? (char*)xstage_ + soff[i] * 2 : nullptr;
+    j.dst = op_bytes ? (char*)xstage_ + soff[i] * op_bytes : nullptr;
     j.dst32 = xstage32_ + soff[i];
     j.rows = L.sec_rows[i];
     j.cols = P.dim[i];
@@ -2446,25 +2451,13 @@ TcPlan* Engine::tc_plan(int node) {
       a.ld = kpad[oc];
       tc.adds.push_back(a);
     }
-    const RowMap& diag = diagonal_map(node, -1)[oc];
-    if (diag.src_sector >= 0) {
-      TcAdd a;
-      a.X32 = x32 + soff[oc];
-      a.map = nullptr;
-      a.val = diag.val;
-      a.alpha = 1.0;
-      a.ld = kpad[oc];
-      tc.adds.push_back(a);
-    }
     for (const HTerm& h : hts) {
       const bool phys = h.op[0].kind == 2 || h.op[1].kind == 2;
       const RowMap* rm = nullptr;
       if (phys) {
-        const std::vector<RowMap>& maps = h.op[0].kind == 2 && h.op[0].term < 0   ? site_ham_map(node, 0, h.op[0].cls)
-                                          : h.op[1].kind == 2 && h.op[1].term < 0 ? site_ham_map(node, 1, h.op[1].cls)
-                                                                                  : rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term);
-        if (bottom_diagonal(node, h)) continue;
-        rm = &maps[oc];
+        if (h.op[0].kind == 2 && h.op[0].term < 0) rm = &site_ham_map(node, 0, h.op[0].cls)[oc];
+        else if (h.op[1].kind == 2 && h.op[1].term < 0) rm = &site_ham_map(node, 1, h.op[1].cls)[oc];
+        else rm = &rowmap(node, h.op[0].kind == 2 ? h.op[0].term : h.op[1].term)[oc];
         if (rm->src_sector < 0) continue;
       }
       const int ic = phys ? rm->src_sector : oc;
@@ -2475,10 +2468,10 @@ TcPlan* Engine::tc_plan(int node) {
           return nullptr;
         }
         TcChunk c;
-        c.X = elem == 2 ? (const void*)((char*)xstage_ + soff[ic] * 2) : (const void*)(xstage32_ + soff[ic]);
+        c.X = op_bytes ? (const void*)((char*)xstage_ + soff[ic] * op_bytes) : (const void*)(xstage32_ + soff[ic]);
         c.map = rm ? rm->map : nullptr;
         c.kpad = kpad[ic];
-        c.xstride = kpad[ic];
+        c.xstride = kpad[ic] * (split ? 2 : 1);
         const long long welems = (long long)o.npad * c.kpad * (split ? 2 : 1);
         wj.push_back({oc, ic, h.op[2].ptr, h.coef, wtot});
         c.W = (const void*)(intptr_t)wtot;   // patched below once the buffer exists
@@ -2510,10 +2503,12 @@ TcPlan* Engine::tc_plan(int node) {
   }
   if (wtot * elem > wbuf_bytes_) {
     clear_tc_cache();   // cached plans point into the old W buffer
-    if (wbuf_) { untrack(wbuf_); cudaFree(wbuf_); }
-    wbuf_bytes_ = (wtot + wtot / 4 + 1024) * elem;
-    if (!check(cudaMalloc(&wbuf_, wbuf_bytes_), "W staging")) return nullptr;
-    track(wbuf_, wbuf_bytes_);
+    if (wbuf_) { untrack(wbuf_); cudaFree(wbuf_); wbuf_ = nullptr; }
+    wbuf_bytes_ = 0;
+    const long long want = (wtot + wtot / 4 + 1024) * elem;
+    if (!check(cudaMalloc(&wbuf_, want), "W staging")) { wbuf_ = nullptr; return nullptr; }
+    track(wbuf_, want);
+    wbuf_bytes_ = want;
   }
   for (TcChunk& c : tc.chunks) c.W = (char*)wbuf_ + (intptr_t)c.W * elem;
   tc.wtot = wtot;
@@ -2530,7 +2525,7 @@ TcPlan* Engine::tc_plan(int node) {
     tc.wjobs.push_back(j);
   }
   // algorithmic bytes: x staging read once, y written once (FP64), W read once
-  tc.bytes_alg = (double)xs * elem + (double)L.size * 8.0 + (double)wtot * elem;
+  tc.bytes_alg = (double)xs * (split ? 8 : elem) + (double)L.size * 8.0 + (double)wtot * elem;
   // longest tiles first: the last ones to start then end soon
   std::stable_sort(tc.tiles.begin(), tc.tiles.end(), [](const TcTile& x, const TcTile& y) {
     return x.chunk_end - x.chunk_begin > y.chunk_end - y.chunk_begin;
@@ -2575,7 +2570,7 @@ int Engine::apply_heff_mixed(const double* x, double* y) {
   if (!tc) return -1;
   const int elem = precision_ == PREC_BF16 ? 2 : 4;
   const int split = precision_ == PREC_TF32X3 ? 1 : 0;
-  launch_convert(elem, tc->d_xjobs, (int)tc->xjobs.size(), tc->x_max_elems, x - x_in_, stream_);
+  launch_convert(elem, split, tc->d_xjobs, (int)tc->xjobs.size(), tc->x_max_elems, x - x_in_, stream_);
   cudaEvent_t e0 = nullptr;
   if (profiling_) ev_begin(&e0);
   int rc = launch_tc_heff(elem, split, tc->d_tiles, (int)tc->tiles.size(), tc->d_outs, tc->d_chunks, tc->d_adds,

@@ -448,9 +448,10 @@ class Engine {
   int apply_heff_tg(const double* x, double* y);
   int tc_w_node_ = -1;          // node whose environment blocks are staged
   void clear_tc_cache();
-  void* xstage_ = nullptr;      // BF16 padded staging of x (BF16 operands)
+  void* xstage_ = nullptr;      // padded operand rows of x (BF16, or split [hi | lo])
   float* xstage32_ = nullptr;   // FP32 padded staging of x
-  long long xstage_elems_ = 0;
+  long long xstage_elems_ = 0;  // entries of xstage32_
+  long long xstage_bytes_ = 0;
   void* wbuf_ = nullptr;
   long long wbuf_bytes_ = 0;
   int* d_err_ = nullptr;

@@ -41,6 +41,25 @@ __device__ __forceinline__ double f2d_bits(float f) {
   return __longlong_as_double((long long)(sign | ((unsigned long long)(e - 127 + 1023) << 52) | (frac << 29)));
 }
 
+// FP64 -> FP32 as the cast does it, FP32 subnormals and signed zeros kept, on
+// the integer pipes in the normal range: the exponent rebiased, the top 23
+// fraction bits, a carry from the other 29.
+static __device__ __noinline__ float d2f_cast(double d) { return (float)d; }
+__device__ __forceinline__ float d2f_rn(double d) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  if ((h & 0x7fffffffu) - (897u << 20) >= (253u << 20))   // outside 2^-126 .. 2^127
+    return ((h << 1) | l) == 0u ? __uint_as_float(h) : d2f_cast(d);
+  const unsigned t = (__funnelshift_l(l, h, 3) - (384u << 23)) & 0x7fffffffu;
+  return __uint_as_float((t + (((l & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29)) | (h & 0x80000000u));
+}
+
+// FP32 -> FP64, exact, subnormals too (brought into the normal range first).
+__device__ __forceinline__ double f2d_exact(float f) {
+  const bool small = fabsf(f) < 0x1p-126f;
+  const double d = f2d_bits(small ? f * 0x1p24f : f);
+  return __hiloint2double(__double2hiint(d) - (small && f != 0.f ? 24 << 20 : 0), __double2loint(d));
+}
+
 // ---- float-float arithmetic: a value hi + lo held in two FP32 numbers
 // (about 48 significant bits), with products and sums made error-free by
 // FMA (Dekker's TwoProduct) and Knuth's TwoSum.  GB300 runs FP32 at many

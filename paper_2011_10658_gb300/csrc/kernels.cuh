@@ -213,12 +213,13 @@ namespace qed {
 // One output c-sector of y (rows x n, FP64, row-major with ld = n) is the
 // sum of GEMM chunks  sign(r) * X[map(r), :] . W^T  accumulated in TMEM
 // (A rows gathered into shared memory, B = W, both K-major) and of add terms
-// alpha * sign(r) * val(r) * X32[map(r), :n] applied in FP32 in the epilogue.
+// alpha * sign(r) * val(r) * X32[map(r), :n], added in FP64 when the tile is
+// written; X32 and ld are the same in all adds of an output.
 struct TcChunk {
   const void* X;      // staging source sector matrix (BF16 or FP32), row stride xstride
   const int* map;     // sign-encoded row map (nullable: identity)
   const void* W;      // B operand in core-matrix order (alpha folded in; split: [hi | lo])
-  int kpad;           // K of the staged rows, multiple of 16
+  int kpad;           // K of the staged rows, multiple of 16 (split: of each part)
   int xstride;        // elements per staged source row
 };
 struct TcAdd {
@@ -241,12 +242,12 @@ struct TcTile {
   int row0;
   int chunk_begin, chunk_end;
 };
-// Staging of x: dst32 (and, for BF16 operands, dst), rows x kpad, zero padded,
-// <- src (rows x cols, ld_src), FP64 source.
+// Staging of x: dst32 (and, for BF16 and split operands, dst), rows x kpad, zero
+// padded, <- src (rows x cols, ld_src), FP64 source.
 struct ConvJob {
   const double* src;
   long long ld_src;   // row stride of the source
-  void* dst;          // BF16 copy (BF16 operands only)
+  void* dst;          // BF16 rows, or split rows [hi | lo] of 2 kpad floats
   float* dst32;       // FP32 copy
   int rows, cols, kpad;
 };
@@ -369,7 +370,8 @@ int launch_oz_gram(const OzTile* tiles, int n_tiles, const OzJob* jobs, const vo
                    const OzOut* outs, int n_outs, const OzSum* sums, int* err, cudaStream_t s, long long polls = -1);
 
 // Staging for launch_tc_heff; shift: added to every source pointer (elements).
-void launch_convert(int elem, const ConvJob* jobs, int n_jobs, long long max_elems, long long shift, cudaStream_t s);
+void launch_convert(int elem, int split, const ConvJob* jobs, int n_jobs, long long max_elems, long long shift,
+                    cudaStream_t s);
 void launch_stage_w(int elem, int split, const WJob* jobs, int n_jobs, cudaStream_t s);
 
 }  // namespace qed

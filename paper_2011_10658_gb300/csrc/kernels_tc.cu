@@ -10,28 +10,31 @@
 // of 8 rows x 16 bytes), the environment block is the B operand, and all
 // product terms of an output tile accumulate in one TMEM accumulator.  Terms
 // without an environment factor (the diagonal of the two sites, the internal
-// hopping) are added in float-float arithmetic when the tile is written.
+// hopping) are added in FP64 when the tile is written.
 //
 // One CTA = one 128-row tile of one output charge sector.  The rows of a
 // sector are ordered by the terms that reach them, so a tile walks only some
 // of the terms (Engine::tc_tiles).  Eight gather warps feed two stages of A,
 // one thread of a ninth warp copies the blocks of W (staged in core-matrix
 // order, bulk copies two terms ahead) and issues the MMAs; they meet on
-// mbarriers only.  x is staged once per product as FP32 (and BF16) rows; the
-// hi and lo TF32 parts of a split product are cut from the FP32 row on its way
-// to shared memory, so a gather moves 4 bytes per entry.  A warp's load takes
-// 8 rows x 64 bytes: eight cache lines instead of one per lane, and stores
-// that fill all banks.  The rows of term j + 1 and the map of term j + 2 are
-// read while term j waits for its stage; rows two terms ahead in registers
-// measured the same.
+// mbarriers only.  x is staged once per product as FP32 rows, for the terms
+// without environment factor, and as operand rows: BF16, or the hi and lo TF32
+// parts of every entry (lo is what the FP64 entry leaves after hi: cutting both
+// from the FP32 row would gather half as much, 22 us less per product of 4x4x4
+// chi=64, but drops the bits that FP32 has rounded away).  A warp's load takes 8
+// rows x 64 bytes: eight cache lines instead of one per lane, and stores that
+// fill all banks.  The rows of term j + 1 and the map of term j + 2 are read
+// while term j waits for its stage; rows two terms ahead in registers measured
+// the same.
 //
 // Bound by the round trip gather -> MMA -> free stage of each term (two CTAs
 // an SM for split TF32).  Product at bottom node 0 of 4x4x4, whole call, GB300:
-// chi=64 split TF32 287 -> 108 us, chi=48 BF16 132 -> 77 us.  On the way: FP64
-// arithmetic out of the epilogue and the staging (two operations per clock and
-// SM; 40 % of the kernel) and coalesced gathers 203 us; gather and issue on
-// separate warps, 16-byte pieces at compile-time places 132 us; rows ordered
-// by their terms 108 us.
+// chi=64 split TF32 287 -> 139 us, chi=48 BF16 132 -> 87 us: coalesced gathers,
+// gather and issue on separate warps, 16-byte pieces at compile-time places (a
+// launch whose rows are narrow has a kernel with fewer registers: 159 us with
+// one for all widths), rows ordered by their terms.  About 10 us are the FP64
+// multiply-adds at the end, which float-float arithmetic on the FP32 pipes would
+// save with fewer bits.
 //
 // Every mbarrier wait is bounded (polls, a launch argument); a timeout sets
 // *err, and the CTA then drains its MMAs through a commit to a fresh barrier
@@ -41,6 +44,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdio>
+#include <type_traits>
 
 #include "ffloat.cuh"
 #include "kernels.cuh"
@@ -54,7 +58,6 @@ constexpr int TC_THREADS = 32 * (TC_GATHER_WARPS + 1);   // and the warp that is
 constexpr int TC_WARP_ROWS = 16;                  // rows of A a warp gathers
 constexpr int TC_ADDS = 8;                        // terms without environment factor whose row factors are held
 constexpr int TC_UNROLL = 4;                      // outputs a thread writes at a time
-constexpr int TC_PRE = 6;                         // 16-byte pieces of a chunk a thread holds
 constexpr long long kWaitPolls = 1LL << 22;   // default bound of one mbarrier wait
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -108,12 +111,13 @@ __device__ __forceinline__ void mma(uint32_t tmem, uint64_t ad, uint64_t bd, uin
 
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 
-// One thread's share of a chunk's A tile: KQ / 2 pieces of 16 bytes.  Piece `it`
-// is piece q of row r of the warp's 16 rows, the eight rows of a core matrix on
-// neighbouring lanes.  mp: lane l holds the map entry of row l (mod 16).
-template <int KQ>
+// One thread's share of a chunk's A tile: KQ / 2 pieces of 16 bytes, of a split
+// row KQ / 2 of each part.  Piece `it` is piece q of row r of the warp's 16
+// rows, the eight rows of a core matrix on neighbouring lanes.  mp: lane l holds
+// the map entry of row l (mod 16).
+template <int KQ, bool SPLIT>
 struct Gather {
-  static constexpr int N = KQ / 2;
+  static constexpr int PARTS = SPLIT ? 2 : 1, HALF = KQ / 2, N = HALF * PARTS;
   static __device__ __forceinline__ int group(int it, int lane) { return it * 4 + (lane >> 3) >= KQ ? 1 : 0; }
   static __device__ __forceinline__ int piece(int it, int lane) { return it * 4 + (lane >> 3) - group(it, lane) * KQ; }
   template <int ELEM>
@@ -122,70 +126,54 @@ struct Gather {
     const uint8_t* x0 = (const uint8_t*)X + (long long)(s0 >> 1) * row_bytes;
     const uint8_t* x1 = (const uint8_t*)X + (long long)(s1 >> 1) * row_bytes;
 #pragma unroll
-    for (int it = 0; it < N; ++it) {
+    for (int i = 0; i < N; ++i) {
+      const int it = i % HALF, part = i / HALF;
       const bool g = group(it, lane);
-      v[it] = make_uint4(0u, 0u, 0u, 0u);
-      if ((g ? s1 : s0) >= 0) v[it] = __ldg((const uint4*)((g ? x1 : x0) + piece(it, lane) * 16));
+      v[i] = make_uint4(0u, 0u, 0u, 0u);
+      if ((g ? s1 : s0) >= 0) v[i] = __ldg((const uint4*)((g ? x1 : x0) + (part * KQ + piece(it, lane)) * 16));
     }
 #pragma unroll
-    for (int it = 0; it < N; ++it) {
-      const int s = group(it, lane) ? s1 : s0;
+    for (int i = 0; i < N; ++i) {
+      const int s = group(i % HALF, lane) ? s1 : s0;
       const uint32_t flip = s < 0 ? 0u : (ELEM == 2 ? (uint32_t)(s & 1) * 0x80008000u : (uint32_t)s << 31);
-      v[it].x ^= flip; v[it].y ^= flip; v[it].z ^= flip; v[it].w ^= flip;
+      v[i].x ^= flip; v[i].y ^= flip; v[i].z ^= flip; v[i].w ^= flip;
     }
   }
-  template <bool SPLIT>
   static __device__ __forceinline__ void store(uint8_t* A, const uint4* v, int warp, int lane) {
-    constexpr int KCH = SPLIT ? 2 * KQ : KQ;
 #pragma unroll
-    for (int it = 0; it < N; ++it) {
-      uint8_t* d = A + ((warp * 2 + group(it, lane)) * KCH + piece(it, lane)) * 128 + (lane & 7) * 16;
-      if (SPLIT) {
-        const float4 x = make_float4(__uint_as_float(v[it].x), __uint_as_float(v[it].y), __uint_as_float(v[it].z),
-                                     __uint_as_float(v[it].w));
-        const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
-        *(float4*)d = h;
-        *(float4*)(d + KQ * 128) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
-      } else {
-        *(uint4*)d = v[it];
-      }
+    for (int i = 0; i < N; ++i) {
+      const int it = i % HALF, part = i / HALF;
+      *(uint4*)(A + ((warp * 2 + group(it, lane)) * PARTS * KQ + part * KQ + piece(it, lane)) * 128 + (lane & 7) * 16) = v[i];
     }
   }
 };
 
-// The same for a width without a specialisation: straight to shared memory.
-template <int ELEM, bool SPLIT>
-__device__ __noinline__ void gather_any(uint8_t* A, const void* X, int row_bytes, int kq, int mp, int warp, int lane) {
-  for (int it = 0; it < kq / 2; ++it) {
-    const int rest = it * 4 + (lane >> 3), g = rest >= kq ? 1 : 0, q = rest - g * kq;
-    const int s = __shfl_sync(0xffffffffu, mp, g * 8 + (lane & 7));
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (s >= 0) {
-      v = __ldg((const uint4*)((const uint8_t*)X + (long long)(s >> 1) * row_bytes + q * 16));
-      const uint32_t flip = ELEM == 2 ? (uint32_t)(s & 1) * 0x80008000u : (uint32_t)s << 31;
-      v.x ^= flip; v.y ^= flip; v.z ^= flip; v.w ^= flip;
-    }
-    uint8_t* d = A + ((warp * 2 + g) * (SPLIT ? 2 : 1) * kq + q) * 128 + (lane & 7) * 16;
-    if (SPLIT) {
-      const float4 x = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
-      const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
-      *(float4*)d = h;
-      *(float4*)(d + kq * 128) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
-    } else {
-      *(uint4*)d = v;
-    }
+// Row widths in pieces (of a part): a K step is 32 bytes, two pieces; 16 columns
+// are two pieces of BF16, four of TF32.  f(integral_constant) of the width.
+template <int KQ, int STEP, int MAXKQ, typename F>
+__device__ __forceinline__ void by_width(int kq, F f) {
+  if constexpr (KQ <= MAXKQ) {
+    if (kq == KQ)
+      f(std::integral_constant<int, KQ>());
+    else
+      by_width<KQ + STEP, STEP, MAXKQ>(kq, f);
   }
 }
 
+// A launch whose rows are at most NARROW pieces wide keeps two (split) or three
+// CTAs on an SM; up to WIDE, what the stages of the widest rows leave in shared
+// memory (see launch_tc_heff) is one or two.
 template <int ELEM, bool SPLIT>
-__global__ void __launch_bounds__(TC_THREADS, SPLIT ? 2 : 3) tc_heff_kernel(const TcTile* __restrict__ tiles,
-                                                                             const TcOutput* __restrict__ outs,
-                                                                             const TcChunk* __restrict__ chunks,
-                                                                             const TcAdd* __restrict__ adds,
-                                                                             int a_bytes, int b_bytes, int b_stages,
-                                                                             long long y_shift, int* err,
-                                                                             long long polls) {
-  constexpr int PARTS = SPLIT ? 2 : 1;
+struct Width {
+  static constexpr int STEP = ELEM, NARROW = SPLIT ? 8 : 12, WIDE = SPLIT ? 16 : (ELEM == 2 ? 20 : 24);
+};
+
+template <int ELEM, bool SPLIT, int MAXKQ>
+__global__ void __launch_bounds__(TC_THREADS, (SPLIT ? 1 : 2) + (MAXKQ <= Width<ELEM, SPLIT>::NARROW ? 1 : 0))
+    tc_heff_kernel(const TcTile* __restrict__ tiles, const TcOutput* __restrict__ outs,
+                   const TcChunk* __restrict__ chunks, const TcAdd* __restrict__ adds, int a_bytes, int b_bytes,
+                   int b_stages, long long y_shift, int* err, long long polls) {
+  constexpr int PARTS = SPLIT ? 2 : 1, STEP = Width<ELEM, SPLIT>::STEP;
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ uint32_t tmem_slot;
   // MMAs of the two A stages, drain, the gathers of the two A stages, the
@@ -221,17 +209,12 @@ __global__ void __launch_bounds__(TC_THREADS, SPLIT ? 2 : 3) tc_heff_kernel(cons
     const int at = tile.row0 + warp * TC_WARP_ROWS + (lane & 15);
     const int row = at < out.rows ? __ldg(out.order + at) : -1;
     auto map_entry = [&](const TcChunk& c) { return row >= 0 ? (c.map ? __ldg(c.map + row) : (row << 1)) : -1; };
-    uint4 pre[TC_PRE];
+    uint4 pre[PARTS * MAXKQ / 2];
     auto load = [&](const TcChunk& c, int mp) {
       const int rb = c.xstride * ELEM;
-      switch (c.kpad * ELEM / 16) {
-        case 2: Gather<2>::load<ELEM>(pre, c.X, rb, mp, lane); break;
-        case 4: Gather<4>::load<ELEM>(pre, c.X, rb, mp, lane); break;
-        case 6: Gather<6>::load<ELEM>(pre, c.X, rb, mp, lane); break;
-        case 8: Gather<8>::load<ELEM>(pre, c.X, rb, mp, lane); break;
-        case 12: Gather<12>::load<ELEM>(pre, c.X, rb, mp, lane); break;
-        default: break;
-      }
+      by_width<STEP, STEP, MAXKQ>(c.kpad * ELEM / 16, [&](auto kq) {
+        Gather<decltype(kq)::value, SPLIT>::template load<ELEM>(pre, c.X, rb, mp, lane);
+      });
     };
     TcChunk c, cn, cnn;
     int mp = -1, mp_next = -1;
@@ -248,14 +231,8 @@ __global__ void __launch_bounds__(TC_THREADS, SPLIT ? 2 : 3) tc_heff_kernel(cons
         s_fail = 1;
         break;
       }
-      switch (c.kpad * ELEM / 16) {
-        case 2: Gather<2>::store<SPLIT>(A, pre, warp, lane); break;
-        case 4: Gather<4>::store<SPLIT>(A, pre, warp, lane); break;
-        case 6: Gather<6>::store<SPLIT>(A, pre, warp, lane); break;
-        case 8: Gather<8>::store<SPLIT>(A, pre, warp, lane); break;
-        case 12: Gather<12>::store<SPLIT>(A, pre, warp, lane); break;
-        default: gather_any<ELEM, SPLIT>(A, c.X, c.xstride * ELEM, c.kpad * ELEM / 16, mp, warp, lane); break;
-      }
+      by_width<STEP, STEP, MAXKQ>(c.kpad * ELEM / 16,
+                                  [&](auto kq) { Gather<decltype(kq)::value, SPLIT>::store(A, pre, warp, lane); });
       asm volatile("fence.proxy.async.shared::cta;");
       __syncwarp();
       if (lane == 0)
@@ -358,77 +335,119 @@ __global__ void __launch_bounds__(TC_THREADS, SPLIT ? 2 : 3) tc_heff_kernel(cons
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
-  // lanes along the rows of y, adds in float-float with the factor and source
-  // row of the first TC_ADDS formed once per row
+  // lanes along the rows of y; the terms without environment factor are added
+  // in FP64 and in their order.  Each row lists those of the first TC_ADDS that
+  // reach it (factor, source row): most of its projectors do not.
   const int rows = min(128, out.rows - tile.row0), total = rows * out.n;
   const int n_add = out.add_end - out.add_begin, held = min(n_add, TC_ADDS);
-  float2* const F = (float2*)(smem + ((size_t)128 * ld * 4 + 15) / 16 * 16);
+  double* const F = (double*)(smem + ((size_t)128 * ld * 4 + 15) / 16 * 16);
   int* const S = (int*)(F + TC_ADDS * 128);
   int* const R = S + TC_ADDS * 128;
-  if (tid < rows) R[tid] = __ldg(out.order + tile.row0 + tid);
-  __syncthreads();
-  auto factor = [&](const TcAdd& a, int r, ff& f) {
-    const int g = R[r];
-    const int src = a.map ? __ldg(a.map + g) : (g << 1);
-    f = d2ff(a.alpha);
-    if (a.val) f = f * d2ff(__ldg(a.val + g));
-    if (src & 1) f = ff(-f.hi, -f.lo);
-    return src < 0 ? -1 : src >> 1;
+  int* const C = R + 128;
+  auto source = [&](const TcAdd& a, int g) { return a.map ? __ldg(a.map + g) : (g << 1); };
+  auto factor = [&](const TcAdd& a, int g, int src) {
+    const double f = (src & 1) ? -a.alpha : a.alpha;
+    return a.val ? f * __ldg(a.val + g) : f;
   };
-  for (int e = tid; e < held * 128; e += TC_THREADS) {
-    const int r = e & 127;
-    ff f;
-    S[e] = r < rows ? factor(adds[out.add_begin + (e >> 7)], r, f) : -1;
-    F[e] = make_float2(f.hi, f.lo);
+  if (tid < rows) {
+    const int g = __ldg(out.order + tile.row0 + tid);
+    int src[TC_ADDS], c = 0;
+#pragma unroll
+    for (int i = 0; i < TC_ADDS; ++i) src[i] = i < held ? source(adds[out.add_begin + i], g) : -1;
+#pragma unroll
+    for (int i = 0; i < TC_ADDS; ++i)
+      if (src[i] >= 0) {
+        F[c * 128 + tid] = factor(adds[out.add_begin + i], g, src[i]);
+        S[c * 128 + tid] = src[i] >> 1;
+        ++c;
+      }
+    R[tid] = g;
+    C[tid] = c;
   }
   __syncthreads();
+  // such a term keeps the parent charge: all of them read the output's own sector
+  const float* const X = n_add > 0 ? adds[out.add_begin].X32 : nullptr;
+  const int ldx = n_add > 0 ? adds[out.add_begin].ld : 0;
   double* const y = out.y + y_shift;
   for (int e0 = tid; e0 < total; e0 += TC_UNROLL * TC_THREADS) {
-    ff acc[TC_UNROLL];
-    int r[TC_UNROLL], n[TC_UNROLL];
+    double acc[TC_UNROLL];
+    int r[TC_UNROLL], n[TC_UNROLL], most = 0;
 #pragma unroll
     for (int u = 0; u < TC_UNROLL; ++u) {
       const int e = min(e0 + u * TC_THREADS, total - 1);
       r[u] = out.n == 1 ? e : (int)__umulhi((unsigned)e, out.div);
       n[u] = e - r[u] * out.n;
-      acc[u] = ff(D[r[u] * ld + n[u]]);
+      acc[u] = f2d_exact(D[r[u] * ld + n[u]]);
+      most = max(most, C[r[u]]);
     }
-    for (int i = 0; i < n_add; ++i) {
-      const TcAdd a = adds[out.add_begin + i];
-      ff f[TC_UNROLL];
+    for (int i = 0; i < most; ++i) {
       float x[TC_UNROLL];
 #pragma unroll
-      for (int u = 0; u < TC_UNROLL; ++u) {
-        int src;
-        if (i < held) {
-          src = S[i * 128 + r[u]];
-          f[u] = ff(F[i * 128 + r[u]].x, F[i * 128 + r[u]].y);
-        } else {
-          src = factor(a, r[u], f[u]);
-        }
-        if (src < 0) f[u] = ff(0.f);
-        x[u] = src < 0 ? 0.f : __ldg(a.X32 + (long long)src * a.ld + n[u]);
-      }
+      for (int u = 0; u < TC_UNROLL; ++u)
+        x[u] = i < C[r[u]] ? __ldg(X + (long long)S[i * 128 + r[u]] * ldx + n[u]) : 0.f;
 #pragma unroll
-      for (int u = 0; u < TC_UNROLL; ++u) acc[u] = kc_fma(f[u], ff(x[u]), acc[u]);
+      for (int u = 0; u < TC_UNROLL; ++u)
+        if (i < C[r[u]]) acc[u] = fma(F[i * 128 + r[u]], f2d_exact(x[u]), acc[u]);
+    }
+    for (int i = held; i < n_add; ++i) {
+      const TcAdd a = adds[out.add_begin + i];
+#pragma unroll
+      for (int u = 0; u < TC_UNROLL; ++u) {
+        const int src = source(a, R[r[u]]);
+        if (src >= 0)
+          acc[u] = fma(factor(a, R[r[u]], src), f2d_exact(__ldg(X + (long long)(src >> 1) * ldx + n[u])), acc[u]);
+      }
     }
 #pragma unroll
     for (int u = 0; u < TC_UNROLL; ++u)
-      if (e0 + u * TC_THREADS < total) y[(long long)R[r[u]] * out.n + n[u]] = to_d<ff>(acc[u]);
+      if (e0 + u * TC_THREADS < total) y[(long long)R[r[u]] * out.n + n[u]] = acc[u];
   }
 }
 
 // FP64 -> BF16, rounded once: the FP32 value rounded to odd (the last bit set
 // when something was cut off) rounds to the same BF16 as the FP64 one.
+static __device__ __noinline__ __nv_bfloat16 d2bf_cast(double d) { return __double2bfloat16(d); }
 __device__ __forceinline__ __nv_bfloat16 d2bf(double d) {
+  const unsigned top = (unsigned)__double2hiint(d) & 0x7fffffffu;
+  if (top - (920u << 20) >= (230u << 20)) return d2bf_cast(d);   // the range of d2ff's short form
   const ff t = d2ff(d);   // hi cut at 24 bits, lo the rest
   return __float2bfloat16_rn(__uint_as_float(__float_as_uint(t.hi) | (t.lo != 0.f ? 1u : 0u)));
 }
 
+// Split operand: x = d in FP32, hi = x cut to the 11 bits that the TF32 units
+// read, lo = d - hi rounded to FP32.  d - hi is formed as an integer in units of
+// d's last place.
+static __device__ __noinline__ void split_cast(double d, float& x, float& hi, float& lo) {
+  x = (float)d;
+  hi = tf32_hi(x);
+  lo = (float)(d - (double)hi);
+}
+__device__ __forceinline__ void split_tf32(double d, float& x, float& hi, float& lo) {
+  const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+  const unsigned top = h & 0x7fffffffu;
+  if (top - (949u << 20) >= (201u << 20)) {   // outside 2^-74 .. 2^127
+    if ((top | l) == 0u) {
+      x = hi = lo = 0.f;
+      return;
+    }
+    split_cast(d, x, hi, lo);
+    return;
+  }
+  x = d2f_rn(d);
+  hi = tf32_hi(x);
+  const unsigned hb = __float_as_uint(hi) & 0x7fffffffu, e = top >> 20;   // hi's exponent is d's or one more
+  const long long m = ((long long)((top & 0xfffffu) | 0x100000u) << 32) | l;
+  const long long hm = (long long)((hb & 0x7fffffu) | 0x800000u) << (29 + (hb >> 23) - (e - 896u));
+  const float r = __ll2float_rn(m - hm) * __uint_as_float((e - 948u) << 23);
+  lo = (h >> 31) ? -r : r;
+}
+
 // One warp per padded row, lanes along the row: coalesced reads of the FP64
-// source and writes of the FP32 copy (DST16: and of the BF16 one).  Converted
-// on the integer pipes: FP64 conversions run at the FP64 rate.
-template <bool DST16>
+// source and writes of the FP32 copy and, for BF16 and split operands, of the
+// operand rows.  Converted on the integer pipes: FP64 conversions run at the
+// FP64 rate.
+enum { CONV_F32 = 0, CONV_BF16 = 1, CONV_SPLIT = 2 };
+template <int MODE>
 __global__ void __launch_bounds__(256) convert_kernel(const ConvJob* __restrict__ jobs, long long shift) {
   const ConvJob j = jobs[blockIdx.y];
   const int lane = threadIdx.x & 31;
@@ -443,10 +462,14 @@ __global__ void __launch_bounds__(256) convert_kernel(const ConvJob* __restrict_
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         if (r + i >= j.rows) break;
-        const float v = d2f_bits(x[i]);
         const long long e = (long long)(r + i) * j.kpad + c;
-        j.dst32[e] = v;
-        if (DST16) ((__nv_bfloat16*)j.dst)[e] = d2bf(x[i]);
+        if (MODE == CONV_SPLIT) {
+          float* d = (float*)j.dst + (long long)(r + i) * 2 * j.kpad + c;
+          split_tf32(x[i], j.dst32[e], d[0], d[j.kpad]);
+        } else {
+          j.dst32[e] = d2f_rn(x[i]);
+          if (MODE == CONV_BF16) ((__nv_bfloat16*)j.dst)[e] = d2bf(x[i]);
+        }
       }
     }
   }
@@ -492,20 +515,31 @@ int launch_tc_heff(int elem, int split, const TcTile* tiles, int n_tiles, const 
   const int sm = 226 * 1024, fit = std::max(1, sm / (2 * (a_bytes + b_bytes) + 1024));
   int b_stages = 2;
   while (b_stages < 4 && sm / (2 * a_bytes + (b_stages + 1) * b_bytes + 1024) >= std::min(fit, 2)) ++b_stages;
-  const int smem = std::max(2 * a_bytes + b_stages * b_bytes, 128 * (max_npad + 1) * 4 + 16 + TC_ADDS * 128 * 12 + 128 * 4);
-  auto kern = elem == 2 ? tc_heff_kernel<2, false> : (split ? tc_heff_kernel<4, true> : tc_heff_kernel<4, false>);
-  static bool attr[3] = {false, false, false};   // set once: host attribute calls cost as much as a launch
-  bool& set = attr[elem == 2 ? 0 : (split ? 2 : 1)];
-  if (!set) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-    set = true;
-  }
+  const int smem = std::max(2 * a_bytes + b_stages * b_bytes, 128 * (max_npad + 1) * 4 + 16 + TC_ADDS * 128 * 12 + 2 * 128 * 4);
+  auto pick = [&](auto type, auto is_split) {
+    constexpr int E = decltype(type)::value;
+    constexpr bool S = decltype(is_split)::value;
+    using W = Width<E, S>;
+    const bool wide = max_kpad * E / 16 > W::NARROW;
+    auto kern = wide ? tc_heff_kernel<E, S, W::WIDE> : tc_heff_kernel<E, S, W::NARROW>;
+    static bool attr[2] = {false, false};   // set once: host attribute calls cost as much as a launch
+    if (!attr[wide]) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+      attr[wide] = true;
+    }
+    return kern;
+  };
+  using Two = std::integral_constant<int, 2>;
+  using Four = std::integral_constant<int, 4>;
+  auto kern = elem == 2 ? pick(Two(), std::false_type()) : (split ? pick(Four(), std::true_type()) : pick(Four(), std::false_type()));
+  if (max_kpad * elem / 16 > (elem == 2 ? Width<2, false>::WIDE : (split ? Width<4, true>::WIDE : Width<4, false>::WIDE))) return -7;
   kern<<<n_tiles, TC_THREADS, smem, s>>>(tiles, outs, chunks, adds, a_bytes, b_bytes, b_stages, y_shift, err, polls);
   count_launches(1);
   return 0;
 }
 
-void launch_convert(int elem, const ConvJob* jobs, int n_jobs, long long max_elems, long long shift, cudaStream_t s) {
+void launch_convert(int elem, int split, const ConvJob* jobs, int n_jobs, long long max_elems, long long shift,
+                    cudaStream_t s) {
   if (n_jobs <= 0) return;
   // rows <= max_elems / 16 (kpad >= 16); 32 rows per block, about 8 blocks per SM in total
   long long gx = (max_elems / 16 + 31) / 32;
@@ -514,9 +548,11 @@ void launch_convert(int elem, const ConvJob* jobs, int n_jobs, long long max_ele
   if (gx < 1) gx = 1;
   dim3 grid((unsigned)gx, (unsigned)n_jobs);
   if (elem == 2)
-    convert_kernel<true><<<grid, 256, 0, s>>>(jobs, shift);
+    convert_kernel<CONV_BF16><<<grid, 256, 0, s>>>(jobs, shift);
+  else if (split)
+    convert_kernel<CONV_SPLIT><<<grid, 256, 0, s>>>(jobs, shift);
   else
-    convert_kernel<false><<<grid, 256, 0, s>>>(jobs, shift);
+    convert_kernel<CONV_F32><<<grid, 256, 0, s>>>(jobs, shift);
   count_launches(1);
 }
 

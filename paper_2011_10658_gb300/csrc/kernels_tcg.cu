@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(TG_THREADS, 4) tg_gemm_kernel(const TgTile* __
           *p = out.accumulate ? *p + f : f;
         } else {
           double* p = (double*)out.C + y_shift + cbase + (long long)col * out.cj;
-          *p = out.accumulate ? *p + f2d_bits(f) : f2d_bits(f);
+          *p = out.accumulate ? *p + f2d_exact(f) : f2d_exact(f);
         }
       }
     }

@@ -81,3 +81,41 @@ def move_digests(q, L, chi, precision, path):
 @pytest.mark.parametrize("L,chi,precision,path", MOVES)
 def test_centre_moves(q, L, chi, precision, path):
     check(move_digests(q, L, chi, precision, path))
+
+
+# Bottom nodes (row gathers: sectors of at most 32 columns, of 33-48 and 49-64)
+# and upper nodes in every operand format.
+PRODUCTS = [((4, 4, 4), 64, "tf32x3", (0, 32, 62)), ((4, 4, 4), 64, "tf32", (0,)), ((4, 4, 4), 48, "bf16", (0, 56)),
+            ((2, 2, 2), 13, "tf32x3", (1, 4)), ((2, 2, 2), 96, "tf32x3", (0, 6)), ((2, 2, 2), 112, "tf32x3", (0, 5)),
+            ((2, 2, 2), 128, "bf16", (0,)), ((2, 2, 2), 128, "tf32", (0,))]
+
+
+def product_digests(q, L, chi, precision, nodes):
+    s = state(q, L, chi, precision)
+    out = {}
+    for node in nodes:
+        s.move_center(node)
+        x = np.random.default_rng(node).random(s.node_size(node)) - 0.5
+        out["product/%s/%d/%s/%d" % ("x".join(map(str, L)), chi, precision, node)] = digest(s.apply_heff(x))
+    s.close()
+    return out
+
+
+@pytest.mark.parametrize("L,chi,precision,nodes", PRODUCTS)
+def test_reduced_precision_products(q, L, chi, precision, nodes):
+    check(product_digests(q, L, chi, precision, nodes))
+
+
+def test_small_magnitudes_are_kept(q):
+    """Entries below FP32's normal range (3 % of these) are rounded as the FP32
+    cast does it and not to zero, which would leave an error of 5e-3.  Their
+    low parts (2^-11 of an entry) may be lost in the tensor cores."""
+    s = state(q, (4, 2, 2), 16, "tf32x3")
+    s.move_center(0)
+    x = (np.random.default_rng(4).random(s.node_size(0)) - 0.5) * 2.0 ** -120
+    y = s.apply_heff(x)
+    s.set_precision("fp64")
+    want = s.apply_heff(x)
+    s.close()
+    scale = 2.0 ** 120
+    assert np.linalg.norm((y - want) * scale) < 1e-3 * np.linalg.norm(want * scale)
