@@ -3007,7 +3007,7 @@ int Engine::lz_thick_restart(int k, int kmax, long long n, int* j0) {
   double* beta = d_scal_ + kBeta;
   const int keep = std::min(kThickKeep, kmax / 4);
   if (keep < 1) {   // explicit restart from the Ritz vector
-    launch_tridiag_lowest(alpha, beta, k, d_scal_ + kOut, d_scal_ + kSvec, 1, stream_);
+    launch_tridiag_vector(alpha, beta, k, d_scal_ + kOut, d_scal_ + kSvec, stream_);
     launch_combine(V_, ld, k, d_scal_ + kSvec, tmp_, n, stream_);
     launch_dot(tmp_, tmp_, n, d_partial_, d_scal_ + kNrm2, stream_);
     launch_scale_inv_sqrt(tmp_, V_, n, d_scal_ + kNrm2, stream_);
@@ -3034,8 +3034,7 @@ int Engine::lz_thick_restart(int k, int kmax, long long n, int* j0) {
 // synchronisation).
 void Engine::lz_finish(int node, int k) {
   const long long n = layout_[node].size;
-  launch_tridiag_lowest(d_scal_ + kAlpha, d_scal_ + kBeta, k, d_scal_ + kOut, d_scal_ + kSvec, 1, stream_,
-                        ring_dev_ + 4 * (k - 1));
+  launch_tridiag_vector(d_scal_ + kAlpha, d_scal_ + kBeta, k, d_scal_ + kOut, d_scal_ + kSvec, stream_);
   launch_combine(V_, nmax_, k, d_scal_ + kSvec, tmp_, n, stream_);
   launch_dot(tmp_, tmp_, n, d_partial_, d_scal_ + kNrm2, stream_);
   launch_scale_inv_sqrt(tmp_, T_[node], n, d_scal_ + kNrm2, stream_);
@@ -3061,7 +3060,7 @@ void Engine::lz_queue_check(int j) {
   cudaStreamWaitEvent(aux_, ev_iter_[j], 0);
   // the slot before holds this run's value for one vector less, or one that a
   // restart has lowered since: an upper bound either way
-  launch_tridiag_lowest(d_scal_ + kAlpha, d_scal_ + kBeta, j + 1, ring_dev_ + 4 * j, d_scal_ + kSvec, 0, aux_,
+  launch_tridiag_lowest(d_scal_ + kAlpha, d_scal_ + kBeta, j + 1, ring_dev_ + 4 * j, aux_,
                         j > 0 ? ring_dev_ + 4 * (j - 1) : nullptr);
   cudaMemcpyAsync(ring_host_ + 4 * j, ring_dev_ + 4 * j, 2 * sizeof(double), cudaMemcpyDeviceToHost, aux_);
   cudaMemcpyAsync(ring_host_ + 4 * j + 2, d_scal_ + kBeta + j, sizeof(double), cudaMemcpyDeviceToHost, aux_);

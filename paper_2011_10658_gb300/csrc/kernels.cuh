@@ -154,8 +154,8 @@ struct LzStep {
   unsigned* bar;
   int* err;
 };
-constexpr int kLzMaxBlocks = 1024;
-constexpr long long kLzPartial = 132LL * kLzMaxBlocks;
+constexpr int kLzRowBlocks = 1216;   // a sum's row blocks: its order does not depend on the grid
+constexpr long long kLzPartial = 132LL * kLzRowBlocks;
 int launch_lz_step(const LzStep& p, int ff_arith, cudaStream_t s);
 // out[0] = sqrt(max(in[0], 0))
 void launch_sqrt(const double* in, double* out, cudaStream_t s);
@@ -190,12 +190,14 @@ void launch_cgs2_qr(double* X, const long long* xoff, const int* rows, const int
 
 // Lowest eigenvalue of the symmetric tridiagonal (alpha[0..k), beta[0..k-1))
 // (1 <= k <= 128).  out[0] = theta, out[1] = |beta[k-1] * s_k| (Ritz residual
-// estimate; beta[k-1] is the trailing coupling).  With want_vec, s[0..k) gets
-// the unit eigenvector (s[0] >= 0) and out[0] its Rayleigh quotient.  prev
-// (optional, device): an upper bound of theta, e.g. the value for a smaller
-// basis of the same run; a wrong one costs a round, not the result.
-void launch_tridiag_lowest(const double* alpha, const double* beta, int k, double* out, double* svec, int want_vec,
-                           cudaStream_t s, const double* prev = nullptr);
+// estimate; beta[k-1] is the trailing coupling).  prev (optional, device): an
+// upper bound of theta, e.g. the value for a smaller basis of the same run; a
+// wrong one costs a round, not the result.
+void launch_tridiag_lowest(const double* alpha, const double* beta, int k, double* out, cudaStream_t s,
+                           const double* prev = nullptr);
+// The same with the unit eigenvector in svec[0..k) (svec[0] >= 0) and its
+// Rayleigh quotient in out[0].
+void launch_tridiag_vector(const double* alpha, const double* beta, int k, double* out, double* svec, cudaStream_t s);
 // Thick restart (keep the m <= 8 lowest Ritz pairs of the k x k tridiagonal,
 // k <= 128): writes the k x p combination C (row-major), the new leading
 // p x p tridiagonal into alpha/beta with beta[p-1] the coupling to the

@@ -483,42 +483,93 @@ __device__ int sturm_minors(const double* a, const double* b2, int k, double x) 
   return cnt;
 }
 
-// Eigenvector of T for the eigenvalue theta: inverse iteration with a shift
-// just below theta, tridiagonal LU (Thomas), orthogonalised against the
-// n_prev rows of prev (stride ld) (vectors of lower eigenvalues of a
-// cluster).  x normalised, x[0] >= 0 when n_prev == 0.
-__device__ void inverse_iteration(const double* a, const double* b, int k, double theta, double scale, int iters,
-                                  double* x, const double* prev, int ld, int n_prev) {
-  double cp[TRI_MAX], dp[TRI_MAX];
+// Eigenvector of T for the eigenvalue theta by inverse iteration with a shift
+// just below theta, one warp: tridiagonal LU (Thomas) once, then solves.  Every
+// chain (elimination, substitution, a dot product) is one FP64 latency per row
+// in lane 0, the rest is one row per lane.  cp, inv: the factors (k doubles of
+// shared memory each), x the vector.
+__device__ void inverse_lu(const double* a, const double* b, int k, double theta, double scale, double* cp,
+                           double* inv) {
   const double shift = theta - 1e-13 * fmax(scale, 1e-300) - 1e-300;
-  for (int i = 0; i < k; ++i) x[i] = n_prev == 0 ? 1.0 : 1.0 + 0.37 * (double)(i % (n_prev + 2));
-  for (int it = 0; it < iters; ++it) {
+  if ((threadIdx.x & 31) == 0) {
     double denom = a[0] - shift;
     if (denom == 0.0) denom = 1e-300;
-    cp[0] = (k > 1 ? b[0] : 0.0) / denom;
-    dp[0] = x[0] / denom;
+    inv[0] = denom;   // the first row divides
+    double c = (k > 1 ? b[0] : 0.0) / denom;
+    cp[0] = c;
     for (int i = 1; i < k; ++i) {
-      double m = (a[i] - shift) - b[i - 1] * cp[i - 1];
+      double m = fma(-b[i - 1], c, a[i] - shift);
       if (m == 0.0) m = 1e-300;
-      const double inv = 1.0 / m;
-      cp[i] = (i < k - 1 ? b[i] : 0.0) * inv;
-      dp[i] = (x[i] - b[i - 1] * dp[i - 1]) * inv;
+      const double r = 1.0 / m;
+      c = (i < k - 1 ? b[i] : 0.0) * r;
+      cp[i] = c;
+      inv[i] = r;
     }
-    x[k - 1] = dp[k - 1];
-    for (int i = k - 2; i >= 0; --i) x[i] = dp[i] - cp[i] * x[i + 1];
-    for (int pass = 0; pass < 2; ++pass)
-      for (int q = 0; q < n_prev; ++q) {
-        double h = 0.0;
-        for (int i = 0; i < k; ++i) h += prev[q * ld + i] * x[i];
-        for (int i = 0; i < k; ++i) x[i] -= h * prev[q * ld + i];
-      }
-    double nrm = 0.0;
-    for (int i = 0; i < k; ++i) nrm += x[i] * x[i];
-    const double inv = 1.0 / sqrt(nrm);
-    for (int i = 0; i < k; ++i) x[i] *= inv;
   }
-  if (n_prev == 0 && x[0] < 0.0)
-    for (int i = 0; i < k; ++i) x[i] = -x[i];
+  __syncwarp();
+}
+
+__device__ void inverse_solve(const double* b, int k, const double* cp, const double* inv, double* x) {
+  if ((threadIdx.x & 31) == 0) {
+    double d = x[0] / inv[0];
+    x[0] = d;
+#pragma unroll 4
+    for (int i = 1; i < k; ++i) {
+      d = fma(-b[i - 1], d, x[i]) * inv[i];
+      x[i] = d;
+    }
+#pragma unroll 4
+    for (int i = k - 2; i >= 0; --i) {
+      d = fma(-cp[i], d, x[i]);
+      x[i] = d;
+    }
+  }
+  __syncwarp();
+}
+
+// sum of x[i] y[i], rows one after another; valid in every lane.
+__device__ double chain_dot(const double* x, const double* y, int k) {
+  double h = 0.0;
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll 8
+    for (int i = 0; i < k; ++i) h = fma(x[i], y[i], h);
+  }
+  return __shfl_sync(0xffffffffu, h, 0);
+}
+
+__device__ void remove_along(const double* q, double* x, int k) {
+  const double h = chain_dot(q, x, k);
+  for (int i = threadIdx.x & 31; i < k; i += 32) x[i] = fma(-h, q[i], x[i]);
+  __syncwarp();
+}
+
+__device__ void make_unit(double* x, int k) {
+  const double inv = 1.0 / sqrt(chain_dot(x, x, k));
+  for (int i = threadIdx.x & 31; i < k; i += 32) x[i] *= inv;
+  __syncwarp();
+}
+
+__device__ void inverse_start(double* x, int k, int n_prev) {
+  for (int i = threadIdx.x & 31; i < k; i += 32) x[i] = n_prev == 0 ? 1.0 : 1.0 + 0.37 * (double)(i % (n_prev + 2));
+  __syncwarp();
+}
+
+constexpr int INV_ITERS = 3;
+
+// The lowest eigenvector: no lower ones to stay orthogonal to, x[0] >= 0.
+__device__ void inverse_iteration(const double* a, const double* b, int k, double theta, double scale, double* cp,
+                                  double* inv, double* x) {
+  inverse_lu(a, b, k, theta, scale, cp, inv);
+  inverse_start(x, k, 0);
+  for (int it = 0; it < INV_ITERS; ++it) {
+    inverse_solve(b, k, cp, inv, x);
+    make_unit(x, k);
+  }
+  const bool flip = x[0] < 0.0;
+  __syncwarp();
+  if (flip)
+    for (int i = threadIdx.x & 31; i < k; i += 32) x[i] = -x[i];
+  __syncwarp();
 }
 
 // Multisection for the eigenvalue of index idx (0 = lowest) by N threads, of
@@ -592,11 +643,11 @@ __device__ void stage_tridiag(const double* alpha, const double* beta, int k, do
 //   gamma_r = (a_r - theta) + b_{r-1} f_{r-1} / f_r + b_r g_{r+1} / g_r
 // when x is f / f_r above r and g / g_r below; r is the row of least |gamma|.
 // Lanes 0 and 1 run the two recurrences in step; the rest is parallel.  f, g,
-// c1: k, k and 2 k doubles of shared memory; f returns the unit vector (first
-// component >= 0 with pos).  False if no row has a finite gamma (the
-// recurrences left the FP64 range), f then undefined.
-__device__ bool twisted_vector(const double* a, const double* b, const double* ib, int k, double theta, bool pos,
-                               double* f, double* g, double* c1) {
+// c1: k, k and 2 k doubles of shared memory; f returns the unit vector.  False
+// if no row has a finite gamma (the recurrences left the FP64 range), f then
+// undefined.
+__device__ bool twisted_vector(const double* a, const double* b, const double* ib, int k, double theta, double* f,
+                               double* g, double* c1) {
   const int lane = threadIdx.x & 31;
   for (int i = lane; i < k; i += 32) {
     const double t = theta - a[i];
@@ -649,7 +700,7 @@ __device__ bool twisted_vector(const double* a, const double* b, const double* i
   }
   n2 = warp_sum(n2);
   __syncwarp();
-  const double inv = (pos && f[0] < 0.0 ? -1.0 : 1.0) / sqrt(n2);
+  const double inv = 1.0 / sqrt(n2);
   __syncwarp();
   for (int i = lane; i < k; i += 32) f[i] *= inv;
   __syncwarp();
@@ -659,18 +710,16 @@ __device__ bool twisted_vector(const double* a, const double* b, const double* i
 // Four warps (one per scheduler: a warp's FP64 instruction holds its
 // scheduler's pipe for 64 cycles, so four warps count at four times the points
 // in the same time).  out[0] = theta (lowest eigenvalue), out[1] = |beta[k-1]|
-// |s_k| (the Ritz residual estimate).  With want_vec the eigenvector goes to s
-// and out[0] is its Rayleigh quotient.  prev (optional): the lowest Ritz value
+// |s_k| (the Ritz residual estimate).  prev (optional): the lowest Ritz value
 // of a smaller basis of the same run, an upper bound of theta; the first round
 // then counts at distances from it that halve every second or third point.
-// GB300: 100 us on average over an FP64 sweep of 2x2x2 before (32 points a
-// round, inverse iteration in one lane for small s_k), 12-90 us now (k = 1-64).
+// GB300: 12-90 us (k = 1-64); 100 us on average over an FP64 sweep of 2x2x2
+// with 32 points a round and inverse iteration.
 constexpr int TRI_THREADS = 128;
 
 __global__ void __launch_bounds__(TRI_THREADS) tridiag_lowest_kernel(const double* __restrict__ alpha,
                                                                      const double* __restrict__ beta, int k,
-                                                                     double* out, double* s, int want_vec,
-                                                                     const double* prev) {
+                                                                     double* out, const double* prev) {
   __shared__ double a[TRI_MAX], b[TRI_MAX], b2[TRI_MAX], ib[TRI_MAX];
   __shared__ double f[TRI_MAX], g[TRI_MAX], c1[2 * TRI_MAX], bracket[3];
   const int t = threadIdx.x;
@@ -697,26 +746,38 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_lowest_kernel(const doubl
   multisect<TRI_THREADS>(a, b2, k, 0, t, below, lo, hi);
   if (t >= 32) return;
   const double theta = 0.5 * (lo + hi);
-  const bool ok = twisted_vector(a, b, ib, k, theta, true, f, g, c1);
-  if (!ok) {
-    if (t == 0) inverse_iteration(a, b, k, theta, scale, 3, f, nullptr, 0, 0);
-    __syncwarp();
-  }
-  double th = theta;
-  if (want_vec) {
-    double rq = 0.0;
-    for (int i = t; i < k; i += 32) {
-      double v = a[i] * f[i];
-      if (i > 0) v += b[i - 1] * f[i - 1];
-      if (i < k - 1) v += b[i] * f[i + 1];
-      rq = fma(f[i], v, rq);
-      s[i] = f[i];
-    }
-    th = warp_sum(rq);
-  }
+  if (!twisted_vector(a, b, ib, k, theta, f, g, c1)) inverse_iteration(a, b, k, theta, scale, g, c1, f);
   if (t == 0) {
-    out[0] = th;
+    out[0] = theta;
     out[1] = fabs(beta[k - 1]) * fabs(f[k - 1]);
+  }
+}
+
+// The Ritz pair that an update ends with: s = unit eigenvector (s[0] >= 0),
+// out[0] = its Rayleigh quotient, out[1] as above.  One warp, once per Lanczos
+// run; the bracket and the vector do not depend on what the checks before it
+// found (the vector becomes the node tensor, to the last place).
+__global__ void __launch_bounds__(32) tridiag_vector_kernel(const double* __restrict__ alpha,
+                                                            const double* __restrict__ beta, int k, double* out,
+                                                            double* s) {
+  __shared__ double a[TRI_MAX], b[TRI_MAX], b2[TRI_MAX], ib[TRI_MAX], x[TRI_MAX], cp[TRI_MAX], inv[TRI_MAX];
+  const int t = threadIdx.x;
+  double lo, hi, scale;
+  stage_tridiag(alpha, beta, k, a, b, b2, ib, lo, hi, scale);
+  multisect<32>(a, b2, k, 0, t, WarpBelow(), lo, hi);
+  inverse_iteration(a, b, k, 0.5 * (lo + hi), scale, cp, inv, x);
+  for (int i = t; i < k; i += 32) {
+    double v = a[i] * x[i];
+    if (i > 0) v += b[i - 1] * x[i - 1];
+    if (i < k - 1) v += b[i] * x[i + 1];
+    cp[i] = v;
+    s[i] = x[i];
+  }
+  __syncwarp();
+  const double rq = chain_dot(x, cp, k);
+  if (t == 0) {
+    out[0] = rq;
+    out[1] = fabs(beta[k - 1]) * fabs(x[k - 1]);
   }
 }
 
@@ -729,15 +790,19 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_lowest_kernel(const doubl
 // last vector alone couples to r with |c|, so the next cycle continues the
 // ordinary three-term recurrence from r at position p.  Writes C = S U
 // reversed (k x p, row-major: C[r * p + i]), alpha[0..p), beta[0..p) (beta[p-1]
-// = |c|) and *p_out.  One warp per Ritz pair; then the vectors of a cluster
-// are made orthogonal to the lower ones, and the small Lanczos process runs
-// on the lanes of warp 0.  GB300, k = 64: 375 us; 3.5 ms in one lane.
+// = |c|) and *p_out.
+//
+// One warp per Ritz pair: eigenvalues, factorisations and first solves side by
+// side.  Vector i is kept orthogonal to the lower ones (twice per inverse
+// iteration), so the vectors are finished one after another; its first pass
+// over a lower vector runs beside the other warps' as soon as that one is
+// final.  Bound by FP64 chains of k; 3.5 ms with everything in one lane.
 __global__ void __launch_bounds__(32 * RESTART_MAX) lanczos_restart_kernel(double* alpha, double* beta, int k, int m,
                                                                            double* C, int* p_out) {
   __shared__ double a[TRI_MAX], b[TRI_MAX], b2[TRI_MAX], ib[TRI_MAX];
-  __shared__ double S[RESTART_MAX][TRI_MAX], G[RESTART_MAX][TRI_MAX], c1[RESTART_MAX][2 * TRI_MAX];
-  __shared__ double th[RESTART_MAX], U[RESTART_MAX][RESTART_MAX], bracket[3];
-  __shared__ int good[RESTART_MAX], p_kept;
+  __shared__ double S[RESTART_MAX][TRI_MAX], cp[RESTART_MAX][TRI_MAX], inv[RESTART_MAX][TRI_MAX];
+  __shared__ double th[RESTART_MAX], U[RESTART_MAX][RESTART_MAX], w[RESTART_MAX], bracket[3];
+  __shared__ int p_kept;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp == 0) {
     double glo, ghi, scale;
@@ -747,81 +812,88 @@ __global__ void __launch_bounds__(32 * RESTART_MAX) lanczos_restart_kernel(doubl
   __syncthreads();
   const double scale = bracket[2];
   if (m > k) m = k;
+  double* x = S[warp];
   if (warp < m) {
     double lo = bracket[0], hi = bracket[1];
     multisect<32>(a, b2, k, warp, lane, WarpBelow(), lo, hi);
     const double theta = 0.5 * (lo + hi);
-    const bool ok = twisted_vector(a, b, ib, k, theta, warp == 0, S[warp], G[warp], c1[warp]);
-    if (lane == 0) { th[warp] = theta; good[warp] = ok; }
+    if (lane == 0) th[warp] = theta;
+    inverse_lu(a, b, k, theta, scale, cp[warp], inv[warp]);
+    inverse_start(x, k, warp);
+    inverse_solve(b, k, cp[warp], inv[warp], x);
+  }
+  for (int done = 0; done < m; ++done) {
+    if (warp == done) {
+      for (int it = 0; it < INV_ITERS; ++it) {
+        if (it > 0) inverse_solve(b, k, cp[warp], inv[warp], x);
+        for (int pass = it > 0 ? 0 : 1; pass < 2; ++pass)
+          for (int q = 0; q < warp; ++q) remove_along(S[q], x, k);
+        make_unit(x, k);
+      }
+      if (warp == 0 && x[0] < 0.0)
+        for (int i = lane; i < k; i += 32) x[i] = -x[i];
+    }
+    __syncthreads();
+    if (warp > done && warp < m) remove_along(S[done], x, k);
   }
   __syncthreads();
-  const double bk = beta[k - 1];
   if (warp == 0) {
-    // orthogonal to the lower vectors (twice); a vector that mostly lies in
-    // their span comes from a cluster and is formed by inverse iteration there
-    for (int i = 0; i < m; ++i) {
-      bool ok = good[i] != 0;
-      if (ok)
-        for (int pass = 0; pass < 2; ++pass) {
-          for (int q = 0; q < i; ++q) {
-            double h = 0.0;
-            for (int r = lane; r < k; r += 32) h = fma(S[q][r], S[i][r], h);
-            h = warp_sum(h);
-            for (int r = lane; r < k; r += 32) S[i][r] = fma(-h, S[q][r], S[i][r]);
-          }
-          double n2 = 0.0;
-          for (int r = lane; r < k; r += 32) n2 = fma(S[i][r], S[i][r], n2);
-          n2 = warp_sum(n2);
-          if (pass == 0 && n2 < 0.5) { ok = false; break; }
-          const double inv = 1.0 / sqrt(n2);
-          for (int r = lane; r < k; r += 32) S[i][r] *= inv;
-        }
-      __syncwarp();
-      if (!ok && lane == 0) inverse_iteration(a, b, k, th[i], scale, 3, S[i], &S[0][0], TRI_MAX, i);
-      __syncwarp();
-    }
     // Lanczos on diag(theta) from c / |c| with full reorthogonalisation, one
-    // kept pair per lane
+    // kept pair per lane, sums in the order of the pairs
     const bool in = lane < m;
-    const double c = in ? bk * S[in ? lane : 0][k - 1] : 0.0, t = in ? th[in ? lane : 0] : 0.0;
-    const double cn = sqrt(warp_sum(c * c));
-    double u[RESTART_MAX], la[RESTART_MAX], lb[RESTART_MAX];
+    const double t = in ? th[in ? lane : 0] : 0.0;
+    const double c = in ? beta[k - 1] * S[in ? lane : 0][k - 1] : 0.0;
+    auto put = [&](double v) {
+      __syncwarp();
+      if (in) w[lane] = v;
+      __syncwarp();
+    };
+    auto dot = [&](const double* u) {   // u . w
+      double h = 0.0;
+      for (int i = 0; i < m; ++i) h = fma(u[i], w[i], h);
+      return h;
+    };
+    put(c);
+    const double cn = sqrt(dot(w));
+    double la[RESTART_MAX], lb[RESTART_MAX];
     int p = 0;
     if (cn > 0.0) {
-      u[0] = c / cn;
+      if (in) U[0][lane] = c / cn;
       p = 1;
 #pragma unroll
       for (int j = 0; j < RESTART_MAX; ++j) {
         if (j >= m || j >= p) break;
-        double w = t * u[j];
-        la[j] = warp_sum(u[j] * w);
+        __syncwarp();
+        double v = in ? t * U[j][lane] : 0.0;
+        put(v);
+        la[j] = dot(U[j]);
         for (int pass = 0; pass < 2; ++pass)
-#pragma unroll
-          for (int q = 0; q <= j; ++q) w = fma(-warp_sum(u[q] * w), u[q], w);
-        const double bj = sqrt(warp_sum(w * w));
+          for (int q = 0; q <= j; ++q) {
+            const double h = dot(U[q]);
+            if (in) v = fma(-h, U[q][lane], v);
+            put(v);
+          }
+        const double bj = sqrt(dot(w));
         if (j + 1 >= m || bj <= 1e-13 * fmax(scale, 1e-300)) break;
         if (j + 1 < RESTART_MAX) {
           lb[j] = bj;
-          u[j + 1] = w / bj;
+          if (in) U[j + 1][lane] = v / bj;
         }
         p = j + 2;
       }
     }
     if (p == 0) {   // r decoupled: keep the lowest Ritz vector alone
       p = 1;
-      u[0] = lane == 0 ? 1.0 : 0.0;
+      if (in) U[0][lane] = lane == 0 ? 1.0 : 0.0;
       la[0] = th[0];
     }
+    if (lane == 0) {   // reversed tridiagonal
 #pragma unroll
-    for (int i = 0; i < RESTART_MAX; ++i)
-      if (i < p) {
-        if (in) U[i][lane] = u[i];
-        if (lane == 0) {   // reversed tridiagonal
+      for (int i = 0; i < RESTART_MAX; ++i)
+        if (i < p) {
           alpha[p - 1 - i] = la[i];
           if (i + 1 < p) beta[p - 2 - i] = lb[i];
         }
-      }
-    if (lane == 0) {
       beta[p - 1] = cn;
       *p_out = p_kept = p;
     }
@@ -1005,10 +1077,16 @@ void launch_rotate_basis(const double* V, long long ld, int k, const double* C, 
   count_launches(1);
 }
 
-void launch_tridiag_lowest(const double* alpha, const double* beta, int k, double* out, double* s, int want_vec,
-                           cudaStream_t st, const double* prev) {
+void launch_tridiag_lowest(const double* alpha, const double* beta, int k, double* out, cudaStream_t st,
+                           const double* prev) {
   if (k <= 0 || k > TRI_MAX) return;
-  tridiag_lowest_kernel<<<1, TRI_THREADS, 0, st>>>(alpha, beta, k, out, s, want_vec, prev);
+  tridiag_lowest_kernel<<<1, TRI_THREADS, 0, st>>>(alpha, beta, k, out, prev);
+  count_launches(1);
+}
+
+void launch_tridiag_vector(const double* alpha, const double* beta, int k, double* out, double* s, cudaStream_t st) {
+  if (k <= 0 || k > TRI_MAX) return;
+  tridiag_vector_kernel<<<1, 32, 0, st>>>(alpha, beta, k, out, s);
   count_launches(1);
 }
 

@@ -32,6 +32,10 @@ constexpr int LZ_THREADS = 256;
 constexpr int LZ_WARPS = LZ_THREADS / 32;
 constexpr int LZ_COLS = 8;                       // basis columns of a dot sweep
 constexpr int LZ_MAX_K = 128;
+constexpr int LZ_ROW_BLOCKS = kLzRowBlocks;      // row blocks of a sum
+constexpr int LZ_ALPHA_BLOCKS = 304;             // of alpha
+constexpr int LZ_LONG_BLOCKS = 4;                // most resident blocks per SM of the long form
+constexpr int LZ_SHORT = 64;                     // row blocks of the short form
 constexpr int LZ_DIRECT = 64;                    // grids up to this size: every block adds all partial sums itself
 constexpr long long kLzPolls = 1LL << 22;        // bound of a grid barrier's wait (seconds)
 
@@ -40,15 +44,6 @@ template <typename A>
 __device__ __forceinline__ A lz_in(double v) { return v; }
 template <>
 __device__ __forceinline__ ff lz_in<ff>(double v) { return d2ff(v); }
-
-template <typename A>
-__device__ __forceinline__ A lz_xor(A v, int m);
-template <>
-__device__ __forceinline__ double lz_xor<double>(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
-template <>
-__device__ __forceinline__ ff lz_xor<ff>(ff v, int m) {
-  return ff(__shfl_xor_sync(0xffffffffu, v.hi, m), __shfl_xor_sync(0xffffffffu, v.lo, m));
-}
 
 __device__ __forceinline__ unsigned lz_load(const unsigned* p) {
   unsigned v;
@@ -73,28 +68,80 @@ __device__ __forceinline__ void grid_sync(unsigned* bar, unsigned& round, int* e
   __syncthreads();
 }
 
-// Sum over the block, valid in every thread.
-template <typename A>
-__device__ __forceinline__ double lz_block_sum(A v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v = v + lz_xor(v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = to_d<A>(v);
-  __syncthreads();
-  double r = 0.0;
+// ---- sums in a fixed order
+// A sum over the rows does not depend on the grid: row block b of LZ_ROW_BLOCKS
+// (LZ_ALPHA_BLOCKS for alpha) holds rows 256 b + t, then 256 LZ_ROW_BLOCKS rows
+// further on, one chain per t; a warp's 32 chains are added in halves (16, 8,
+// 4, 2, 1), its eight warps either one after another (columns of a dot phase)
+// or in halves again (single sums), and the row blocks as if they were rows.
+// A node update in reduced precision rounds its vectors to FP32 in every
+// product, so one changed last place in a coefficient ends as a difference of
+// 1e-4 in the update; with this order the launch geometry is free.
+__host__ __device__ __forceinline__ int lz_row_blocks(long long n, int most) {
+  return (int)(n < (long long)most * LZ_THREADS ? (n + LZ_THREADS - 1) / LZ_THREADS : most);
+}
+
+__device__ __forceinline__ double lz_halves8(const double* s) {
+  return ((s[0] + s[4]) + (s[2] + s[6])) + ((s[1] + s[5]) + (s[3] + s[7]));
+}
+
+__device__ __forceinline__ double lz_warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Eight warp sums at once: lane l ends with the sum of v[(l >> 2) & 7] with its
+// bits reversed as 4 (lane bit 4), 2 (bit 3), 1 (bit 2): lz_slot.
+__device__ __forceinline__ double lz_warp_sum8(double* v, int lane) {
 #pragma unroll
-  for (int u = 0; u < LZ_WARPS; ++u) r += red[u];
+  for (int h = LZ_COLS / 2, m = 16; h >= 1; h >>= 1, m >>= 1)
+#pragma unroll
+    for (int t = 0; t < h; ++t) {
+      const bool up = (lane & m) != 0;
+      const double keep = up ? v[t + h] : v[t];
+      const double give = up ? v[t] : v[t + h];
+      v[t] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+    }
+  double r = v[0];
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+  return r;
+}
+__device__ __forceinline__ int lz_slot(int lane) { return ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1); }
+
+// Sum over the block, valid in every thread.
+__device__ __forceinline__ double lz_block_sum(double v, double* red) {
+  v = lz_warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  const double r = lz_halves8(red);
   __syncthreads();
   return r;
 }
 
-// Sum of `count` values (one per block), in block order by lanes; valid in
-// every thread.
+// Sum of the values of `count` row blocks by one warp, valid in every lane.
+__device__ __forceinline__ double lz_total(const double* part, int count, int lane) {
+  double v[LZ_COLS];
+#pragma unroll
+  for (int w = 0; w < LZ_COLS; ++w) v[w] = 0.0;
+  for (int base = 0; base < count; base += LZ_THREADS)
+#pragma unroll
+    for (int w = 0; w < LZ_COLS; ++w) {
+      const int i = base + 32 * w + lane;
+      if (i < count) v[w] += __ldcg(part + i);
+    }
+  double r = lz_warp_sum8(v, lane);
+  r += __shfl_xor_sync(0xffffffffu, r, 16);
+  r += __shfl_xor_sync(0xffffffffu, r, 8);
+  r += __shfl_xor_sync(0xffffffffu, r, 4);
+  return r;
+}
+
+// The same, valid in every thread.
 __device__ __forceinline__ double lz_grid_sum(const double* part, int count, double* red) {
   if (threadIdx.x < 32) {
-    double v = 0.0;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < count; i += 32) v += __ldcg(part + i);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) red[0] = v;
+    const double r = lz_total(part, count, threadIdx.x);
+    if (threadIdx.x == 0) red[0] = r;
   }
   __syncthreads();
   const double r = red[0];
@@ -102,78 +149,96 @@ __device__ __forceinline__ double lz_grid_sum(const double* part, int count, dou
   return r;
 }
 
-// part[col * gridDim.x + block] = this block's V_col . y for col < k, and y . y
-// for col = k.
-template <typename A>
-__device__ __forceinline__ void lz_dots(const LzStep& p, double (*sh)[LZ_COLS], long long i0, long long step) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int g = 0; g <= p.k; g += LZ_COLS) {
-    A acc[LZ_COLS];
+// One thread's products V_col . row for the columns g .. g + 7 (col = k: row .
+// row), for its rows of a row block; then summed over the warp.
+template <typename A, typename Row>
+__device__ __forceinline__ double lz_dot8(const LzStep& p, int g, long long i0, long long step, int lane, Row row) {
+  A acc[LZ_COLS];
 #pragma unroll
-    for (int t = 0; t < LZ_COLS; ++t) acc[t] = A(0);
-    const int cols = min(LZ_COLS, p.k - g);   // basis columns of this sweep
-    const double* col[LZ_COLS];
+  for (int t = 0; t < LZ_COLS; ++t) acc[t] = A(0);
+  const int cols = min(LZ_COLS, p.k - g);   // basis columns among them
+  if (cols == LZ_COLS) {
+#pragma unroll 1
+    for (long long i = i0; i < p.n; i += step) {
+      const double* q = p.V + (long long)g * p.ldq + i;
+      double v[LZ_COLS];
 #pragma unroll
-    for (int t = 0; t < LZ_COLS; ++t) col[t] = p.V + (long long)(g + (t < cols ? t : 0)) * p.ldq;
-    if (cols == LZ_COLS) {
-#pragma unroll 2
-      for (long long i = i0; i < p.n; i += step) {
-        double v[LZ_COLS];
+      for (int t = 0; t < LZ_COLS; ++t, q += p.ldq) v[t] = __ldg(q);
+      const A ya = lz_in<A>(row(i));
 #pragma unroll
-        for (int t = 0; t < LZ_COLS; ++t) v[t] = __ldg(col[t] + i);
-        const A ya = lz_in<A>(p.y[i]);
+      for (int t = 0; t < LZ_COLS; ++t) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
+    }
+  } else {
+#pragma unroll 1
+    for (long long i = i0; i < p.n; i += step) {
+      const double* q = p.V + (long long)g * p.ldq + i;
+      double v[LZ_COLS];
 #pragma unroll
-        for (int t = 0; t < LZ_COLS; ++t) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
-      }
-    } else {
-      for (long long i = i0; i < p.n; i += step) {
-        double v[LZ_COLS];
+      for (int t = 0; t < LZ_COLS; ++t, q += p.ldq) v[t] = t < cols ? __ldg(q) : 0.0;
+      const A ya = lz_in<A>(row(i));
 #pragma unroll
-        for (int t = 0; t < LZ_COLS; ++t) v[t] = t < cols ? __ldg(col[t] + i) : 0.0;
-        const A ya = lz_in<A>(p.y[i]);
-#pragma unroll
-        for (int t = 0; t < LZ_COLS; ++t) {
-          if (t < cols) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
-          else if (t == cols) acc[t] = kc_fma(ya, ya, acc[t]);
-        }
+      for (int t = 0; t < LZ_COLS; ++t) {
+        if (t < cols) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
+        else if (t == cols) acc[t] = kc_fma(ya, ya, acc[t]);
       }
     }
-    // exchange halves: lane bits 4, 3, 2 choose the column a lane ends with
+  }
+  double s[LZ_COLS];
 #pragma unroll
-    for (int h = LZ_COLS / 2, m = 16; h >= 1; h >>= 1, m >>= 1)
+  for (int t = 0; t < LZ_COLS; ++t) s[t] = to_d<A>(acc[t]);
+  return lz_warp_sum8(s, lane);
+}
+
+// y_i - sum_j c_j V_j[i], columns in order.
+template <typename A>
+__device__ __forceinline__ A lz_minus(const LzStep& p, const A* cs, double y, long long i) {
+  A v = lz_in<A>(y);
+  const double* q = p.V + i;
+  int j = 0;
+  for (; j + LZ_COLS <= p.k; j += LZ_COLS) {
+    double x[LZ_COLS];
 #pragma unroll
-      for (int t = 0; t < h; ++t) {
-        const bool up = (lane & m) != 0;
-        const A keep = up ? acc[t + h] : acc[t];
-        const A give = up ? acc[t] : acc[t + h];
-        acc[t] = keep + lz_xor(give, m);
-      }
-    A r = acc[0];
-    r = r + lz_xor(r, 2);
-    r = r + lz_xor(r, 1);
-    if ((lane & 3) == 0) sh[warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = to_d<A>(r);
+    for (int t = 0; t < LZ_COLS; ++t, q += p.ldq) x[t] = __ldg(q);
+#pragma unroll
+    for (int t = 0; t < LZ_COLS; ++t) v = kc_fma(cs[j + t], lz_in<A>(x[t]), v);
+  }
+  for (; j < p.k; ++j, q += p.ldq) v = kc_fma(cs[j], lz_in<A>(__ldg(q)), v);
+  return v;
+}
+
+// partial[col * blocks + b] = row block b's V_col . y for col < k, and y . y
+// for col = k.
+template <typename A>
+__device__ __forceinline__ void lz_dots(const LzStep& p, int blocks, double (*sh)[LZ_MAX_K + LZ_COLS]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long step = (long long)LZ_ROW_BLOCKS * LZ_THREADS;
+  for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+    const long long i0 = (long long)b * LZ_THREADS + threadIdx.x;
+    for (int g = 0; g <= p.k; g += LZ_COLS) {
+      const double r = lz_dot8<A>(p, g, i0, step, lane, [&](long long i) { return p.y[i]; });
+      if ((lane & 3) == 0) sh[warp][g + lz_slot(lane)] = r;
+    }
     __syncthreads();
-    if (threadIdx.x < LZ_COLS && g + (int)threadIdx.x <= p.k) {
+    if ((int)threadIdx.x <= p.k) {
       double v = 0.0;
 #pragma unroll
       for (int u = 0; u < LZ_WARPS; ++u) v += sh[u][threadIdx.x];
-      __stcg(p.partial + (long long)(g + threadIdx.x) * gridDim.x + blockIdx.x, v);
+      __stcg(p.partial + (long long)threadIdx.x * blocks + b, v);
     }
     __syncthreads();
   }
 }
 
-// c[col] = sum over the blocks of partial[col], col < ncol, in every block's
-// shared memory.  Large grids: block b adds columns b, b + grid, .. first.
-__device__ __forceinline__ void lz_columns(const LzStep& p, int ncol, double* coef, double* c, unsigned& round) {
+// c[col] = sum over the row blocks of partial[col], col < ncol, in every
+// block's shared memory.  Large grids: one warp of the grid a column first.
+__device__ __forceinline__ void lz_columns(const LzStep& p, int ncol, int blocks, double* coef, double* c,
+                                           unsigned& round) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool direct = (int)gridDim.x <= LZ_DIRECT;
   const int first = direct ? warp : (int)blockIdx.x + (int)gridDim.x * warp;
   const int step = direct ? LZ_WARPS : (int)gridDim.x * LZ_WARPS;
   for (int col = first; col < ncol; col += step) {
-    double v = 0.0;
-    for (int i = lane; i < (int)gridDim.x; i += 32) v += __ldcg(p.partial + (long long)col * gridDim.x + i);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const double v = lz_total(p.partial + (long long)col * blocks, blocks, lane);
     if (lane == 0) {
       if (direct) c[col] = v;
       else __stcg(coef + col, v);
@@ -186,29 +251,24 @@ __device__ __forceinline__ void lz_columns(const LzStep& p, int ncol, double* co
   __syncthreads();
 }
 
-// y -= V c; returns this thread's part of |y|^2.
+// y -= V c; part[b] = row block b's part of |y|^2.
 template <typename A>
-__device__ __forceinline__ A lz_update(const LzStep& p, const double* c, A* cs, long long i0, long long step) {
+__device__ __forceinline__ void lz_update(const LzStep& p, int blocks, const double* c, A* cs, double* part,
+                                          double* red) {
   for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = lz_in<A>(-c[j]);
   __syncthreads();
-  A nrm = A(0);
+  const long long step = (long long)LZ_ROW_BLOCKS * LZ_THREADS;
+  for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+    A nrm = A(0);
 #pragma unroll 2
-  for (long long i = i0; i < p.n; i += step) {
-    A v = lz_in<A>(p.y[i]);
-    const double* q = p.V + i;
-    int j = 0;
-    for (; j + LZ_COLS <= p.k; j += LZ_COLS) {
-      double x[LZ_COLS];
-#pragma unroll
-      for (int t = 0; t < LZ_COLS; ++t) x[t] = __ldg(q + (long long)(j + t) * p.ldq);
-#pragma unroll
-      for (int t = 0; t < LZ_COLS; ++t) v = kc_fma(cs[j + t], lz_in<A>(x[t]), v);
+    for (long long i = (long long)b * LZ_THREADS + threadIdx.x; i < p.n; i += step) {
+      const A v = lz_minus<A>(p, cs, p.y[i], i);
+      p.y[i] = to_d<A>(v);
+      nrm = kc_fma(v, v, nrm);
     }
-    for (; j < p.k; ++j) v = kc_fma(cs[j], lz_in<A>(__ldg(q + (long long)j * p.ldq)), v);
-    p.y[i] = to_d<A>(v);
-    nrm = kc_fma(v, v, nrm);
+    const double s = lz_block_sum(to_d<A>(nrm), red);
+    if (threadIdx.x == 0) __stcg(part + b, s);
   }
-  return nrm;
 }
 
 // The last block to leave zeroes the counters for the next launch.
@@ -226,44 +286,18 @@ __device__ __forceinline__ void lz_leave(const LzStep& p, double alpha, double n
 }
 
 // ---- short vectors: the basis columns are shared out as well
-// (a step at n = 5104 with 1-46 vectors: 25-55 us in the long form, 22 here)
-// Block (rb, cg) of row_blocks x column_groups: rows rb * 256 .., column sweeps
-// cg, cg + column_groups, ..  A short vector leaves a thread a row or two, so
-// the time is the number of trips to L2 one after another; here a dot phase is
-// one sweep per block, and four lanes share a row of an update.
-// part[rb * (k + 1) + col]; `w` gives w' (or y) of a row.
+// Block (rb, cg) of row_blocks x column_groups: row block rb, column sweeps cg,
+// cg + column_groups, ..  A short vector leaves a thread one row, so the time
+// is the number of trips to L2 one after another; here a dot phase is one sweep
+// per block, and the warps of an update are spread over all blocks.
+// part[rb * (k + 1) + col]; `row` gives w' (or y) of a row.
 template <typename A, typename Row>
-__device__ __forceinline__ void lz_short_dots(const LzStep& p, int rb, int row_blocks, int cg, int column_groups,
-                                              double (*sh)[LZ_COLS], Row row) {
+__device__ __forceinline__ void lz_short_dots(const LzStep& p, int rb, int cg, int column_groups,
+                                              double (*sh)[LZ_MAX_K + LZ_COLS], Row row) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int g = cg * LZ_COLS; g <= p.k; g += column_groups * LZ_COLS) {
-    A acc[LZ_COLS];
-#pragma unroll
-    for (int t = 0; t < LZ_COLS; ++t) acc[t] = A(0);
-    for (long long i = (long long)rb * LZ_THREADS + threadIdx.x; i < p.n; i += (long long)row_blocks * LZ_THREADS) {
-      double v[LZ_COLS];
-#pragma unroll
-      for (int t = 0; t < LZ_COLS; ++t) v[t] = g + t < p.k ? __ldg(p.V + (long long)(g + t) * p.ldq + i) : 0.0;
-      const A ya = lz_in<A>(row(i));
-#pragma unroll
-      for (int t = 0; t < LZ_COLS; ++t) {
-        if (g + t < p.k) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
-        else if (g + t == p.k) acc[t] = kc_fma(ya, ya, acc[t]);
-      }
-    }
-#pragma unroll
-    for (int h = LZ_COLS / 2, m = 16; h >= 1; h >>= 1, m >>= 1)
-#pragma unroll
-      for (int t = 0; t < h; ++t) {
-        const bool up = (lane & m) != 0;
-        const A keep = up ? acc[t + h] : acc[t];
-        const A give = up ? acc[t] : acc[t + h];
-        acc[t] = keep + lz_xor(give, m);
-      }
-    A r = acc[0];
-    r = r + lz_xor(r, 2);
-    r = r + lz_xor(r, 1);
-    if ((lane & 3) == 0) sh[warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = to_d<A>(r);
+    const double r = lz_dot8<A>(p, g, (long long)rb * LZ_THREADS + threadIdx.x, p.n, lane, row);
+    if ((lane & 3) == 0) sh[warp][lz_slot(lane)] = r;
     __syncthreads();
     if (threadIdx.x < LZ_COLS && g + (int)threadIdx.x <= p.k) {
       double v = 0.0;
@@ -275,53 +309,71 @@ __device__ __forceinline__ void lz_short_dots(const LzStep& p, int rb, int row_b
   }
 }
 
-// c[col] = sum over the row blocks, one thread a column, in every block.
+// c[col] = sum over the (at most 64) row blocks, in every block, a warp eight
+// columns at a time.
 __device__ __forceinline__ void lz_short_columns(const LzStep& p, int ncol, int row_blocks, double* c) {
-  if ((int)threadIdx.x < ncol) {
-    double v = 0.0;
-#pragma unroll 8
-    for (int b = 0; b < row_blocks; ++b) v += __ldcg(p.partial + (long long)b * (p.k + 1) + threadIdx.x);
-    c[threadIdx.x] = v;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int g = warp * LZ_COLS; g < ncol; g += LZ_WARPS * LZ_COLS) {
+    double v[2][LZ_COLS];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int t = 0; t < LZ_COLS; ++t)
+        v[h][t] = lane + 32 * h < row_blocks && g + t < ncol
+                      ? __ldcg(p.partial + (long long)(lane + 32 * h) * (p.k + 1) + g + t)
+                      : 0.0;
+    double r = lz_warp_sum8(v[0], lane);
+    if (row_blocks > 32) r += lz_warp_sum8(v[1], lane);
+    if ((lane & 3) == 0 && g + lz_slot(lane) < ncol) c[g + lz_slot(lane)] = r;
   }
   __syncthreads();
 }
 
-// y = row - V c by quads of lanes; returns this thread's part of |y|^2.
+// y = row - V c, a lane a row; part[u] = |y|^2 over rows 32 u .. 32 u + 31.
 template <typename A, typename Row>
-__device__ __forceinline__ A lz_short_update(const LzStep& p, const double* c, A* cs, Row row) {
+__device__ __forceinline__ void lz_short_update(const LzStep& p, int row_blocks, const double* c, A* cs, double* part,
+                                                Row row) {
   for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = lz_in<A>(-c[j]);
   __syncthreads();
-  const int sub = threadIdx.x & 3;
-  const long long quads = (long long)gridDim.x * (LZ_THREADS / 4);
-  A nrm = A(0);
-  for (long long i0 = 0; i0 < p.n; i0 += quads) {   // uniform trip count: the quads exchange below
-    const long long i = i0 + blockIdx.x * (LZ_THREADS / 4) + (threadIdx.x >> 2);
-    const bool in = i < p.n;
-    const double* q = p.V + (in ? i : 0);
-    A v = A(0);
-    for (int j = sub; j < p.k; j += 32) {
-      double x[8];
-#pragma unroll
-      for (int t = 0; t < 8; ++t) x[t] = j + 4 * t < p.k ? __ldg(q + (long long)(j + 4 * t) * p.ldq) : 0.0;
-#pragma unroll
-      for (int t = 0; t < 8; ++t)
-        if (j + 4 * t < p.k) v = kc_fma(cs[j + 4 * t], lz_in<A>(x[t]), v);
-    }
-    v = v + lz_xor(v, 1);
-    v = v + lz_xor(v, 2);
-    if (in && sub == 0) {
-      v = lz_in<A>(row(i)) + v;
+  const int lane = threadIdx.x & 31;
+  for (int u = (int)blockIdx.x + (int)gridDim.x * (threadIdx.x >> 5); u < row_blocks * LZ_WARPS;
+       u += (int)gridDim.x * LZ_WARPS) {
+    const long long i = 32LL * u + lane;
+    A nrm = A(0);
+    if (i < p.n) {
+      const A v = lz_minus<A>(p, cs, row(i), i);
       p.y[i] = to_d<A>(v);
       nrm = kc_fma(v, v, nrm);
     }
+    const double s = lz_warp_sum(to_d<A>(nrm));
+    if (lane == 0) __stcg(part + u, s);
   }
-  return nrm;
+}
+
+// Sum of the warp sums of at most 64 row blocks, valid in every thread.
+__device__ __forceinline__ double lz_short_sum(const double* part, int row_blocks, double* red) {
+  if (threadIdx.x < 32) {
+    double r = 0.0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int b = threadIdx.x + 32 * h;
+      double s[LZ_WARPS];
+#pragma unroll
+      for (int u = 0; u < LZ_WARPS; ++u) s[u] = b < row_blocks ? __ldcg(part + b * LZ_WARPS + u) : 0.0;
+      if (32 * h < row_blocks) r += lz_warp_sum(lz_halves8(s));
+    }
+    if (threadIdx.x == 0) red[0] = r;
+  }
+  __syncthreads();
+  const double r = red[0];
+  __syncthreads();
+  return r;
 }
 
 template <bool FF>
 __global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int row_blocks, int column_groups) {
   using A = typename std::conditional<FF, ff, double>::type;
-  __shared__ double sh[LZ_WARPS][LZ_COLS];
+  __shared__ double sh[LZ_WARPS][LZ_MAX_K + LZ_COLS];
   __shared__ double c[LZ_MAX_K + 4];
   __shared__ A cs[LZ_MAX_K];
   double* red = &sh[0][0];
@@ -329,13 +381,11 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int r
   const int rb = blockIdx.x % row_blocks, cg = blockIdx.x / row_blocks;
   const double* vj = p.V + (long long)(p.k - 1) * p.ldq;
   const double* vp = vj - p.ldq;
-  double* part_a = p.partial + (long long)(LZ_MAX_K + 1) * row_blocks;
-  double* part_b = part_a + gridDim.x;
+  double* part_a = p.partial + (long long)(LZ_MAX_K + 1) * LZ_ROW_BLOCKS;
+  double* part_b = part_a + LZ_ROW_BLOCKS;
   if (cg == 0) {
-    double a = 0.0;
-    for (long long i = (long long)rb * LZ_THREADS + threadIdx.x; i < p.n; i += (long long)row_blocks * LZ_THREADS)
-      a = fma(__ldg(vj + i), __ldcg(p.y + i), a);
-    a = lz_block_sum<double>(a, red);
+    const long long i = (long long)rb * LZ_THREADS + threadIdx.x;
+    const double a = lz_block_sum(i < p.n ? __ldg(vj + i) * __ldcg(p.y + i) : 0.0, red);
     if (threadIdx.x == 0) __stcg(part_a + rb, a);
   }
   grid_sync(p.bar, round, p.err);
@@ -346,25 +396,21 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int r
     double v = fma(-alpha, __ldg(vj + i), __ldcg(p.y + i));
     return p.k >= 2 ? fma(-beta, __ldg(vp + i), v) : v;
   };
-  lz_short_dots<A>(p, rb, row_blocks, cg, column_groups, sh, residual);
+  lz_short_dots<A>(p, rb, cg, column_groups, sh, residual);
   grid_sync(p.bar, round, p.err);
   lz_short_columns(p, p.k + 1, row_blocks, c);
   const double before = c[p.k];
-  A t = lz_short_update<A>(p, c, cs, residual);
-  double s = lz_block_sum<A>(t, red);
-  if (threadIdx.x == 0) __stcg(part_b + blockIdx.x, s);
+  lz_short_update<A>(p, row_blocks, c, cs, part_b, residual);
   grid_sync(p.bar, round, p.err);
-  double nrm2 = lz_grid_sum(part_b, gridDim.x, red);
+  double nrm2 = lz_short_sum(part_b, row_blocks, red);
   if (nrm2 < p.ratio * before) {
     auto plain = [&](long long i) { return __ldcg(p.y + i); };
-    lz_short_dots<A>(p, rb, row_blocks, cg, column_groups, sh, plain);
+    lz_short_dots<A>(p, rb, cg, column_groups, sh, plain);
     grid_sync(p.bar, round, p.err);
     lz_short_columns(p, p.k, row_blocks, c);
-    t = lz_short_update<A>(p, c, cs, plain);
-    s = lz_block_sum<A>(t, red);
-    if (threadIdx.x == 0) __stcg(part_a + blockIdx.x, s);
+    lz_short_update<A>(p, row_blocks, c, cs, part_a, plain);
     grid_sync(p.bar, round, p.err);
-    nrm2 = lz_grid_sum(part_a, gridDim.x, red);
+    nrm2 = lz_short_sum(part_a, row_blocks, red);
   }
   const double inv = 1.0 / sqrt(nrm2);
   for (long long i = blockIdx.x * (long long)LZ_THREADS + threadIdx.x; i < p.n; i += (long long)gridDim.x * LZ_THREADS)
@@ -373,81 +419,93 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int r
 }
 
 template <bool FF>
-__global__ void __launch_bounds__(LZ_THREADS, 3) lz_step_kernel(LzStep p) {
+__global__ void __launch_bounds__(LZ_THREADS, LZ_LONG_BLOCKS) lz_step_kernel(LzStep p) {
   using A = typename std::conditional<FF, ff, double>::type;
-  __shared__ double sh[LZ_WARPS][LZ_COLS];
+  __shared__ double sh[LZ_WARPS][LZ_MAX_K + LZ_COLS];
   __shared__ double c[LZ_MAX_K + 4];
   __shared__ A cs[LZ_MAX_K];
   double* red = &sh[0][0];
   unsigned round = 0;
-  const long long i0 = blockIdx.x * (long long)LZ_THREADS + threadIdx.x;
-  const long long step = (long long)gridDim.x * LZ_THREADS;
+  const int blocks = lz_row_blocks(p.n, LZ_ROW_BLOCKS), blocks_a = lz_row_blocks(p.n, LZ_ALPHA_BLOCKS);
   const double* vj = p.V + (long long)(p.k - 1) * p.ldq;
   const double* vp = vj - p.ldq;
-  // two partial-sum regions that scalars use in turn
-  double* part_a = p.partial + (long long)(LZ_MAX_K + 1) * gridDim.x;
-  double* part_b = part_a + gridDim.x;
+  double* part_a = p.partial + (long long)(LZ_MAX_K + 1) * LZ_ROW_BLOCKS;
+  double* part_b = part_a + LZ_ROW_BLOCKS;
   // alpha_j = v_j . y
-  double a = 0.0;
-  for (long long i = i0; i < p.n; i += step) a = fma(__ldg(vj + i), p.y[i], a);
-  a = lz_block_sum<double>(a, red);
-  if (threadIdx.x == 0) __stcg(part_a + blockIdx.x, a);
-  grid_sync(p.bar, round, p.err);
-  const double alpha = lz_grid_sum(part_a, gridDim.x, red);
-  // w' = y - alpha_j v_j - beta_{j-1} v_{j-1}
-  const double beta = p.k >= 2 ? *p.beta_prev : 0.0;
-  for (long long i = i0; i < p.n; i += step) {
-    double v = fma(-alpha, __ldg(vj + i), p.y[i]);
-    if (p.k >= 2) v = fma(-beta, __ldg(vp + i), v);
-    p.y[i] = v;
+  for (int b = blockIdx.x; b < blocks_a; b += gridDim.x) {
+    double a = 0.0;
+#pragma unroll 4
+    for (long long i = (long long)b * LZ_THREADS + threadIdx.x; i < p.n; i += (long long)LZ_ALPHA_BLOCKS * LZ_THREADS)
+      a = fma(__ldg(vj + i), __ldcg(p.y + i), a);
+    a = lz_block_sum(a, red);
+    if (threadIdx.x == 0) __stcg(part_a + b, a);
   }
-  lz_dots<A>(p, sh, i0, step);
   grid_sync(p.bar, round, p.err);
-  lz_columns(p, p.k + 1, p.coef, c, round);
+  const double alpha = lz_grid_sum(part_a, blocks_a, red);
+  // w' = y - alpha_j v_j - beta_{j-1} v_{j-1}; a thread keeps its rows from here on
+  const double beta = p.k >= 2 ? *p.beta_prev : 0.0;
+  for (int b = blockIdx.x; b < blocks; b += gridDim.x)
+#pragma unroll 2
+    for (long long i = (long long)b * LZ_THREADS + threadIdx.x; i < p.n; i += (long long)LZ_ROW_BLOCKS * LZ_THREADS) {
+      double v = fma(-alpha, __ldg(vj + i), __ldcg(p.y + i));
+      if (p.k >= 2) v = fma(-beta, __ldg(vp + i), v);
+      p.y[i] = v;
+    }
+  lz_dots<A>(p, blocks, sh);
+  grid_sync(p.bar, round, p.err);
+  lz_columns(p, p.k + 1, blocks, p.coef, c, round);
   const double before = c[p.k];
-  A t = lz_update<A>(p, c, cs, i0, step);
-  double s = lz_block_sum<A>(t, red);
-  if (threadIdx.x == 0) __stcg(part_b + blockIdx.x, s);
+  lz_update<A>(p, blocks, c, cs, part_b, red);
   grid_sync(p.bar, round, p.err);
-  double nrm2 = lz_grid_sum(part_b, gridDim.x, red);
+  double nrm2 = lz_grid_sum(part_b, blocks, red);
   if (nrm2 < p.ratio * before) {
-    lz_dots<A>(p, sh, i0, step);
+    lz_dots<A>(p, blocks, sh);
     grid_sync(p.bar, round, p.err);
-    lz_columns(p, p.k, p.coef, c, round);
-    t = lz_update<A>(p, c, cs, i0, step);
-    s = lz_block_sum<A>(t, red);
-    if (threadIdx.x == 0) __stcg(part_a + blockIdx.x, s);
+    lz_columns(p, p.k, blocks, p.coef, c, round);
+    lz_update<A>(p, blocks, c, cs, part_a, red);
     grid_sync(p.bar, round, p.err);
-    nrm2 = lz_grid_sum(part_a, gridDim.x, red);
+    nrm2 = lz_grid_sum(part_a, blocks, red);
   }
   const double inv = 1.0 / sqrt(nrm2);
-  for (long long i = i0; i < p.n; i += step) p.v_next[i] = p.y[i] * inv;
+  for (int b = blockIdx.x; b < blocks; b += gridDim.x)
+#pragma unroll 2
+    for (long long i = (long long)b * LZ_THREADS + threadIdx.x; i < p.n; i += (long long)LZ_ROW_BLOCKS * LZ_THREADS)
+      p.v_next[i] = p.y[i] * inv;
   lz_leave(p, alpha, nrm2);
 }
 
 }  // namespace
 
 // Vectors of up to 16384 rows: a row per thread in the dots, the column sweeps
-// on further blocks.  Longer ones: two rows a thread up to the resident maximum.
+// on further blocks.  Longer ones: two row blocks a block up to the resident
+// maximum, four blocks an SM, which divides the 1216 of a long vector evenly
+// (n = 1.7 M, 1-56 vectors: 222 us a step on average, 272 with three an SM, 316
+// with two; n = 100 k in FP64: 77 us, 97 with one row block a block).
 int launch_lz_step(const LzStep& p, int ff_arith, cudaStream_t s) {
   if (p.k < 1 || p.k > LZ_MAX_K) return -7;
-  const bool is_short = p.n <= 64 * LZ_THREADS;
-  const void* kern = is_short ? (ff_arith ? (const void*)lz_short_kernel<true> : (const void*)lz_short_kernel<false>)
-                              : (ff_arith ? (const void*)lz_step_kernel<true> : (const void*)lz_step_kernel<false>);
+  int row_blocks = lz_row_blocks(p.n, LZ_ROW_BLOCKS);
   static int resident[4] = {0, 0, 0, 0};
-  int& cap = resident[(ff_arith ? 1 : 0) + (is_short ? 2 : 0)];
-  if (!cap) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, LZ_THREADS, 0);
-    cap = std::max(1, std::min(kLzMaxBlocks, std::min(3, per) * sms));
+  const void* kern = nullptr;
+  int cap = 0;
+  bool is_short = row_blocks <= LZ_SHORT;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    kern = is_short ? (ff_arith ? (const void*)lz_short_kernel<true> : (const void*)lz_short_kernel<false>)
+                    : (ff_arith ? (const void*)lz_step_kernel<true> : (const void*)lz_step_kernel<false>);
+    int& known = resident[(ff_arith ? 1 : 0) + (is_short ? 2 : 0)];
+    if (!known) {
+      int dev = 0, sms = 0, per = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, LZ_THREADS, 0);
+      known = std::max(1, std::min(is_short ? 3 : LZ_LONG_BLOCKS, per) * sms);
+    }
+    cap = known;
+    if (!is_short || row_blocks <= cap) break;
+    is_short = false;   // a row block of the short form needs a block of its own
   }
   LzStep arg = p;
-  int row_blocks = (int)std::min<long long>(std::min(64, cap), (p.n + LZ_THREADS - 1) / LZ_THREADS);
   int column_groups = std::max(1, std::min(cap / row_blocks, (p.k + LZ_COLS) / LZ_COLS));
-  const long long want = (p.n + 2 * LZ_THREADS - 1) / (2 * LZ_THREADS);
-  const int blocks = is_short ? row_blocks * column_groups : (int)std::max(1LL, std::min<long long>(cap, want));
+  const int blocks = is_short ? row_blocks * column_groups : std::min(cap, (row_blocks + 1) / 2);
   void* args[] = {&arg, &row_blocks, &column_groups};
   if (cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(LZ_THREADS), args, 0, s) != cudaSuccess) return -3;
   count_launches(1);
