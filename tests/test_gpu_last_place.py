@@ -119,3 +119,25 @@ def test_small_magnitudes_are_kept(q):
     s.close()
     scale = 2.0 ** 120
     assert np.linalg.norm((y - want) * scale) < 1e-3 * np.linalg.norm(want * scale)
+
+
+# A node update in reduced precision: long and short vectors, a basis that is
+# never full and one that restarts; one product of the residual correction.
+UPDATES = [((4, 4, 4), 64, "tf32x3", 0, 64), ((4, 4, 4), 32, "tf32x3", 3, 16), ((4, 4, 4), 32, "tf32x3", 56, 64),
+           ((4, 4, 4), 32, "tf32x3", 60, 12), ((4, 2, 2), 16, "bf16", 8, 20), ((2, 2, 2), 13, "tf32", 1, 24)]
+
+
+def update_digests(q, L, chi, precision, node, krylov):
+    s = state(q, L, chi, precision)
+    s.move_center(node)
+    s.optimize_node(node, tol=1e-3, max_krylov=krylov)
+    u = s.last_update()
+    v = s.node_export(node)
+    s.close()
+    key = "update/%s/%d/%s/%d/%d" % ("x".join(map(str, L)), chi, precision, node, krylov)
+    return {key: digest(v), key + "/products": "%d+%d" % (u["iters_mixed"], u["iters_fp64"])}
+
+
+@pytest.mark.parametrize("L,chi,precision,node,krylov", UPDATES)
+def test_reduced_precision_updates(q, L, chi, precision, node, krylov):
+    check(update_digests(q, L, chi, precision, node, krylov))
