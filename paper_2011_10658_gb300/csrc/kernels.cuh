@@ -8,6 +8,9 @@ namespace qed {
 // Number of kernels launched by this library since load (all streams).
 long long launch_count();
 void count_launches(int n);
+// Lets `kern` use up to `bytes` of dynamic shared memory on the current device:
+// one attribute call per kernel and device (a call costs as much as a launch).
+void allow_smem(const void* kern, int bytes);
 
 // One contribution A(MxK) * B(KxN) to an output.  Element addressing:
 //   A[m,k] = sA * aval[m] * A[row*a_m + k*a_k],  amap[m] = (row << 1) | negate, -1 = zero row

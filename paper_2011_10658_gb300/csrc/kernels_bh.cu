@@ -192,11 +192,7 @@ void launch(const BhTile* tiles, int n_tiles, const BhOut* outs, const BhChunk* 
   const size_t per = bh_warp_bytes(max_n, max_k, ROWS);
   int warps = BH_WARPS;
   while (!SHARE && warps > 1 && warps * per > (size_t)BH_SMEM) warps >>= 1;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(bh_kernel<T, ROWS, SHARE>, cudaFuncAttributeMaxDynamicSharedMemorySize, BH_SMEM);
-    attr = true;
-  }
+  allow_smem((const void*)bh_kernel<T, ROWS, SHARE>, BH_SMEM);
   const int grid = SHARE ? n_tiles : (n_tiles + warps - 1) / warps;
   bh_kernel<T, ROWS, SHARE><<<grid, 32 * warps, warps * per, s>>>(tiles, n_tiles, outs, chunks, (const T*)w, max_n,
                                                                   max_k | 1);

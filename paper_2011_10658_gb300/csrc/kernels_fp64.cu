@@ -7,6 +7,9 @@
 #include <atomic>
 #include <type_traits>
 #include <cstdio>
+#include <mutex>
+#include <set>
+#include <utility>
 
 #include "ffloat.cuh"
 #include "kernels.cuh"
@@ -16,6 +19,15 @@ namespace qed {
 static std::atomic<long long> g_launches{0};
 long long launch_count() { return g_launches.load(); }
 void count_launches(int n) { g_launches += n; }
+
+void allow_smem(const void* kern, int bytes) {
+  static std::mutex lock;
+  static std::set<std::pair<int, const void*>> done;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> guard(lock);
+  if (done.insert({dev, kern}).second) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
 
 namespace {
 
@@ -1047,11 +1059,7 @@ void launch_to_double(const float* x, double* y, long long n, cudaStream_t s) {
 void launch_cholesky_inv(double* G, double* Rinv, const long long* off, const int* n, const int* ld, int count,
                          int max_n, double ill_cond, int* status, cudaStream_t s) {
   if (count <= 0) return;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(cholesky_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 161 * 8);
-    configured = true;
-  }
+  allow_smem((const void*)cholesky_inv_kernel, 160 * 161 * 8);
   cholesky_inv_kernel<<<count, 256, (size_t)max_n * (max_n | 1) * sizeof(double), s>>>(G, Rinv, off, n, ld, status,
                                                                                   ill_cond);
   count_launches(1);

@@ -4,21 +4,21 @@
 // The step is two passes over the Krylov basis (V^T w', then w' - V c) with a
 // few scalars in between.  The grid is resident as a whole (cooperative
 // launch): every thread owns the same rows in every phase, so only scalars
-// cross blocks, through per-block partial sums that are added in block order
-// (the result does not depend on scheduling) between grid barriers.
+// cross blocks, through partial sums between grid barriers.
 //
 // A dot phase takes eight basis columns at a time, each thread summing its
 // rows in registers; a warp then exchanges halves of the eight sums (four,
-// two, one), which costs nine additions where eight separate reductions cost
-// forty -- on GB300's FP64 pipes, and in float-float arithmetic on the FP32
-// pipes, the additions of a reduction cost as much as the products.
+// two, one), which costs nine FP64 additions where eight separate reductions
+// cost forty: on GB300's FP64 pipes the additions of a reduction cost as much
+// as the products.
 //
-// Bound by HBM at bottom nodes (n = 1.7 M, 48 vectors: 331 us for 1.5 GB with
-// the pass over y, 5.2 TB/s per added column; eleven launches took 560), by
-// the latency of its barriers and loads at upper nodes.  Whole updates, GB300:
-// bottom node of 4x4x4 chi=64 48.0 -> 34.5 ms, layer 3 at chi=32 13.7 -> 9.7
-// ms; FP64 sweep of 2x2x2 chi=8 192 -> 129 ms.
+// Bound by HBM and the FP64 additions at bottom nodes (n = 1.7 M: 222 us a step
+// on average over 1-56 vectors, 365 with 56; eleven launches took 560 with 48),
+// by the latency of its barriers and loads at upper nodes (n = 5104: 17 us; 25-55
+// in the long form).  Whole updates, GB300: bottom node of 4x4x4 chi=64 48.0 ->
+// 26 ms, layer 3 at chi=32 14.0 -> 5.9 ms, with the faster products.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "ffloat.cuh"
@@ -36,6 +36,7 @@ constexpr int LZ_ROW_BLOCKS = kLzRowBlocks;      // row blocks of a sum
 constexpr int LZ_ALPHA_BLOCKS = 304;             // of alpha
 constexpr int LZ_LONG_BLOCKS = 4;                // most resident blocks per SM of the long form
 constexpr int LZ_SHORT = 64;                     // row blocks of the short form
+constexpr int LZ_DEVICES = 64;
 constexpr int LZ_DIRECT = 64;                    // grids up to this size: every block adds all partial sums itself
 constexpr long long kLzPolls = 1LL << 22;        // bound of a grid barrier's wait (seconds)
 
@@ -484,17 +485,18 @@ __global__ void __launch_bounds__(LZ_THREADS, LZ_LONG_BLOCKS) lz_step_kernel(LzS
 int launch_lz_step(const LzStep& p, int ff_arith, cudaStream_t s) {
   if (p.k < 1 || p.k > LZ_MAX_K) return -7;
   int row_blocks = lz_row_blocks(p.n, LZ_ROW_BLOCKS);
-  static int resident[4] = {0, 0, 0, 0};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  static std::atomic<int> resident[LZ_DEVICES][4];   // blocks a device holds at once, per kernel
   const void* kern = nullptr;
   int cap = 0;
   bool is_short = row_blocks <= LZ_SHORT;
   for (int attempt = 0; attempt < 2; ++attempt) {
     kern = is_short ? (ff_arith ? (const void*)lz_short_kernel<true> : (const void*)lz_short_kernel<false>)
                     : (ff_arith ? (const void*)lz_step_kernel<true> : (const void*)lz_step_kernel<false>);
-    int& known = resident[(ff_arith ? 1 : 0) + (is_short ? 2 : 0)];
-    if (!known) {
-      int dev = 0, sms = 0, per = 0;
-      cudaGetDevice(&dev);
+    std::atomic<int>& known = resident[dev % LZ_DEVICES][(ff_arith ? 1 : 0) + (is_short ? 2 : 0)];
+    if (!known || dev >= LZ_DEVICES) {
+      int sms = 0, per = 0;
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, LZ_THREADS, 0);
       known = std::max(1, std::min(is_short ? 3 : LZ_LONG_BLOCKS, per) * sms);

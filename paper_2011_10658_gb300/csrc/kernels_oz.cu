@@ -405,11 +405,7 @@ int launch_oz_gram(const OzTile* tiles, int n_tiles, const OzJob* jobs, const vo
   constexpr int S = kOzDigits;
   const int smem = 2 * S * (128 * OZ_KB * 2 + npad * OZ_KB * 2);
   auto kern = npad == 32 ? oz_gram_kernel<S, 32> : oz_gram_kernel<S, 64>;
-  static bool attr[2] = {false, false};
-  if (!attr[npad == 64]) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-    attr[npad == 64] = true;
-  }
+  allow_smem((const void*)kern, 220 * 1024);
   static int sms = 0;
   if (!sms) {
     int dev = 0;

@@ -520,19 +520,13 @@ int launch_tc_heff(int elem, int split, const TcTile* tiles, int n_tiles, const 
     constexpr int E = decltype(type)::value;
     constexpr bool S = decltype(is_split)::value;
     using W = Width<E, S>;
-    const bool wide = max_kpad * E / 16 > W::NARROW;
-    auto kern = wide ? tc_heff_kernel<E, S, W::WIDE> : tc_heff_kernel<E, S, W::NARROW>;
-    static bool attr[2] = {false, false};   // set once: host attribute calls cost as much as a launch
-    if (!attr[wide]) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-      attr[wide] = true;
-    }
-    return kern;
+    return max_kpad * E / 16 <= W::NARROW ? tc_heff_kernel<E, S, W::NARROW> : tc_heff_kernel<E, S, W::WIDE>;
   };
   using Two = std::integral_constant<int, 2>;
   using Four = std::integral_constant<int, 4>;
   auto kern = elem == 2 ? pick(Two(), std::false_type()) : (split ? pick(Four(), std::true_type()) : pick(Four(), std::false_type()));
   if (max_kpad * elem / 16 > (elem == 2 ? Width<2, false>::WIDE : (split ? Width<4, true>::WIDE : Width<4, false>::WIDE))) return -7;
+  allow_smem((const void*)kern, 226 * 1024);
   kern<<<n_tiles, TC_THREADS, smem, s>>>(tiles, outs, chunks, adds, a_bytes, b_bytes, b_stages, y_shift, err, polls);
   count_launches(1);
   return 0;

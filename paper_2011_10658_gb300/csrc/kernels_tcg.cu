@@ -439,16 +439,10 @@ int launch_tg_gemm(int elem, int split, const TgTile* tiles, int n_tiles, const 
   int a_bytes = 0, b_bytes = 0;
   const int smem = tg_stage_bytes(elem, split, max_npad, &a_bytes, &b_bytes);
   if (smem > 200 * 1024) return -7;
-  // kernel attributes and occupancy are looked up once per configuration
-  // (host API calls of this kind cost as much as a small launch)
   const int kind = elem == 2 ? 0 : (split ? 2 : 1);
   auto kern = kind == 0 ? tg_gemm_kernel<2, false> : (kind == 2 ? tg_gemm_kernel<4, true> : tg_gemm_kernel<4, false>);
-  static bool attr_set[3] = {false, false, false};
+  allow_smem((const void*)kern, 200 * 1024);
   static int sms = 0;
-  if (!attr_set[kind]) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr_set[kind] = true;
-  }
   if (!sms) {
     int dev = 0;
     cudaGetDevice(&dev);
