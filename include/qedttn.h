@@ -235,12 +235,14 @@ typedef struct {
  * NULL with cap 0 allowed); *n = sweeps run.  QED_OK once converged,
  * QED_ENOCONV if max_sweeps ran out first (records valid). */
 int ttn_drive(ttn_state *s, const qed_drive *d, qed_drive_record *log, int32_t cap, int32_t *n);
-/* Bound of every mbarrier wait inside the tensor-core kernels of this state,
- * in polls (each poll is one mbarrier test plus a 32 ns sleep); polls < 0
- * restores the default (2^22 polls, about a quarter of a second).  A wait
- * that runs out sets a device flag, the kernel drains the MMAs it issued,
- * frees its tensor memory and returns; the node update then returns
- * QED_ETIMEOUT and the state stays usable.  No counterpart in the paper: a
+/* Bound of every wait inside the kernels of this state, in polls: the mbarrier
+ * waits of the tensor-core kernels (each poll is one mbarrier test plus a 32 ns
+ * sleep) and the grid barriers of a Lanczos step (each poll reads a counter);
+ * polls < 0 restores the defaults (2^22 polls each, about a quarter of a second
+ * and a few seconds).  A wait that runs out sets a device flag, the kernel
+ * drains the MMAs it issued, frees its tensor memory and returns; the node
+ * update then returns QED_ETIMEOUT and the state stays usable (after a grid
+ * barrier with the tensor it had).  No counterpart in the paper: a
  * failure-detection control (polls = 0 makes every such wait give up at
  * once, which is how the tests reach that path without a GPU fault). */
 int ttn_set_wait_limit(ttn_state *s, int64_t polls);

@@ -2964,6 +2964,7 @@ int Engine::lz_prepare(int kmax) {
 
 // v_0 = T[node] / |T[node]|
 void Engine::lz_start(int node) {
+  cudaMemsetAsync(d_err_ + 3, 0, 3 * sizeof(int), stream_);   // an earlier run may have ended on an error
   const long long n = layout_[node].size;
   launch_copy(T_[node], tmp_, n, stream_);
   launch_dot(tmp_, tmp_, n, d_partial_, d_scal_ + kNrm2, stream_);
@@ -2994,6 +2995,7 @@ int Engine::lz_iteration(int j, long long n) {
   p.v_next = V_ + (long long)(j + 1) * nmax_;
   p.bar = (unsigned*)(d_err_ + 4);
   p.err = d_err_ + 3;
+  p.polls = wait_polls;
   const int rc = launch_lz_step(p, precision_ != PREC_FP64 ? 1 : 0, stream_);
   if (rc) err_ = "Lanczos step launch failed";
   return rc;
@@ -3029,26 +3031,25 @@ int Engine::lz_thick_restart(int k, int kmax, long long n, int* j0) {
   return 0;
 }
 
-// Ritz vector x = V s of the last k vectors, normalised into T[node]; the
-// Ritz value and residual estimate go to the final ring slot (read after a
-// synchronisation).
+// Ritz vector x = V s of the last k vectors, normalised into T[node] (which
+// stays as it was if a grid barrier ran out); the Ritz value and residual
+// estimate go to the final ring slot (read after a synchronisation).
 void Engine::lz_finish(int node, int k) {
   const long long n = layout_[node].size;
   launch_tridiag_vector(d_scal_ + kAlpha, d_scal_ + kBeta, k, d_scal_ + kOut, d_scal_ + kSvec, stream_);
   launch_combine(V_, nmax_, k, d_scal_ + kSvec, tmp_, n, stream_);
   launch_dot(tmp_, tmp_, n, d_partial_, d_scal_ + kNrm2, stream_);
-  launch_scale_inv_sqrt(tmp_, T_[node], n, d_scal_ + kNrm2, stream_);
+  launch_scale_inv_sqrt(tmp_, T_[node], n, d_scal_ + kNrm2, stream_, d_err_ + 3);
   cudaMemcpyAsync(ring_host_ + 4 * kMaxKrylov, d_scal_ + kOut, 2 * sizeof(double), cudaMemcpyDeviceToHost, stream_);
   cudaMemcpyAsync(ring_host_ + 4 * kMaxKrylov + 2, d_err_ + 3, sizeof(int), cudaMemcpyDeviceToHost, stream_);
 }
 
 // After the synchronisation behind lz_finish: -6 if a grid barrier of a
-// Lanczos step ran out (the flag is cleared for the next update).
+// Lanczos step ran out (lz_start clears the flag).
 int Engine::lz_waits() {
   int flag = 0;
   std::memcpy(&flag, ring_host_ + 4 * kMaxKrylov + 2, sizeof(int));
   if (!flag) return 0;
-  cudaMemsetAsync(d_err_ + 3, 0, sizeof(int), stream_);
   err_ = "Lanczos step: a grid barrier hit its iteration limit";
   return -6;
 }

@@ -139,8 +139,10 @@ void launch_combine(const double* Q, long long ldq, int k, const double* c, doub
 // first left less than ratio |w'|^2 (Daniel-Gragg-Kaufman-Stewart, decided on
 // the device), then beta_j = |w| and v_next = w / |w|.  y is overwritten.
 // partial: kLzPartial doubles; coef: 256 doubles; bar: two zeroed counters,
-// zero again afterwards; *err set if a wait ran out.  ff_arith != 0: dots
-// and updates in float-float arithmetic (the data stay FP64).
+// zero again afterwards.  polls: bound of each grid barrier's wait (< 0: the
+// default, 2^22); a wait that runs out sets *err, and a step that finds *err set
+// does nothing: both leave alpha_j = beta_j = 0, which ends the run.  ff_arith
+// != 0: dots and updates in float-float arithmetic (the data stay FP64).
 struct LzStep {
   const double* V;
   long long ldq;
@@ -156,6 +158,7 @@ struct LzStep {
   double* v_next;
   unsigned* bar;
   int* err;
+  long long polls;
 };
 constexpr int kLzRowBlocks = 1216;   // a sum's row blocks: its order does not depend on the grid
 constexpr long long kLzPartial = 132LL * kLzRowBlocks;
@@ -166,7 +169,9 @@ void launch_sqrt(const double* in, double* out, cudaStream_t s);
 void launch_axpby(const double* x, double* y, long long n, const double* a_dev, double a_const, double a_sign,
                   const double* b_dev, double b_const, cudaStream_t s);
 // y = x / sqrt(*nrm2) ; returns nothing
-void launch_scale_inv_sqrt(const double* x, double* y, long long n, const double* nrm2, cudaStream_t s);
+// (nothing is written where *gate, if given, is not zero)
+void launch_scale_inv_sqrt(const double* x, double* y, long long n, const double* nrm2, cudaStream_t s,
+                           const int* gate = nullptr);
 void launch_copy(const double* x, double* y, long long n, cudaStream_t s);
 void launch_fill_uniform(double* x, long long n, uint64_t seed, uint64_t start, cudaStream_t s);
 void launch_add_scaled(const double* x, double* y, long long n, double a, cudaStream_t s);

@@ -213,7 +213,8 @@ __global__ void axpby_kernel(const double* __restrict__ x, double* __restrict__ 
 }
 
 __global__ void scale_inv_sqrt_kernel(const double* __restrict__ x, double* __restrict__ y, long long n,
-                                      const double* nrm2) {
+                                      const double* nrm2, const int* gate) {
+  if (gate && *gate) return;
   const double inv = 1.0 / sqrt(*nrm2);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = x[i] * inv;
@@ -1008,8 +1009,9 @@ void launch_axpby(const double* x, double* y, long long n, const double* a_dev, 
   count_launches(1);
 }
 
-void launch_scale_inv_sqrt(const double* x, double* y, long long n, const double* nrm2, cudaStream_t s) {
-  scale_inv_sqrt_kernel<<<grid_for(n), 256, 0, s>>>(x, y, n, nrm2);
+void launch_scale_inv_sqrt(const double* x, double* y, long long n, const double* nrm2, cudaStream_t s,
+                           const int* gate) {
+  scale_inv_sqrt_kernel<<<grid_for(n), 256, 0, s>>>(x, y, n, nrm2, gate);
   count_launches(1);
 }
 

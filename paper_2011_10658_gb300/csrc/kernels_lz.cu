@@ -38,7 +38,7 @@ constexpr int LZ_LONG_BLOCKS = 4;                // most resident blocks per SM 
 constexpr int LZ_SHORT = 64;                     // row blocks of the short form
 constexpr int LZ_DEVICES = 64;
 constexpr int LZ_DIRECT = 64;                    // grids up to this size: every block adds all partial sums itself
-constexpr long long kLzPolls = 1LL << 22;        // bound of a grid barrier's wait (seconds)
+constexpr long long kLzPolls = 1LL << 22;        // default bound of a grid barrier's wait (seconds)
 
 // Operands as they come: the sums' own rounding is above what to_t would save.
 template <typename A>
@@ -53,16 +53,17 @@ __device__ __forceinline__ unsigned lz_load(const unsigned* p) {
 }
 
 // Barrier of the whole grid; round counts them.  A wait that runs out sets
-// *err and goes on (the host then rejects the step).
-__device__ __forceinline__ void grid_sync(unsigned* bar, unsigned& round, int* err) {
+// *err and goes on: every access stays in bounds whatever the sums hold, and the
+// host rejects the run.
+__device__ __forceinline__ void grid_sync(const LzStep& p, unsigned& round) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    atomicAdd(bar, 1u);
+    atomicAdd(p.bar, 1u);
     const unsigned want = ++round * gridDim.x;
     bool ok = false;
-    for (long long it = 0; it < kLzPolls && !ok; ++it) ok = lz_load(bar) >= want;
-    if (!ok) atomicExch(err, 1);
+    for (long long it = 0; it < p.polls && !ok; ++it) ok = lz_load(p.bar) >= want;
+    if (!ok) atomicExch(p.err, 1);
   } else {
     ++round;
   }
@@ -246,7 +247,7 @@ __device__ __forceinline__ void lz_columns(const LzStep& p, int ncol, int blocks
     }
   }
   if (!direct) {
-    grid_sync(p.bar, round, p.err);
+    grid_sync(p, round);
     for (int col = threadIdx.x; col < ncol; col += LZ_THREADS) c[col] = __ldcg(coef + col);
   }
   __syncthreads();
@@ -272,12 +273,16 @@ __device__ __forceinline__ void lz_update(const LzStep& p, int blocks, const dou
   }
 }
 
+// A wait ran out, in this launch or before it.
+__device__ __forceinline__ bool lz_failed(const LzStep& p) { return lz_load((const unsigned*)p.err) != 0u; }
+
 // The last block to leave zeroes the counters for the next launch.
 __device__ __forceinline__ void lz_leave(const LzStep& p, double alpha, double nrm2) {
   if (threadIdx.x == 0) {
     if (blockIdx.x == 0) {
-      *p.alpha_j = alpha;
-      *p.beta_j = sqrt(fmax(nrm2, 0.0));
+      const bool failed = lz_failed(p);
+      *p.alpha_j = failed ? 0.0 : alpha;
+      *p.beta_j = failed ? 0.0 : sqrt(fmax(nrm2, 0.0));
     }
     if (atomicAdd(p.bar + 1, 1u) == gridDim.x - 1) {
       p.bar[0] = 0u;
@@ -378,6 +383,11 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int r
   __shared__ double c[LZ_MAX_K + 4];
   __shared__ A cs[LZ_MAX_K];
   double* red = &sh[0][0];
+  // one reader per block: another block may set the flag meanwhile
+  if (__syncthreads_or(threadIdx.x == 0 && lz_failed(p))) {
+    lz_leave(p, 0.0, 0.0);
+    return;
+  }
   unsigned round = 0;
   const int rb = blockIdx.x % row_blocks, cg = blockIdx.x / row_blocks;
   const double* vj = p.V + (long long)(p.k - 1) * p.ldq;
@@ -389,7 +399,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int r
     const double a = lz_block_sum(i < p.n ? __ldg(vj + i) * __ldcg(p.y + i) : 0.0, red);
     if (threadIdx.x == 0) __stcg(part_a + rb, a);
   }
-  grid_sync(p.bar, round, p.err);
+  grid_sync(p, round);
   const double alpha = lz_grid_sum(part_a, row_blocks, red);
   const double beta = p.k >= 2 ? *p.beta_prev : 0.0;
   // w' of a row, formed wherever it is needed: y is written in the update only
@@ -398,19 +408,19 @@ __global__ void __launch_bounds__(LZ_THREADS, 3) lz_short_kernel(LzStep p, int r
     return p.k >= 2 ? fma(-beta, __ldg(vp + i), v) : v;
   };
   lz_short_dots<A>(p, rb, cg, column_groups, sh, residual);
-  grid_sync(p.bar, round, p.err);
+  grid_sync(p, round);
   lz_short_columns(p, p.k + 1, row_blocks, c);
   const double before = c[p.k];
   lz_short_update<A>(p, row_blocks, c, cs, part_b, residual);
-  grid_sync(p.bar, round, p.err);
+  grid_sync(p, round);
   double nrm2 = lz_short_sum(part_b, row_blocks, red);
   if (nrm2 < p.ratio * before) {
     auto plain = [&](long long i) { return __ldcg(p.y + i); };
     lz_short_dots<A>(p, rb, cg, column_groups, sh, plain);
-    grid_sync(p.bar, round, p.err);
+    grid_sync(p, round);
     lz_short_columns(p, p.k, row_blocks, c);
     lz_short_update<A>(p, row_blocks, c, cs, part_a, plain);
-    grid_sync(p.bar, round, p.err);
+    grid_sync(p, round);
     nrm2 = lz_short_sum(part_a, row_blocks, red);
   }
   const double inv = 1.0 / sqrt(nrm2);
@@ -426,6 +436,11 @@ __global__ void __launch_bounds__(LZ_THREADS, LZ_LONG_BLOCKS) lz_step_kernel(LzS
   __shared__ double c[LZ_MAX_K + 4];
   __shared__ A cs[LZ_MAX_K];
   double* red = &sh[0][0];
+  // one reader per block: another block may set the flag meanwhile
+  if (__syncthreads_or(threadIdx.x == 0 && lz_failed(p))) {
+    lz_leave(p, 0.0, 0.0);
+    return;
+  }
   unsigned round = 0;
   const int blocks = lz_row_blocks(p.n, LZ_ROW_BLOCKS), blocks_a = lz_row_blocks(p.n, LZ_ALPHA_BLOCKS);
   const double* vj = p.V + (long long)(p.k - 1) * p.ldq;
@@ -441,7 +456,7 @@ __global__ void __launch_bounds__(LZ_THREADS, LZ_LONG_BLOCKS) lz_step_kernel(LzS
     a = lz_block_sum(a, red);
     if (threadIdx.x == 0) __stcg(part_a + b, a);
   }
-  grid_sync(p.bar, round, p.err);
+  grid_sync(p, round);
   const double alpha = lz_grid_sum(part_a, blocks_a, red);
   // w' = y - alpha_j v_j - beta_{j-1} v_{j-1}; a thread keeps its rows from here on
   const double beta = p.k >= 2 ? *p.beta_prev : 0.0;
@@ -453,18 +468,18 @@ __global__ void __launch_bounds__(LZ_THREADS, LZ_LONG_BLOCKS) lz_step_kernel(LzS
       p.y[i] = v;
     }
   lz_dots<A>(p, blocks, sh);
-  grid_sync(p.bar, round, p.err);
+  grid_sync(p, round);
   lz_columns(p, p.k + 1, blocks, p.coef, c, round);
   const double before = c[p.k];
   lz_update<A>(p, blocks, c, cs, part_b, red);
-  grid_sync(p.bar, round, p.err);
+  grid_sync(p, round);
   double nrm2 = lz_grid_sum(part_b, blocks, red);
   if (nrm2 < p.ratio * before) {
     lz_dots<A>(p, blocks, sh);
-    grid_sync(p.bar, round, p.err);
+    grid_sync(p, round);
     lz_columns(p, p.k, blocks, p.coef, c, round);
     lz_update<A>(p, blocks, c, cs, part_a, red);
-    grid_sync(p.bar, round, p.err);
+    grid_sync(p, round);
     nrm2 = lz_grid_sum(part_a, blocks, red);
   }
   const double inv = 1.0 / sqrt(nrm2);
@@ -506,6 +521,7 @@ int launch_lz_step(const LzStep& p, int ff_arith, cudaStream_t s) {
     is_short = false;   // a row block of the short form needs a block of its own
   }
   LzStep arg = p;
+  if (arg.polls < 0) arg.polls = kLzPolls;
   int column_groups = std::max(1, std::min(cap / row_blocks, (p.k + LZ_COLS) / LZ_COLS));
   const int blocks = is_short ? row_blocks * column_groups : std::min(cap, (row_blocks + 1) / 2);
   void* args[] = {&arg, &row_blocks, &column_groups};
