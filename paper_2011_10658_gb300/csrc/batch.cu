@@ -12,6 +12,7 @@
 // that the grouped GEMM of a batch is tuned and split on the whole batch.
 #include <algorithm>
 #include <cmath>
+#include <deque>
 #include <map>
 #include <memory>
 #include <stdexcept>
@@ -307,9 +308,10 @@ int BatchRunner::lanczos(int node, const std::vector<double>& tol, int max_krylo
     bool active = true;
   };
   std::vector<St> st(B);
+  std::deque<Engine::MixedScope> scopes;   // of every member, whichever call fails
+  for (Engine* e : es_) scopes.emplace_back(e->use_mixed_, mixed);
   for (int b = 0; b < B; ++b) {
     Engine* e = es_[b];
-    e->use_mixed_ = mixed;
     St& z = st[b];
     z.n = e->layout_[node].size;
     z.kmax = std::min(std::max(max_krylov, 2), kMaxKrylov);
@@ -372,17 +374,17 @@ int BatchRunner::lanczos(int node, const std::vector<double>& tol, int max_krylo
   energy->assign(B, 0.0);
   resid->assign(B, 0.0);
   iters->assign(B, 0);
+  int failed = 0;
   for (int b = 0; b < B; ++b) {
     Engine* e = es_[b];
-    e->use_mixed_ = false;
     e->last_conv_ = -1;
     const int rc = e->lz_waits();
-    if (rc) return rc;
+    failed = failed ? failed : rc;
     (*energy)[b] = e->ring_host_[4 * kMaxKrylov];
     (*resid)[b] = e->ring_host_[4 * kMaxKrylov + 1];
     (*iters)[b] = st[b].iters;
   }
-  return 0;
+  return failed;
 }
 
 int BatchRunner::optimize(int node, double tol, int max_krylov, std::vector<SweepStats>* stats) {

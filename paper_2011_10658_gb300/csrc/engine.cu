@@ -3079,7 +3079,7 @@ bool Engine::lz_converged(int slot, double tol, double* theta, double* res) cons
 
 int Engine::lanczos_run(int node, double tol, int max_krylov, bool mixed, int max_restarts, double* energy,
                         double* resid, int* iters) {
-  use_mixed_ = mixed;
+  MixedScope scope(use_mixed_, mixed);
   const long long n = layout_[node].size;
   int kmax = std::min(std::max(max_krylov, 2), kMaxKrylov);
   if (kmax > n) kmax = (int)n;
@@ -3137,7 +3137,6 @@ int Engine::lanczos_run(int node, double tol, int max_krylov, bool mixed, int ma
     prev_res = std::min(prev_res, res);
   }
   lz_finish(node, k);
-  use_mixed_ = false;
   if (!check(cudaStreamSynchronize(stream_), "lanczos end")) return -3;
   // a speculative iteration's convergence data may still be in flight
   if (last_conv_ >= 0 && !check(cudaEventSynchronize(ev_conv_[last_conv_]), "lanczos end")) return -3;

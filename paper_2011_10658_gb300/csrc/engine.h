@@ -547,6 +547,13 @@ class Engine {
   bool lz_converged(int slot, double tol, double* theta, double* res) const;
   friend class BatchRunner;
   bool use_mixed_ = false;   // current matvec precision inside lanczos
+  struct MixedScope {        // on for the life of a run, however it ends
+    bool& on;
+    MixedScope(bool& flag, bool v) : on(flag) { on = v; }
+    ~MixedScope() { on = false; }
+    MixedScope(const MixedScope&) = delete;
+    MixedScope& operator=(const MixedScope&) = delete;
+  };
   // products of a mixed state's FP64 residual correction run in float-float
   // arithmetic (FP64-level accuracy on the FP32 pipes)
   bool ff_products_ = false;

@@ -43,3 +43,35 @@ def test_timeout_keeps_the_tensor(q, L, chi, node):
     assert abs(e - want) <= 1e-11 * abs(want)
     s.close()
     r.close()
+
+
+def test_batch_member_that_times_out(q):
+    """One member's failure ends the call; no member is left on its
+    reduced-precision operator (the gradient of the second one is what an FP64
+    state with its tensors has, up to the operators' 1e-11; 1e-6 apart otherwise)."""
+    import torch
+    stream = torch.cuda.current_stream().cuda_stream
+    model = q.Model(2, 2, 2, **KW)
+    pair = [q.TTN(model, 8, seed=i, precision="tf32x3", stream=stream) for i in (1, 2)]
+    pair[0].set_wait_limit(0)
+    with pytest.raises(q.QedError) as ei:
+        q.batch_sweep(pair, 1, tol=1e-6, max_krylov=16)
+    assert ei.value.code == -6
+    s = pair[1]
+    s.move_center(s.info()["n_nodes"] - 1)
+    r = q.TTN(model, 8, seed=2, precision="fp64", stream=stream)
+    r.load_tensors([s.node_export(i) for i in range(s.info()["n_nodes"])])
+    node = 0
+    got = []
+    for t in (s, r):
+        t.move_center(node)
+        x = torch.from_numpy(np.random.default_rng(3).random(t.node_size(node)) - 0.5).cuda()
+        y = torch.empty_like(x)
+        t.energy_grad_device(node, x.data_ptr(), y.data_ptr(), x.numel())
+        torch.cuda.synchronize()
+        got.append(y.cpu().numpy())
+    assert np.linalg.norm(got[0] - got[1]) < 1e-9 * np.linalg.norm(got[1])
+    pair[0].set_wait_limit(-1)
+    q.batch_sweep(pair, 1, tol=1e-6, max_krylov=16)
+    for t in pair + [r]:
+        t.close()
