@@ -164,10 +164,8 @@ int BatchRunner::build(int node, const std::vector<int>& members, std::unique_pt
     // plans again now that all exist)
     for (int i = 0; i < 3; ++i) {
       KPlan& b = g->st[i];
-      bool gather = true;
       for (int m : members) {
         const KPlan& p = es_[m]->heff_plans(node, -1, false)->st[i];
-        gather = gather && p.gather;
         const int c0 = (int)b.chunks.size();
         for (KOutput o : p.outs) {
           o.chunk_begin += c0;
@@ -178,7 +176,7 @@ int BatchRunner::build(int node, const std::vector<int>& members, std::unique_pt
       }
       b.finalize(4096);
       b.fine = true;
-      b.gather = gather;
+      b.gather = es_[members[0]]->heff_plans(node, -1, false)->st[i].gather;
     }
   }
   for (int m : members) g->gens.push_back(es_[m]->gen_);
@@ -275,7 +273,7 @@ int BatchRunner::product(int node, const std::vector<int>& active) {
   for (KPlan& p : g->st)
     if (!p.outs.empty()) {
       const int shape = e0->forced_shape_ >= 0 ? e0->forced_shape_ : p.shape[g->fp32];
-      e0->ensure_scratch(std::max<long long>(p.scratch_need(shape, s), 1));
+      e0->ensure_scratch(std::max<long long>(e0->runs_gather(p) ? p.bh_plan(s).w_elems : p.variant(shape, s).scratch_need, 1));
     }
   const long long before = launch_count();
   if (!e0->check(cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed), "graph capture")) return -3;

@@ -627,7 +627,7 @@ int KPlan::candidates(int* out) const {
 int Engine::launch_kplan(KPlan& pl, int fp32, bool tune) {
   if (pl.outs.empty()) return 0;
   const int mode = fp32;   // 0 FP64, 1 FP32, 2 float-float
-  if (pl.gather && mode != 1) {
+  if (runs_gather(pl) && mode != 1) {
     BhPlan& b = pl.bh_plan(stream_);
     ensure_scratch(std::max<long long>(b.w_elems, 1));
     if (validate_ && !validate_plan(pl, nullptr, "plan")) return -1;
@@ -2172,9 +2172,7 @@ Engine::HeffPlans* Engine::heff_plans(int node, int cls, bool adjoint) {
   }
   s3.finalize(kKPart);
   for (int i = 0; i < 3; ++i) st[i].fine = true;
-  int widest = 1;
-  for (int d : L.leg[2].dim) widest = std::max(widest, d);
-  s3.gather = bottom && bh_fits(widest, widest);
+  s3.gather = bottom;
   for (int i = 0; i < 3; ++i) hp->flops += st[i].flops;
   if (!check(cudaGetLastError(), "plan")) return nullptr;
   HeffPlans* raw = hp.get();

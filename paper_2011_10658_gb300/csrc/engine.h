@@ -108,13 +108,11 @@ struct KPlan {
   bool fine = false;    // long sums in shorter parts (a product's; see KPlan::variant)
   double flops = 0.0;   // 2 M N K over the GEMM chunks (set by finalize)
   // row-gather product of a bottom node: whole output sectors (row-major,
-  // not accumulated), A rows of unit stride; runs on kernels_bh.cu
+  // not accumulated), A rows of unit stride; runs on kernels_bh.cu unless a
+  // tile shape is forced
   bool gather = false;
   BhPlan bh;
   BhPlan& bh_plan(cudaStream_t s);
-  long long scratch_need(int shape, cudaStream_t s) {
-    return gather ? bh_plan(s).w_elems : variant(shape, s).scratch_need;
-  }
   KVariant var[KS_COUNT];
   int shape[3] = {-1, -1, -1};    // tuned tile shape per arithmetic (FP64, FP32, float-float), -1 while tuning
   int trials[3] = {0, 0, 0};
@@ -387,7 +385,8 @@ class Engine {
   KPlan* cached_plan(int kind, int a, int b, int c, const std::function<void(KPlan&)>& build);
   int launch_plan(KPlan* pl, int fp32 = 0);
   int launch_kplan(KPlan& pl, int fp32, bool tune);
-  int forced_shape_ = -1;   // QED_KC_SHAPE
+  int forced_shape_ = -1;   // QED_KC_SHAPE: every grouped product on the dense kernel with this tile
+  bool runs_gather(const KPlan& pl) const { return pl.gather && forced_shape_ < 0; }
   double ops_flops_ = 0.0;   // flops of the plans launched since the last reset (profiling)
   void clear_plan_caches();
   // three-stage plans (Z stages of upper nodes, then the output stage)

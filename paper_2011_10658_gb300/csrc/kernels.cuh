@@ -118,11 +118,9 @@ struct BhJob {
   double alpha;
   int K, N;
 };
-// Rows of a tile for outputs up to max_n and terms up to max_k wide, the shared
-// memory of the warp that owns it, and whether that fits the SM.
+// Rows of a tile for outputs up to max_n and terms up to max_k wide (at most 160:
+// the widest sector that the QR of a centre move takes).
 int bh_rows(int max_n, int max_k);
-size_t bh_warp_bytes(int max_n, int max_k, int rows);
-bool bh_fits(int max_n, int max_k);
 // w: staging of 8 bytes per entry.  ff_arith: float-float arithmetic.
 void launch_bh(const BhTile* tiles, int n_tiles, const BhOut* outs, const BhChunk* chunks, const BhJob* jobs,
                int n_jobs, int max_n, int max_k, double* w, cudaStream_t s, int ff_arith);

@@ -37,7 +37,7 @@ namespace qed {
 
 namespace {
 
-constexpr int BH_WARPS = 4;       // warps of a CTA (fewer where their tiles do not fit)
+constexpr int BH_WARPS = 4;       // warps of a CTA
 constexpr int BH_SMEM = 200 * 1024;
 
 // e / d for the small item indices here (e d < 2^32): m = ceil(2^32 / d)
@@ -186,31 +186,28 @@ __global__ void __launch_bounds__(32 * BH_WARPS) bh_kernel(const BhTile* __restr
   for (int e = lane; e < rows * N; e += 32) y[e] = to_d<T>(acc[e]);
 }
 
+// Shared memory of a warp: 16 rows of 160 columns take 41 KB, four warps 165 of
+// the SM's 227.  The rows of an odd leading dimension start in different banks.
+size_t bh_warp_bytes(int max_n, int max_k, int rows) {
+  return (size_t)rows * ((max_n + (max_k | 1) + 1) * 8 + 2 * sizeof(int));
+}
+
 template <typename T, int ROWS, bool SHARE>
 void launch(const BhTile* tiles, int n_tiles, const BhOut* outs, const BhChunk* chunks, int max_n, int max_k,
             const double* w, cudaStream_t s) {
   const size_t per = bh_warp_bytes(max_n, max_k, ROWS);
-  int warps = BH_WARPS;
-  while (!SHARE && warps > 1 && warps * per > (size_t)BH_SMEM) warps >>= 1;
   allow_smem((const void*)bh_kernel<T, ROWS, SHARE>, BH_SMEM);
-  const int grid = SHARE ? n_tiles : (n_tiles + warps - 1) / warps;
-  bh_kernel<T, ROWS, SHARE><<<grid, 32 * warps, warps * per, s>>>(tiles, n_tiles, outs, chunks, (const T*)w, max_n,
+  const int grid = SHARE ? n_tiles : (n_tiles + BH_WARPS - 1) / BH_WARPS;
+  bh_kernel<T, ROWS, SHARE><<<grid, 32 * BH_WARPS, BH_WARPS * per, s>>>(tiles, n_tiles, outs, chunks, (const T*)w, max_n,
                                                                   max_k | 1);
   count_launches(1);
 }
 
 }  // namespace
 
-// The rows of an odd leading dimension start in different banks.
-size_t bh_warp_bytes(int max_n, int max_k, int rows) {
-  return (size_t)rows * ((max_n + (max_k | 1) + 1) * 8 + 2 * sizeof(int));
-}
-
 int bh_rows(int max_n, int max_k) {
   return max_n + max_k > 24 ? 16 : 32;
 }
-
-bool bh_fits(int max_n, int max_k) { return bh_warp_bytes(max_n, max_k, bh_rows(max_n, max_k)) <= (size_t)BH_SMEM; }
 
 void launch_bh(const BhTile* tiles, int n_tiles, const BhOut* outs, const BhChunk* chunks, const BhJob* jobs,
                int n_jobs, int max_n, int max_k, double* w, cudaStream_t s, int ff_arith) {
