@@ -1017,7 +1017,13 @@ const std::vector<RowMap>& Engine::diagonal_map(int node, int cls) {
   const int sl = leg_site(node, 0);
   std::vector<double> diag((size_t)kLocalDim * kLocalDim, 0.0);
   for (int k = 0; k < (int)terms_.size(); ++k) {
-    if ((cls >= 0 && terms_[k].cls != cls) || !local_diagonal(node, k)) continue;
+    if (cls >= 0 && terms_[k].cls != cls) continue;
+    if (!local_diagonal(node, k)) {
+      // bottom_diagonal takes every site Hamiltonian to be part of this map
+      if (terms_[k].ops.size() == 1 && (terms_[k].ops[0].first == sl || terms_[k].ops[0].first == leg_site(node, 1)))
+        throw std::logic_error("a single-site term is not diagonal");
+      continue;
+    }
     const SiteOp* A = nullptr;
     const SiteOp* B = nullptr;
     for (auto& so : terms_[k].ops) (so.first == sl ? A : B) = site_op(lat_.parity(so.first), so.second);
