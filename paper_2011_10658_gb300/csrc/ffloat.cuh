@@ -130,6 +130,13 @@ __device__ __forceinline__ ff to_t<ff>(double v) {
   return ff_norm(t.hi, t.lo);
 }
 
+// Operands as they come, hi cut and not rounded: coefficients, and vectors whose
+// sums round above what to_t would save.
+template <typename T>
+__device__ __forceinline__ T raw_t(double v) { return to_t<T>(v); }
+template <>
+__device__ __forceinline__ ff raw_t<ff>(double v) { return d2ff(v); }
+
 // Values outside the range of the short form below: zeros, magnitudes below
 // 2^-103 (whose lo part nears the FP32 subnormals) or past the FP32 range,
 // infinities and NaN.

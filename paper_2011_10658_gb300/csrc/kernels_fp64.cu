@@ -95,11 +95,11 @@ __global__ void __launch_bounds__(THREADS) kc_gemm_kernel(const KTile* __restric
 #pragma unroll
         for (int j = 0; j < TN; ++j) {
           const int m = tile.m0 + ty * TM + i, n = tile.n0 + tx * TN + j;
-          if (m < out.M && n < out.N) acc[i][j] += to_t<T>(c.alpha) * load_a<T>(c, m, n);
+          if (m < out.M && n < out.N) acc[i][j] += raw_t<T>(c.alpha) * load_a<T>(c, m, n);
         }
       continue;
     }
-    const T alpha = to_t<T>(c.alpha);
+    const T alpha = raw_t<T>(c.alpha);
     for (int k0 = 0; k0 < c.K; k0 += BK) {
       for (int e = tid; e < BM * BK; e += THREADS) {
         const int mm = e / BK, kk = e % BK;

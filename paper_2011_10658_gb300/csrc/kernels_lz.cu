@@ -40,12 +40,6 @@ constexpr int LZ_DEVICES = 64;
 constexpr int LZ_DIRECT = 64;                    // grids up to this size: every block adds all partial sums itself
 constexpr long long kLzPolls = 1LL << 22;        // default bound of a grid barrier's wait (seconds)
 
-// Operands as they come: the sums' own rounding is above what to_t would save.
-template <typename A>
-__device__ __forceinline__ A lz_in(double v) { return v; }
-template <>
-__device__ __forceinline__ ff lz_in<ff>(double v) { return d2ff(v); }
-
 __device__ __forceinline__ unsigned lz_load(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -166,9 +160,9 @@ __device__ __forceinline__ double lz_dot8(const LzStep& p, int g, long long i0, 
       double v[LZ_COLS];
 #pragma unroll
       for (int t = 0; t < LZ_COLS; ++t, q += p.ldq) v[t] = __ldg(q);
-      const A ya = lz_in<A>(row(i));
+      const A ya = raw_t<A>(row(i));
 #pragma unroll
-      for (int t = 0; t < LZ_COLS; ++t) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
+      for (int t = 0; t < LZ_COLS; ++t) acc[t] = kc_fma(raw_t<A>(v[t]), ya, acc[t]);
     }
   } else {
 #pragma unroll 1
@@ -177,10 +171,10 @@ __device__ __forceinline__ double lz_dot8(const LzStep& p, int g, long long i0, 
       double v[LZ_COLS];
 #pragma unroll
       for (int t = 0; t < LZ_COLS; ++t, q += p.ldq) v[t] = t < cols ? __ldg(q) : 0.0;
-      const A ya = lz_in<A>(row(i));
+      const A ya = raw_t<A>(row(i));
 #pragma unroll
       for (int t = 0; t < LZ_COLS; ++t) {
-        if (t < cols) acc[t] = kc_fma(lz_in<A>(v[t]), ya, acc[t]);
+        if (t < cols) acc[t] = kc_fma(raw_t<A>(v[t]), ya, acc[t]);
         else if (t == cols) acc[t] = kc_fma(ya, ya, acc[t]);
       }
     }
@@ -194,7 +188,7 @@ __device__ __forceinline__ double lz_dot8(const LzStep& p, int g, long long i0, 
 // y_i - sum_j c_j V_j[i], columns in order.
 template <typename A>
 __device__ __forceinline__ A lz_minus(const LzStep& p, const A* cs, double y, long long i) {
-  A v = lz_in<A>(y);
+  A v = raw_t<A>(y);
   const double* q = p.V + i;
   int j = 0;
   for (; j + LZ_COLS <= p.k; j += LZ_COLS) {
@@ -202,9 +196,9 @@ __device__ __forceinline__ A lz_minus(const LzStep& p, const A* cs, double y, lo
 #pragma unroll
     for (int t = 0; t < LZ_COLS; ++t, q += p.ldq) x[t] = __ldg(q);
 #pragma unroll
-    for (int t = 0; t < LZ_COLS; ++t) v = kc_fma(cs[j + t], lz_in<A>(x[t]), v);
+    for (int t = 0; t < LZ_COLS; ++t) v = kc_fma(cs[j + t], raw_t<A>(x[t]), v);
   }
-  for (; j < p.k; ++j, q += p.ldq) v = kc_fma(cs[j], lz_in<A>(__ldg(q)), v);
+  for (; j < p.k; ++j, q += p.ldq) v = kc_fma(cs[j], raw_t<A>(__ldg(q)), v);
   return v;
 }
 
@@ -257,7 +251,7 @@ __device__ __forceinline__ void lz_columns(const LzStep& p, int ncol, int blocks
 template <typename A>
 __device__ __forceinline__ void lz_update(const LzStep& p, int blocks, const double* c, A* cs, double* part,
                                           double* red) {
-  for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = lz_in<A>(-c[j]);
+  for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = raw_t<A>(-c[j]);
   __syncthreads();
   const long long step = (long long)LZ_ROW_BLOCKS * LZ_THREADS;
   for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
@@ -339,7 +333,7 @@ __device__ __forceinline__ void lz_short_columns(const LzStep& p, int ncol, int 
 template <typename A, typename Row>
 __device__ __forceinline__ void lz_short_update(const LzStep& p, int row_blocks, const double* c, A* cs, double* part,
                                                 Row row) {
-  for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = lz_in<A>(-c[j]);
+  for (int j = threadIdx.x; j < p.k; j += LZ_THREADS) cs[j] = raw_t<A>(-c[j]);
   __syncthreads();
   const int lane = threadIdx.x & 31;
   for (int u = (int)blockIdx.x + (int)gridDim.x * (threadIdx.x >> 5); u < row_blocks * LZ_WARPS;

@@ -16,5 +16,7 @@ for case in t.PRODUCTS:
     out.update(t.product_digests(q, *case))
 for case in t.UPDATES:
     out.update(t.update_digests(q, *case))
+for node in (0, 32, 56):
+    out.update(t.update_digests(q, (4, 4, 4), 32, "tf32x3", node, 64, t.ODD))
 for k, v in out.items():
     print(k, v)

@@ -17,6 +17,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 KW = dict(t=1.0, m=1.0, ge2=1.0, cB=0.5, nu=10.0, Q=0)
+# coefficients that FP32 does not hold
+ODD = dict(t=0.9, m=0.7, ge2=0.3, cB=1.0 / 0.6, nu=16.7, Q=0)
 GOLDEN = os.path.join(os.path.dirname(__file__), "golden", "last_place.txt")
 
 
@@ -27,11 +29,11 @@ def digest(*arrays):
     return h.hexdigest()[:16]
 
 
-def state(q, L, chi, precision):
+def state(q, L, chi, precision, kw=KW):
     old = os.environ.get("QED_KC_SHAPE")
     os.environ["QED_KC_SHAPE"] = "32"
     try:
-        return q.TTN(q.Model(*L, **KW), chi, seed=1, precision=precision)
+        return q.TTN(q.Model(*L, **kw), chi, seed=1, precision=precision)
     finally:
         if old is None:
             del os.environ["QED_KC_SHAPE"]
@@ -127,17 +129,22 @@ UPDATES = [((4, 4, 4), 64, "tf32x3", 0, 64), ((4, 4, 4), 32, "tf32x3", 3, 16), (
            ((4, 4, 4), 32, "tf32x3", 60, 12), ((4, 2, 2), 16, "bf16", 8, 20), ((2, 2, 2), 13, "tf32", 1, 24)]
 
 
-def update_digests(q, L, chi, precision, node, krylov):
-    s = state(q, L, chi, precision)
+def update_digests(q, L, chi, precision, node, krylov, kw=KW):
+    s = state(q, L, chi, precision, kw)
     s.move_center(node)
     s.optimize_node(node, tol=1e-3, max_krylov=krylov)
     u = s.last_update()
     v = s.node_export(node)
     s.close()
-    key = "update/%s/%d/%s/%d/%d" % ("x".join(map(str, L)), chi, precision, node, krylov)
+    key = ("update" if kw is KW else "odd") + "/%s/%d/%s/%d/%d" % ("x".join(map(str, L)), chi, precision, node, krylov)
     return {key: digest(v), key + "/products": "%d+%d" % (u["iters_mixed"], u["iters_fp64"])}
 
 
 @pytest.mark.parametrize("L,chi,precision,node,krylov", UPDATES)
 def test_reduced_precision_updates(q, L, chi, precision, node, krylov):
     check(update_digests(q, L, chi, precision, node, krylov))
+
+
+@pytest.mark.parametrize("node", [0, 32, 56])
+def test_updates_with_other_couplings(q, node):
+    check(update_digests(q, (4, 4, 4), 32, "tf32x3", node, 64, ODD))
